@@ -97,7 +97,9 @@ enum { WM_FP32 = 0, WM_BF16 = 1 };
  *             controller and reward), taken while the batch needs at most 4 waves
  *             of clusters.  Neither writes log-probs or values, takes a population
  *             or a hierarchical action.
- *   TENSOR    three tcgen05 GEMM launches per step (H % 64 == 0, A % 64 == 0). */
+ *   TENSOR    three tcgen05 GEMM launches per step (H % 64 == 0, A % 64 == 0).  AUTO also
+ *             gives it bf16 models of other sizes (A <= 512, K <= 8), padded with zero
+ *             weights. */
 enum { WM_PATH_AUTO = 0, WM_PATH_STEPWISE = 1, WM_PATH_FUSED = 2, WM_PATH_TENSOR = 3 };
 
 typedef struct {

@@ -261,8 +261,14 @@ cudaError_t pack_step(wm_handle *h, const wm_weights *w) {
 // batch (its tcgen05 member up to B = 2048; its small-batch member while the batch needs at
 // most 4 waves of 16-episode clusters), else the tensor-core family for large bf16 batches
 // and for fp32 models of any batch (its three-pass split beat the stepwise fp32 SIMT family
-// 2x even at B = 16), the stepwise family otherwise.  fused_ok / tc_ok: whether this call's
-// options allow those families.
+// 2x even at B = 16).  The bf16 calls left over (sizes that are no multiple of the tiles', and
+// batches below 256) take the tensor family with padded sizes and accurate nonlinearities:
+// rollouts of 20 steps at Z, A, H, K = 50, 101, 300, 6 take 581 / 627 / 700 / 1274 us at B = 1 /
+// 600 / 2000 / 8000 against 1791 / 2615 / 3819 / 12135 us stepwise, at 128, 512, 1024, 8 and
+// B = 64 1017 against 6616 us, so no size is left to the stepwise family; it keeps fp32 models
+// of such sizes (its fp32 sums are more accurate than three bf16 products), K > 8, A > 512 and
+// populations that do not fill row tiles.  fused_ok / tc_ok: whether this call's options allow
+// those families.
 int pick_path(const wm_handle *h, int B, bool fused_ok = true, bool tc_ok = true) {
     const int p = h->cfg.path;
     if (p != WM_PATH_AUTO) return p;
@@ -270,6 +276,7 @@ int pick_path(const wm_handle *h, int B, bool fused_ok = true, bool tc_ok = true
     if (fu && B <= 2048) return WM_PATH_FUSED;
     if (tc && (B >= 256 || h->cfg.precision == WM_FP32)) return WM_PATH_TENSOR;
     if (fu) return WM_PATH_FUSED;
+    if (tc_ok && wm_tc_auto_ok(h)) return WM_PATH_TENSOR;
     return WM_PATH_STEPWISE;
 }
 
@@ -324,7 +331,7 @@ wm_status wm_create(const wm_config *cfg, const wm_weights *w, wm_handle **out) 
     h->fused.force_cluster = cfg->fused_cluster;
     if (e == cudaSuccess) e = wm_fused_pack(h, w);
     if (e == cudaSuccess) e = wm_small_prepare(h);
-    if (e == cudaSuccess) e = wm_tc_pack(h, w);
+    if (e == cudaSuccess) e = wm_tc_pack(h);
     if (e == cudaSuccess) e = cudaMalloc((void **)&h->status, sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(h->status, 0, sizeof(int));
     if (e != cudaSuccess) {
@@ -532,7 +539,7 @@ wm_status wm_rollout(wm_handle *h, int B, int T, unsigned long long episode_offs
     int path = pick_path(h, B, fused_ok, tc_ok);
     if (path == WM_PATH_FUSED && !(fused_ok && wm_fused_supported(h, B)))
         return fail(h, WM_ERR_UNSUPPORTED, "the fused family does not take this model / batch / outputs");
-    if (path == WM_PATH_TENSOR && !(tc_ok && wm_tc_supported(h)))
+    if (c.path == WM_PATH_TENSOR && !(tc_ok && wm_tc_supported(h)))
         return fail(h, WM_ERR_UNSUPPORTED, "the tensor family does not take this model / call");
 
     size_t need = path == WM_PATH_STEPWISE ? wm_step_rollout_ws(h, B) : path == WM_PATH_TENSOR ? wm_tc_ws(h, B) : 0;
@@ -584,7 +591,7 @@ wm_status wm_set_controllers(wm_handle *h, int P, int E, const float *W_ctrl, co
         e = upload(&h->step.Wp, wp);
         if (e == cudaSuccess) e = upload(&h->step.bp, bpv);
     }
-    if (e == cudaSuccess && h->tc.ok) e = wm_tc_set_controllers(h, P, W_ctrl, b_ctrl);
+    if (e == cudaSuccess && h->tc.ok) e = wm_tc_set_controllers(h, P);
     // the fused family packs the controller into its per-rank images: repack them
     if (e == cudaSuccess && P == 1) {
         h->host.W_ctrl.assign(W_ctrl, W_ctrl + KX * A);
@@ -671,7 +678,7 @@ wm_status wm_mdn_nll_backward(wm_handle *h, int N, int T, const float *z_seq, co
     const int path = pick_path(h, N);
     if (path == WM_PATH_FUSED && !wm_fused_supported(h, N))
         return fail(h, WM_ERR_UNSUPPORTED, "the fused family does not take this model / batch");
-    if (path == WM_PATH_TENSOR && !wm_tc_supported(h))
+    if (c.path == WM_PATH_TENSOR && !wm_tc_supported(h))
         return fail(h, WM_ERR_UNSUPPORTED, "the tensor family does not take this model");
     size_t need = path == WM_PATH_FUSED ? wm_fused_nll_ws(h, N) : path == WM_PATH_TENSOR ? wm_tc_ws(h, N, T)
                                                                                       : wm_step_nll_ws(h, N);
@@ -739,7 +746,7 @@ wm_status wm_mdn_nll(wm_handle *h, int N, int T, const float *z_seq, const int32
     int path = pick_path(h, N);
     if (path == WM_PATH_FUSED && !wm_fused_supported(h, N))
         return fail(h, WM_ERR_UNSUPPORTED, "the fused family does not take this model / batch");
-    if (path == WM_PATH_TENSOR && !wm_tc_supported(h))
+    if (c.path == WM_PATH_TENSOR && !wm_tc_supported(h))
         return fail(h, WM_ERR_UNSUPPORTED, "the tensor family does not take this model");
     size_t need = path == WM_PATH_FUSED ? wm_fused_nll_ws(h, N) : path == WM_PATH_TENSOR ? wm_tc_ws(h, N, T)
                                                                                       : wm_step_nll_ws(h, N);

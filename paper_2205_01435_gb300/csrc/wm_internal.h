@@ -97,6 +97,8 @@ struct wm_tc_weights {
     float *bg_n;
     float *bc, *bg, *bh;
     int dims_per_tile, n_head_tiles, rd_tile, rd_col;  // reward, done (, runtime, memory) columns
+    int Zp, Hp, Ap;  // Z, H and A rounded up (zero weights) to the tiles' granularity
+    int aligned;     // Zp, Hp, Ap are Z, H, A
     int sms;
     int ok;
 };
@@ -189,15 +191,16 @@ class wm_ktime {
 };
 
 // ---- tensor-core family (wm_tensor.cu) ----------------------------------------
-int wm_tc_supported(const wm_handle *h);
+int wm_tc_supported(const wm_handle *h);  // the model's sizes are multiples of the tiles'
+int wm_tc_auto_ok(const wm_handle *h);    // a bf16 model it runs with its sizes padded
 // workspace of a call of B rows; T_teacher >= 0: teacher-forced scoring of T_teacher steps
 // (its operand rows of all T_teacher + 1 frames), -1: a rollout
 size_t wm_tc_ws(const wm_handle *h, int B, int T_teacher = -1);
-cudaError_t wm_tc_pack(wm_handle *h, const wm_weights *w);
+cudaError_t wm_tc_pack(wm_handle *h);  // from the stepwise family's weights
 void wm_tc_free(wm_handle *h);
 cudaError_t wm_tc_rollout(const wm_handle *h, const wm_rollout_dev &a, void *ws, cudaStream_t s);
 cudaError_t wm_tc_nll(const wm_handle *h, const wm_nll_dev &a, void *ws, cudaStream_t s);
-cudaError_t wm_tc_set_controllers(wm_handle *h, int P, const float *W_ctrl, const float *b_ctrl);
+cudaError_t wm_tc_set_controllers(wm_handle *h, int P);
 // whether the tensor family can run a rollout call starting at this episode (population tiles)
 int wm_tc_call_ok(const wm_handle *h, unsigned long long episode_offset);
 

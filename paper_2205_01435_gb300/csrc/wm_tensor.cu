@@ -30,7 +30,6 @@
 #include <string.h>
 
 #include <algorithm>
-#include <vector>
 
 #include "tc_ptx.cuh"
 #include "wm_device.cuh"
@@ -143,6 +142,10 @@ struct GemmGrid {
 // Epilogue parameters (device pointers; one step)
 struct StepIO {
     int B, Z, A, H, K, T, t;
+    // The sizes the packed operands are laid out by: Z, H and A rounded up with zero weights
+    // (see wm_tc_pack).  Internal rows (x, c, h32, hfin, cfin, W_a, logits, b_ctrl) have the
+    // padded strides; the caller's arrays have Z, H and A.
+    int Zp, Hp, Ap;
     uint32_t step;
     unsigned long long ep0, seed;
     int teacher, ctrl_sample, sigma_sqrt_tau, done_terminates, noop_terminates;
@@ -193,7 +196,7 @@ struct StepIO {
     // kernel picks the xfer (act) and the location, whose action row n_xfers + location is
     // act2 (-1: none)
     int n_xfers;
-    float *logits;                  // [B, A]
+    float *logits;                  // [B, Ap]
     const uint32_t *loc_mask;       // [T, B, NX, WL] or null
     int32_t *loc_actions;           // [T, B] optional
     int32_t *act2;                  // [B]
@@ -246,7 +249,7 @@ struct EpiCtx {
 // ---- controller epilogue: A columns in TMEM, A/4 per column group ---------------
 // Every thread of a warp issues the same TMEM loads (they are warp-collective);
 // rows past B only skip their memory accesses.  The column group's columns are
-// taken 16 at a time ("chunks"; A % 64 == 0 puts each chunk inside one mask word).
+// taken 16 at a time ("chunks"; Ap % 64 == 0 puts each chunk inside one mask word).
 // The row's mask bits and frozen flag are loaded before the accumulator wait, and
 // the bias is read from a copy in shared memory.  The tempered draw keeps each
 // chunk's sum of weights, so only the chunk that holds the drawn point is read a
@@ -268,7 +271,7 @@ struct EpiCtrl {
     // bias of a single controller into every quadrant's copy
     static __device__ void init(const StepIO &p, EpiCtx &x, int e) {
         if (p.pop_P > 1) return;
-        for (int i = e; i < 4 * p.A; i += 32 * EPI_WARPS) x.red[RED_FLOATS + (i / p.A) * MAX_A + i % p.A] = p.b_ctrl[i % p.A];
+        for (int i = e; i < 4 * p.Ap; i += 32 * EPI_WARPS) x.red[RED_FLOATS + (i / p.Ap) * MAX_A + i % p.Ap] = p.b_ctrl[i % p.Ap];
     }
     static __device__ void prefetch(const StepIO &, int, int, EpiCtx &) {}
     static __device__ void pre(const StepIO &p, int m, int, EpiCtx &x, Pre &q) {
@@ -276,20 +279,25 @@ struct EpiCtrl {
         q.valid = b < p.live_rows();
         q.live = q.valid && !p.fz_cur[b];
         q.e = q.valid ? p.ep_of(b) : 0;
-        const int A = p.A, W = (A + 31) >> 5, CW = A / 4, c_lo = x.cg * CW;
+        const int A = p.A, Ap = p.Ap, W = (A + 31) >> 5, CW = Ap / 4, c_lo = x.cg * CW;
         const uint32_t *mw = (q.live && p.mask) ? p.mask + ((size_t)p.t * p.B + q.e) * W : nullptr;
 #pragma unroll
-        for (int k = 0; k < NCH; ++k) {
+        for (int k = 0; k < NCH; ++k) {  // (the loads apart from their use: all in flight together)
             const int c0 = c_lo + 16 * k;
-            q.bits[k] = (!q.live || 16 * k >= CW) ? 0u : mw ? (mw[c0 >> 5] >> (c0 & 31)) & 0xFFFFu : 0xFFFFu;
+            q.bits[k] = (!q.live || 16 * k >= CW || c0 >= A) ? 0u : mw ? mw[c0 >> 5] : 0xFFFFFFFFu;
+        }
+#pragma unroll
+        for (int k = 0; k < NCH; ++k) {
+            const int c0 = c_lo + 16 * k, left = A - c0;  // columns from c0 on that are actions
+            q.bits[k] = (q.bits[k] >> (c0 & 31)) & (left >= 16 ? 0xFFFFu : (1u << max(left, 0)) - 1u);
         }
         if (p.pop_P > 1) {  // the tile's candidate's bias into the quadrant's copy (the previous
                             // tile's readers are past its closing barrier)
             const unsigned long long cand = ((p.ep0 + (unsigned long long)m * BM) / (unsigned long long)p.pop_E) %
                                             (unsigned long long)p.pop_P;
-            const float *bc = p.b_ctrl + cand * p.A;
+            const float *bc = p.b_ctrl + cand * Ap;
             float *bq = x.red + RED_FLOATS + x.quad * MAX_A;
-            for (int i = x.cg * 32 + x.lane; i < A; i += 128) bq[i] = bc[i];
+            for (int i = x.cg * 32 + x.lane; i < Ap; i += 128) bq[i] = bc[i];
         }
     }
     // logits of chunk k (accumulator + bias)
@@ -320,7 +328,7 @@ struct EpiCtrl {
         (void)n;
         const int b = m * BM + x.row;
         const bool valid = q.valid, live = q.live;
-        const int CW = p.A / 4, c_lo = x.cg * CW, nch = CW / 16;  // nch is warp-uniform
+        const int CW = p.Ap / 4, c_lo = x.cg * CW, nch = CW / 16;  // nch is warp-uniform
         const float *bs = x.red + RED_FLOATS + x.quad * MAX_A;
         if (p.pop_P > 1) x.sync();  // the quadrant's bias copy (pre) is complete
         // pass 1: masked argmax over this group's columns (lowest index on ties): per chunk,
@@ -493,12 +501,12 @@ struct EpiLogits {
         const int b = m * BM + x.row;
         const int nrows = p.live_rows();
         const bool store = b < nrows && !p.fz_cur[b < nrows ? b : 0];  // frozen rows choose nothing
-        const int CW = p.A / 4, c_lo = x.cg * CW, nch = CW / 16;  // nch is warp-uniform
+        const int CW = p.Ap / 4, c_lo = x.cg * CW, nch = CW / 16;  // nch is warp-uniform
         const unsigned long long cand =
             p.pop_P > 1 ? ((p.ep0 + (unsigned long long)m * BM) / (unsigned long long)p.pop_E) % (unsigned long long)p.pop_P
                         : 0ull;
-        const float *bias = p.b_ctrl + cand * p.A;
-        float *out = p.logits + (size_t)(b < p.B ? b : 0) * p.A;
+        const float *bias = p.b_ctrl + cand * p.Ap;
+        float *out = p.logits + (size_t)(b < p.B ? b : 0) * p.Ap;
         for (int k = 0; k < nch; ++k) {  // every lane issues the (warp-collective) TMEM loads
             const int c0 = c_lo + 16 * k;
             uint32_t r[16];
@@ -536,7 +544,7 @@ __global__ void __launch_bounds__(256) k_tc_select(StepIO p) {
         ws.seed = p.seed;
         ws.episode = p.ep0 + e;
         ws.step = p.step;
-        const float *l = p.logits + (size_t)b * A;
+        const float *l = p.logits + (size_t)b * p.Ap;
         const uint32_t *mw = p.mask ? p.mask + tb * W : nullptr;
         x = warp_select(ws, l, NX, mw, 0, &lp);
         if (x >= 0 && x != NX - 1) {
@@ -573,9 +581,11 @@ __global__ void __launch_bounds__(256) k_tc_select(StepIO p) {
 // UNITS: hidden units per tile (64: a 256-column tile; 32: a 128-column tile, for calls with
 // few row tiles, where twice the tiles keep twice the CTA pairs busy and each tile's
 // epilogue is half as long).  Each thread of a quadrant's 4 column groups takes UT units.
-template <int MODE, int UNITS = 64>
+// ACC: the accurate nonlinearities on the bf16 path, for the calls that the stepwise family's
+// accurate ones served before (padded sizes, small batches).
+template <int MODE, int UNITS = 64, bool ACC = false>
 struct EpiGatesT {
-    static constexpr bool TWO = MODE != 0, F32 = MODE == 2;
+    static constexpr bool TWO = MODE != 0, F32 = MODE == 2, PRECISE = F32 || ACC;
     static constexpr int UT = UNITS / 4, WW = UT / 2;  // units per thread, W_a words per gate
     static_assert(UNITS == 64 || UNITS == 32, "gate tile of 64 or 32 units");
     static constexpr uint32_t C_SLAB = 32 * UNITS * 4;  // UNITS / 32 boxes of 32 fp32 x 32 rows
@@ -616,7 +626,7 @@ struct EpiGatesT {
             return;
         }
         const __nv_bfloat16 *src =
-            (lo ? p.wa_lo : p.wa) + (size_t)a * 4 * p.H + 4 * UNITS * n + UNITS * gate + UT * q;
+            (lo ? p.wa_lo : p.wa) + (size_t)a * 4 * p.Hp + 4 * UNITS * n + UNITS * gate + UT * q;
         if constexpr (WW == 8)
             asm volatile("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                          : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7])
@@ -655,8 +665,8 @@ struct EpiGatesT {
     }
     // the cell's nonlinearities: the hardware tanh on the bf16 path; accurate ones on the
     // fp32 path (tanh.approx's relative error, about 2^-11, is above its tolerance)
-    static __device__ __forceinline__ float sig_(float x) { return F32 ? fmaf(0.5f, tanhf(0.5f * x), 0.5f) : sigmoid_hw(x); }
-    static __device__ __forceinline__ float tanh_(float x) { return F32 ? tanhf(x) : tanh_hw(x); }
+    static __device__ __forceinline__ float sig_(float x) { return PRECISE ? fmaf(0.5f, tanhf(0.5f * x), 0.5f) : sigmoid_hw(x); }
+    static __device__ __forceinline__ float tanh_(float x) { return PRECISE ? tanhf(x) : tanh_hw(x); }
     // pre-activations of one gate for the thread's 16 units: accumulator + bias + W_a[a]
     // (+ W_a[a2] when TWO)
     static __device__ __forceinline__ void gate_pre(uint32_t tacc, const float *bg, int gate, int ut,
@@ -693,7 +703,7 @@ struct EpiGatesT {
         const int b = m * BM + x.row;
         const bool valid = b < p.live_rows();
         const int bb = valid ? b : 0;  // rows past the batch compute on row 0; TMA stores clip them
-        const int H = p.H, r = x.lane, q = x.cg;
+        const int Hp = p.Hp, r = x.lane, q = x.cg;
         const bool fz = pr.fz;
         const int ut = UT * q, u0 = UNITS * n + ut;  // the thread's first unit: in the tile, in H
         // gates f and o: loaded while i and g are computed
@@ -739,7 +749,7 @@ struct EpiGatesT {
             for (int j = 0; j < UT; ++j) hv[j] = sig_(g[j]) * tanh_(cv[j]);
         }
         if (fz) {  // frozen: h is the carried one
-            const float4 *h4 = reinterpret_cast<const float4 *>(p.h32 + (size_t)bb * H + u0);
+            const float4 *h4 = reinterpret_cast<const float4 *>(p.h32 + (size_t)bb * Hp + u0);
 #pragma unroll
             for (int i = 0; i < UT / 4; ++i) {
                 const float4 t = h4[i];
@@ -771,16 +781,19 @@ struct EpiGatesT {
             }
         }
         if (store_h32) {
-            float4 *h4 = reinterpret_cast<float4 *>(p.h32 + (size_t)b * H + u0);
+            float4 *h4 = reinterpret_cast<float4 *>(p.h32 + (size_t)b * Hp + u0);
 #pragma unroll
             for (int i = 0; i < UT / 4; ++i) h4[i] = make_float4(hv[4 * i], hv[4 * i + 1], hv[4 * i + 2], hv[4 * i + 3]);
         }
         if (valid) {
-            const size_t o = ((size_t)p.t * p.B + pr.e) * H + u0;
+            const size_t o = ((size_t)p.t * p.B + pr.e) * p.H + u0;
+            const int nu = p.H - u0;  // units from u0 on that are not padding
             if (p.h_seq)
-                for (int j = 0; j < UT; ++j) p.h_seq[o + j] = hv[j];
+                for (int j = 0; j < UT; ++j)
+                    if (j < nu) p.h_seq[o + j] = hv[j];
             if (p.c_seq)
-                for (int j = 0; j < UT; ++j) p.c_seq[o + j] = cv[j];
+                for (int j = 0; j < UT; ++j)
+                    if (j < nu) p.c_seq[o + j] = cv[j];
         }
         // the slab's generic-proxy reads and writes are ordered before the TMA (async-proxy)
         // stores and the refill by this fence and the barrier
@@ -790,8 +803,8 @@ struct EpiGatesT {
             const int y = m * BM + 32 * x.quad;
             if (y < p.B) {  // rows past B are clipped by the stores; a slab wholly past B is skipped
                 for (int bx = 0; bx < UNITS / 32; ++bx) tma_store_2d(x.tm_c, UNITS * n + 32 * bx, y, x.stage_u + 4096 * bx);
-                tma_store_2d(x.tm_xs, p.Z + UNITS * n, y, x.stage_u + C_SLAB);
-                if (F32) tma_store_2d(x.tm_xs2, p.Z + UNITS * n, y, x.stage_u + C_SLAB + X_SLAB);
+                tma_store_2d(x.tm_xs, p.Zp + UNITS * n, y, x.stage_u + C_SLAB);
+                if (F32) tma_store_2d(x.tm_xs2, p.Zp + UNITS * n, y, x.stage_u + C_SLAB + X_SLAB);
                 bulk_commit();
                 bulk_wait_read();  // the slab may be refilled
             }
@@ -805,6 +818,9 @@ using EpiGates2 = EpiGatesT<1>;
 using EpiGates32 = EpiGatesT<2>;
 using EpiGatesN = EpiGatesT<0, 32>;  // 128-column tiles (few row tiles)
 using EpiGates32N = EpiGatesT<2, 32>;  // the same, fp32 path (teacher-forced scoring)
+using EpiGatesA = EpiGatesT<0, 64, true>;    // accurate nonlinearities, bf16 path
+using EpiGates2A = EpiGatesT<1, 64, true>;
+using EpiGatesNA = EpiGatesT<0, 32, true>;
 
 // ---- head epilogue: dims_per_tile latent dims, DS columns each; reward / done -----
 // Before the accumulator wait, the quadrant's 128 threads make the tile's random draws:
@@ -815,7 +831,9 @@ using EpiGates32N = EpiGatesT<2, 32>;  // the same, fp32 path (teacher-forced sc
 // quadrant's z' values are staged in shared memory ([32 rows][33], conflict-free) and
 // stored by all 128 threads in row-major order, so a warp's stores cover a few contiguous
 // row segments instead of 32 rows.
-struct EpiHeads {
+// ACC: accurate exponentials and divisions in the draw (as EpiGatesT's ACC).
+template <bool ACC>
+struct EpiHeadsT {
     static constexpr bool TMA_STAGE = false;
     static constexpr int ZS_PITCH = 33;
     static constexpr uint32_t ZS_BYTES = 32 * ZS_PITCH * 4;  // [32 rows][<= 32 dims] floats
@@ -862,7 +880,7 @@ struct EpiHeads {
         const bool valid = b0 < nrows;
         const int b = valid ? b0 : 0;  // rows past the batch compute on row 0 and store nothing
         const int e = p.ep_of(b);     // the row's episode
-        const int Z = p.Z, K = p.K, KZ = K * Z, M = 3 * KZ, KX = Z + p.H;
+        const int Z = p.Z, K = p.K, KZ = K * Z, M = 3 * KZ, KX = p.Zp + p.Hp;
         const int DS = (3 * K + 7) & ~7;  // columns per latent dim (8-aligned TMEM loads)
         const bool fz = !p.teacher && p.fz_cur[b] != 0;
         const size_t tb = (size_t)p.t * p.B + e;
@@ -958,16 +976,25 @@ struct EpiHeads {
                             if (k < K && lg[k] > best) { best = lg[k]; kc = k; zn = mu[k]; }
                     } else {
                         const float itau = __fdividef(1.f, p.mdn_tau);
+                        auto scaled = [&](float l) {  // l / tau
+                            if constexpr (ACC) return l / p.mdn_tau;
+                            else return l * itau;
+                        };
+                        auto ex = [](float v) {
+                            if constexpr (ACC) return expf(v);
+                            else return __expf(v);
+                        };
                         float mx = -INFINITY;
 #pragma unroll
-                        for (int k = 0; k < 8; ++k) if (k < K) mx = fmaxf(mx, lg[k] * itau);
+                        for (int k = 0; k < 8; ++k) if (k < K) mx = fmaxf(mx, scaled(lg[k]));
                         float pk[8], s = 0.f;
 #pragma unroll
                         for (int k = 0; k < 8; ++k) {
-                            pk[k] = k < K ? __expf(lg[k] * itau - mx) : 0.f;
+                            pk[k] = k < K ? ex(scaled(lg[k]) - mx) : 0.f;
                             s += pk[k];
                         }
-                        const float u = us[x.lane * ZS_PITCH + i], is = __fdividef(1.f, s);  // drawn in pre()
+                        const float u = us[x.lane * ZS_PITCH + i];  // drawn in pre()
+                        const float is = ACC ? 1.f : __fdividef(1.f, s);
                         // first k with u < C_k (the last component when rounding leaves u >= C_{K-2}),
                         // from a compare mask: no per-lane branches
                         float cum = 0.f;
@@ -975,7 +1002,7 @@ struct EpiHeads {
 #pragma unroll
                         for (int k = 0; k < 8; ++k) {
                             if (k < K - 1) {  // uniform
-                                cum += pk[k] * is;
+                                cum += ACC ? pk[k] / s : pk[k] * is;
                                 hit |= (u < cum ? 1u : 0u) << k;
                             }
                         }
@@ -988,7 +1015,7 @@ struct EpiHeads {
                         }
                         const float eps = zs[x.lane * ZS_PITCH + i];  // drawn in pre()
                         const float scale = p.sigma_sqrt_tau ? sqrtf(p.mdn_tau) : 1.f;
-                        zn = muc + __expf(lsc) * scale * eps;
+                        zn = muc + ex(lsc) * scale * eps;
                     }
                     if (p.comp_seq) p.comp_seq[tb * Z + d] = (uint8_t)kc;
                 }
@@ -1060,6 +1087,9 @@ struct EpiHeads {
         x.sync();  // the staging may be rewritten by the next tile
     }
 };
+
+using EpiHeads = EpiHeadsT<false>;
+using EpiHeadsA = EpiHeadsT<true>;
 
 // ---------------------------------------------------------------------------
 // The persistent warp-specialised GEMM on CTA pairs.  A pair computes 256-row tiles of
@@ -1287,25 +1317,30 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
 
 // ---------------------------------------------------------------------------
 __global__ void k_tc_init(StepIO p, const float *z0, const float *h0, const float *c0, const uint8_t *done0,
-                          __nv_bfloat16 *x0, __nv_bfloat16 *x0_lo, uint8_t *fz0, uint8_t *fz1, int n_head_tiles,
-                          int *dstep, int *cnt) {
+                          __nv_bfloat16 *x0, __nv_bfloat16 *x0_lo, __nv_bfloat16 *x1, uint8_t *fz0, uint8_t *fz1,
+                          int n_head_tiles, int *dstep, int *cnt) {
     if (cnt && blockIdx.x == 0 && threadIdx.x < 4) cnt[threadIdx.x] = 0;
-    const int KX = p.Z + p.H;
-    const size_t nx = (size_t)p.B * KX;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < nx; i += (size_t)gridDim.x * blockDim.x) {
-        const size_t b = i / KX, k = i % KX;
-        float v;
-        if (k < (size_t)p.Z) v = p.teacher ? p.z_seq[b * p.Z + k] : z0[b * p.Z + k];
-        else v = h0 ? h0[b * p.H + (k - p.Z)] : 0.f;
-        const __nv_bfloat16 vh = __float2bfloat16_rn(v);
-        x0[i] = vh;
-        if (x0_lo) x0_lo[i] = __float2bfloat16_rn(v - __bfloat162float(vh));
-        if (k >= (size_t)p.Z) {
-            const size_t j = b * p.H + (k - p.Z);
-            p.h32[j] = h0 ? h0[j] : 0.f;
-            p.c[j] = c0 ? c0[j] : 0.f;
-        } else if (!p.teacher) {
-            p.z_out[b * p.Z + k] = z0[b * p.Z + k];
+    const int Zp = p.Zp, Hp = p.Hp, KX = Zp + Hp;
+    for (size_t b = blockIdx.x; b < (size_t)p.B; b += gridDim.x) {  // a block per row: no divisions
+        for (int k = threadIdx.x; k < KX; k += blockDim.x) {
+            const size_t i = b * KX + k;
+            const int u = k - Zp;  // hidden unit (k >= Zp)
+            const bool is_z = k < p.Z, is_h = u >= 0 && u < p.H;
+            float v = 0.f;  // the padded columns are 0
+            if (is_z) v = p.teacher ? p.z_seq[b * p.Z + k] : z0[b * p.Z + k];
+            else if (is_h && h0) v = h0[b * p.H + u];
+            const __nv_bfloat16 vh = __float2bfloat16_rn(v);
+            x0[i] = vh;
+            if (x0_lo) x0_lo[i] = __float2bfloat16_rn(v - __bfloat162float(vh));
+            // the other operand buffer's padded z columns, which no epilogue writes
+            if (x1 && k >= p.Z && k < Zp) x1[i] = vh;
+            if (u >= 0) {
+                const size_t j = b * Hp + u;
+                p.h32[j] = v;
+                p.c[j] = c0 && is_h ? c0[b * p.H + u] : 0.f;
+            } else if (is_z && !p.teacher) {
+                p.z_out[b * p.Z + k] = v;
+            }
         }
     }
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < (size_t)p.B; i += (size_t)gridDim.x * blockDim.x) {
@@ -1323,12 +1358,13 @@ __global__ void k_tc_init(StepIO p, const float *z0, const float *h0, const floa
     }
 }
 
-__global__ void k_tc_finish(int B, int H, const float *h32, const float *c, float *h_final, float *c_final,
+__global__ void k_tc_finish(int B, int H, int Hp, const float *h32, const float *c, float *h_final, float *c_final,
                             const float *nll_part, int n_parts, float *nll) {
     const size_t n = (size_t)B * H;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        if (h_final) h_final[i] = h32[i];
-        if (c_final) c_final[i] = c[i];
+        const size_t j = H == Hp ? i : (i / H) * Hp + i % H;  // the state's rows are Hp wide
+        if (h_final) h_final[i] = h32[j];
+        if (c_final) c_final[i] = c[j];
     }
     if (nll)
         for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < (size_t)B; i += (size_t)gridDim.x * blockDim.x) {
@@ -1343,12 +1379,12 @@ __global__ void k_tc_finish(int B, int H, const float *h32, const float *c, floa
 // (frame f, sequence n at row f N + n: z part from z_seq; the h part of frame f + 1 is
 // written by step f's gate epilogue), the recurrence runs one gate GEMM per step, and one
 // head GEMM then scores all N T (step, sequence) rows.
-__global__ void k_tc_frames(int N, int T, int Z, int KX, const float *__restrict__ z_seq,
+__global__ void k_tc_frames(int N, int T, int Z, int Zp, int KX, const float *__restrict__ z_seq,
                             __nv_bfloat16 *__restrict__ x, __nv_bfloat16 *__restrict__ x_lo) {
-    const size_t n = (size_t)T * N * Z;  // frames 1..T (frame 0 is the init kernel's)
+    const size_t n = (size_t)T * N * Zp;  // frames 1..T (frame 0 is the init kernel's); padded columns 0
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const size_t r = (size_t)N + i / Z, k = i % Z;  // operand row, z column
-        const float v = z_seq[r * Z + k];
+        const size_t r = (size_t)N + i / Zp, k = i % Zp;  // operand row, z column
+        const float v = k < (size_t)Z ? z_seq[r * Z + k] : 0.f;
         const __nv_bfloat16 vh = __float2bfloat16_rn(v);
         x[r * KX + k] = vh;
         if (x_lo) x_lo[r * KX + k] = __float2bfloat16_rn(v - __bfloat162float(vh));
@@ -1380,7 +1416,8 @@ __global__ void k_tc_nll_reduce(int N, int T, int parts, const float *__restrict
 // tile, so the order in which blocks claim their output rows (an atomic per block) changes
 // no result.  One block per 256 rows of step t-1, one warp per row copy.
 struct CompactIO {
-    int B, Z, H, KX, M, t;
+    int B, Z, H, KX, M, t;  // KX: the operand rows' (padded) width
+    int Hp;                 // row stride of c, h32, hfin, cfin
     const int32_t *rows_in;           // [B] row -> episode at step t-1 (null: row b is episode b)
     const int *n_in;                  // rows of step t-1 (null: B)
     const uint8_t *dies;              // [B] row-keyed: the episode ended at step t-1 (at t = 0: done0)
@@ -1501,7 +1538,7 @@ __global__ void __launch_bounds__(CTHREADS) k_tc_compact(CompactIO q) {
             }
         }
         __syncthreads();
-        const int XC = q.KX / 8, CC = q.H / 4;  // 16-byte chunks per row
+        const int XC = q.KX / 8, CC = q.Hp / 4;  // 16-byte chunks per row
         if (warp < nrow) {
             const size_t rr = (size_t)(r0 + warp);
             const int pos = s_pos[warp];
@@ -1521,7 +1558,7 @@ __global__ void __launch_bounds__(CTHREADS) k_tc_compact(CompactIO q) {
                 if (q.fill) {  // its step-t outputs, from its row
                     const int fe = fill_elems(q);
                     for (int k = lane; k < fe; k += 32)
-                        fill_elem(q, (int)e, k, q.h32 + rr * q.H, q.c_in + rr * q.H);
+                        fill_elem(q, (int)e, k, q.h32 + rr * q.Hp, q.c_in + rr * q.Hp);
                 }
             }
         }
@@ -1534,7 +1571,7 @@ __global__ void __launch_bounds__(CTHREADS) k_tc_compact(CompactIO q) {
         for (size_t i = (size_t)blockIdx.x * CTHREADS + tid; i < n; i += stride) {
             const int e = (int)(i / fe), k = (int)(i - (size_t)e * fe);
             if (q.dstep[e] >= q.t) continue;
-            fill_elem(q, e, k, q.hfin + (size_t)e * q.H, q.cfin + (size_t)e * q.H);
+            fill_elem(q, e, k, q.hfin + (size_t)e * q.Hp, q.cfin + (size_t)e * q.Hp);
         }
     }
     if (blockIdx.x == 0 && tid == 0) {
@@ -1567,7 +1604,7 @@ __global__ void k_tc_fill_frozen(CompactIO q) {
         }
         if (q.h_seq || q.c_seq)
             for (int k = lane; k < q.H; k += 32) {
-                const float hv = q.hfin[(size_t)e * q.H + k], cv = q.cfin[(size_t)e * q.H + k];
+                const float hv = q.hfin[(size_t)e * q.Hp + k], cv = q.cfin[(size_t)e * q.Hp + k];
                 for (int t = d; t < q.T; ++t) {
                     const size_t tb = (size_t)t * B + e;
                     if (q.h_seq) q.h_seq[tb * q.H + k] = hv;
@@ -1594,7 +1631,7 @@ __global__ void k_tc_fill_frozen(CompactIO q) {
 
 // h_final, c_final after a compacted rollout: the last step's rows, and the recorded state
 // of the episodes frozen before it
-__global__ void k_tc_finish_compact(int B, int H, int T, const int *dstep, const int32_t *rows, const int *n_rows,
+__global__ void k_tc_finish_compact(int B, int H, int Hp, int T, const int *dstep, const int32_t *rows, const int *n_rows,
                                     const float *h32, const float *c, const float *hfin, const float *cfin,
                                     float *h_final, float *c_final) {
     const int warp = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
@@ -1604,15 +1641,15 @@ __global__ void k_tc_finish_compact(int B, int H, int T, const int *dstep, const
     for (int r = warp; r < n; r += nw) {
         const int e = rows[r];
         for (int i = lane; i < H; i += 32) {
-            if (h_final) h_final[(size_t)e * H + i] = h32[(size_t)r * H + i];
-            if (c_final) c_final[(size_t)e * H + i] = c[(size_t)r * H + i];
+            if (h_final) h_final[(size_t)e * H + i] = h32[(size_t)r * Hp + i];
+            if (c_final) c_final[(size_t)e * H + i] = c[(size_t)r * Hp + i];
         }
     }
     for (int e = warp; e < B; e += nw) {
         if (dstep[e] >= T) continue;  // live at the last step: one of its rows
         for (int i = lane; i < H; i += 32) {
-            if (h_final) h_final[(size_t)e * H + i] = hfin[(size_t)e * H + i];
-            if (c_final) c_final[(size_t)e * H + i] = cfin[(size_t)e * H + i];
+            if (h_final) h_final[(size_t)e * H + i] = hfin[(size_t)e * Hp + i];
+            if (c_final) c_final[(size_t)e * H + i] = cfin[(size_t)e * Hp + i];
         }
     }
 }
@@ -1733,7 +1770,7 @@ inline bool can_compact(const wm_config &c) { return c.done_terminates || c.noop
 
 TcWs carve_ws(const wm_handle *h, int B, void *ws, int T_teacher = -1) {
     const wm_config &c = h->cfg;
-    const size_t KX = (size_t)c.z_dim + c.h_dim, H = c.h_dim;
+    const size_t KX = (size_t)h->tc.Zp + h->tc.Hp, H = h->tc.Hp;
     char *p = (char *)ws;
     TcWs w{};
     for (int i = 0; i < 2; ++i) { w.x[i] = (__nv_bfloat16 *)p; p += a256((size_t)B * KX * 2); }
@@ -1746,7 +1783,7 @@ TcWs carve_ws(const wm_handle *h, int B, void *ws, int T_teacher = -1) {
     w.rt = (float *)p; p += a256((size_t)B * 4);
     w.mem = (float *)p; p += a256((size_t)B * 4);
     if (c.n_xfers > 0) {
-        w.logits = (float *)p; p += a256((size_t)B * c.a_dim * 4);
+        w.logits = (float *)p; p += a256((size_t)B * h->tc.Ap * 4);
         w.act2 = (int32_t *)p; p += a256((size_t)B * 4);
     }
     if (can_compact(c)) {
@@ -1768,38 +1805,128 @@ TcWs carve_ws(const wm_handle *h, int B, void *ws, int T_teacher = -1) {
     return w;
 }
 
+// ---------------------------------------------------------------------------
+// The packed operands, from the stepwise family's fp32 matrices (on a bf16 model their values are
+// bf16 numbers already): dst [rows, cols] = bf16(src), and its lo part bf16(src - hi) when asked.
+//   PACK_GATES    row n = 4 U j + U gate + u, U = units, column k: unit U j + u's gate against
+//                 operand column k (z | h); the bias in the same row order
+//   PACK_ACTIONS  dst [A, 4Hp]: action row a with its columns in PACK_GATES's row order
+//   PACK_HEADS    row 240 j + DS i + 3 k + p: dim j dpt + i, component k, part p; reward, done ...
+//                 rows from (rd_tile, rd_col) on
+//   PACK_CTRL     row P Ap: candidate, action
+// Padding is 0.  (Host loops over these took several ms of wm_create; one thread per element here.)
+enum { PACK_GATES, PACK_ACTIONS, PACK_HEADS, PACK_CTRL };
+struct PackGeo {
+    int Z, A, H, K, Zp, Hp, dpt, DS, rd_tile, rd_col, NR, Ap;
+};
+template <int WHAT>
+__global__ void k_tc_pack(PackGeo g, int units, int rows, int cols, const float *__restrict__ src, long lds,
+                          __nv_bfloat16 *__restrict__ hi, __nv_bfloat16 *__restrict__ lo,
+                          const float *__restrict__ bsrc, float *__restrict__ bias) {
+    const size_t n_el = (size_t)rows * cols;
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n_el; i += (size_t)gridDim.x * blockDim.x) {
+        // PACK_ACTIONS runs along the packed row (n), the others along k
+        const int n = WHAT == PACK_ACTIONS ? (int)(i % rows) : (int)(i / cols);
+        const int k = WHAT == PACK_ACTIONS ? (int)(i / rows) : (int)(i % cols);
+        long col = -1;  // the source column of packed row n
+        const float *s = src, *b = bsrc;
+        if (WHAT == PACK_GATES || WHAT == PACK_ACTIONS) {
+            const int j = n / (4 * units), gate = n % (4 * units) / units, u = units * j + n % units;
+            if (u < g.H) col = (long)gate * g.H + u;
+        } else if (WHAT == PACK_HEADS) {
+            const int tile = n / HEAD_TILE, r = n % HEAD_TILE, d = tile * g.dpt + r / g.DS, q = r % g.DS;
+            if (tile == g.rd_tile && r >= g.rd_col) {
+                if (r - g.rd_col < g.NR) col = 3L * g.K * g.Z + (r - g.rd_col);
+            } else if (r / g.DS < g.dpt && d < g.Z && q < 3 * g.K) {
+                col = (long)(q % 3) * g.K * g.Z + (long)d * g.K + q / 3;
+            }
+        } else {
+            const int cand = n / g.Ap, a = n % g.Ap;
+            if (a < g.A) col = a;
+            s += (size_t)cand * (g.Z + g.H) * g.A;  // (cand = 0 unless src is the population's)
+            b += (size_t)cand * g.A;
+        }
+        long row = k;  // the source row of packed column k
+        if (WHAT == PACK_GATES || WHAT == PACK_CTRL)
+            row = k < g.Z ? k : (k >= g.Zp && k - g.Zp < g.H) ? g.Z + (k - g.Zp) : -1;
+        if (WHAT == PACK_HEADS && k >= g.H) row = -1;
+        const float v = col >= 0 && row >= 0 ? s[row * lds + col] : 0.f;
+        const __nv_bfloat16 h = __float2bfloat16_rn(v);
+        const size_t o = WHAT == PACK_ACTIONS ? (size_t)k * rows + n : i;
+        hi[o] = h;
+        if (lo) lo[o] = __float2bfloat16_rn(v - __bfloat162float(h));
+        if (WHAT != PACK_ACTIONS && k == 0) bias[n] = col >= 0 ? b[col] : 0.f;
+    }
+}
+
 }  // namespace
 
 // ---------------------------------------------------------------------------
 // Host side: packing, support test, per-call orchestration.
 
-int wm_tc_supported(const wm_handle *h) { return h->tc.ok; }
+int wm_tc_supported(const wm_handle *h) { return h->tc.ok && h->tc.aligned; }
+int wm_tc_auto_ok(const wm_handle *h) { return h->tc.ok && h->cfg.precision == WM_BF16; }
 
 size_t wm_tc_ws(const wm_handle *h, int B, int T_teacher) {
     const wm_config &c = h->cfg;
-    const size_t KX = (size_t)c.z_dim + c.h_dim, H = c.h_dim;
+    const size_t KX = (size_t)h->tc.Zp + h->tc.Hp, H = h->tc.Hp;
     const size_t rows = T_teacher >= 0 ? (size_t)(T_teacher + 1) * B : 0;
     const size_t teach = T_teacher >= 0 ? (c.precision == WM_FP32 ? 2 : 1) * a256(rows * KX * 2) +
                                               a256((size_t)4 * h->tc.n_head_tiles * T_teacher * B * 4)
                                         : 0;
     return teach + 2 * a256((size_t)B * KX * 2) + 2 * a256((size_t)B * H * 4) + a256((size_t)B * 4) + 2 * a256(B) +
            2 * a256((size_t)B * 4) + a256((size_t)4 * h->tc.n_head_tiles * B * 4) + 256 +
-           (c.n_xfers > 0 ? a256((size_t)B * c.a_dim * 4) + a256((size_t)B * 4) : 0) +
+           (c.n_xfers > 0 ? a256((size_t)B * h->tc.Ap * 4) + a256((size_t)B * 4) : 0) +
            (can_compact(c) ? 3 * a256((size_t)B * H * 4) + 3 * a256((size_t)B * 4) + 256 : 0) +
            (c.precision == WM_FP32 ? 2 * a256((size_t)B * KX * 2) : 0);
 }
 
-cudaError_t wm_tc_pack(wm_handle *h, const wm_weights *w) {
+// Packs the controllers of the stepwise family's weights (one in Wg / bg, P > 1 candidates in
+// Wp / bp): W_c^T [P Ap, KX] and b_c [P, Ap].
+cudaError_t wm_tc_set_controllers(wm_handle *h, int P) {
+    wm_tc_weights &T = h->tc;
+    const wm_config &c = h->cfg;
+    const int A = c.a_dim, H = c.h_dim, KX = T.Zp + T.Hp;
+    const size_t bytes = (size_t)P * T.Ap * KX * 2;
+    cudaFree(T.wc);
+    cudaFree(T.wc_lo);
+    cudaFree(T.bc);
+    T.wc = T.wc_lo = nullptr;
+    T.bc = nullptr;
+    cudaError_t e = cudaMalloc(&T.wc, bytes);
+    if (e == cudaSuccess && c.precision == WM_FP32) e = cudaMalloc(&T.wc_lo, bytes);
+    if (e == cudaSuccess) e = cudaMalloc((void **)&T.bc, (size_t)P * T.Ap * 4);
+    if (e != cudaSuccess) return e;
+    PackGeo g{c.z_dim, A, H, c.k_mix, T.Zp, T.Hp};
+    g.Ap = T.Ap;
+    const bool pop = P > 1;
+    k_tc_pack<PACK_CTRL><<<1024, 256>>>(g, 0, P * T.Ap, KX, pop ? h->step.Wp : h->step.Wg + 4 * H, pop ? A : 4L * H + A,
+                                        (__nv_bfloat16 *)T.wc, (__nv_bfloat16 *)T.wc_lo,
+                                        pop ? h->step.bp : h->step.bg + 4 * H, T.bc);
+    e = cudaGetLastError();
+    return e != cudaSuccess ? e : cudaDeviceSynchronize();
+}
+
+cudaError_t wm_tc_pack(wm_handle *h) {
     const wm_config &c = h->cfg;
     wm_tc_weights &T = h->tc;
     memset(&T, 0, sizeof(T));
-    const int Z = c.z_dim, A = c.a_dim, H = c.h_dim, K = c.k_mix, KX = Z + H;
-    // fp32 models: the split path (flat actions only: the gate epilogue's second-row slots
-    // carry the action row's lo part)
+    const int Z = c.z_dim, A = c.a_dim, H = c.h_dim, K = c.k_mix;
     const bool f32 = c.precision == WM_FP32;
-    if ((f32 && c.n_xfers > 0) || H % 64 != 0 || A % 64 != 0 || (A > 256 && A != 512) || K > 8 || Z % 8 != 0 ||
-        !get_encode())
-        return cudaSuccess;
+    if (A > 512 || K > 8 || !get_encode()) return cudaSuccess;
+    const bool aligned = H % 64 == 0 && A % 64 == 0 && (A <= 256 || A == 512) && Z % 8 == 0;
+    // fp32 models: the split path (flat actions only: the gate epilogue's second-row slots
+    // carry the action row's lo part).  It takes no padded sizes: those stay with the stepwise
+    // family, whose fp32 sums are more accurate than three bf16 products.
+    if (f32 && (c.n_xfers > 0 || !aligned)) return cudaSuccess;
+    // The sizes rounded up to the tiles' granularity, with zero weights: a padded hidden unit has
+    // gates sigma(0), tanh(0) and stays exactly 0, a padded latent column is 0 and no epilogue
+    // makes one, a padded action is never valid.
+    const int Zp = (Z + 7) & ~7, Hp = (H + 63) & ~63, Ap = A > 256 ? 512 : (A + 63) & ~63, KX = Zp + Hp;
+    T.Zp = Zp;
+    T.Hp = Hp;
+    T.Ap = Ap;
+    T.aligned = aligned;
     const int DS = (3 * K + 7) & ~7;  // head columns per latent dim
     const int dpt = HEAD_TILE / DS;
     int nht = (Z + dpt - 1) / dpt;
@@ -1814,144 +1941,30 @@ cudaError_t wm_tc_pack(wm_handle *h, const wm_weights *w) {
     T.n_head_tiles = nht;
     T.rd_tile = rd_tile;
     T.rd_col = rd_col;
-    auto bf = [](float v) { return __float2bfloat16_rn(v); };
-    // controller: W_c^T [A, KX]
-    std::vector<__nv_bfloat16> wc((size_t)A * KX), wg((size_t)4 * H * KX), wa((size_t)A * 4 * H),
-        wh((size_t)nht * HEAD_TILE * H, bf(0.f));
-    std::vector<float> bc(A), bg(4 * H), bh((size_t)nht * HEAD_TILE, 0.f);
-    for (int a = 0; a < A; ++a) {
-        for (int k = 0; k < KX; ++k) wc[(size_t)a * KX + k] = bf(w->W_ctrl[(size_t)k * A + a]);
-        bc[a] = w->b_ctrl[a];
-    }
-    // gates: row n = 256*j + 64*gate + u  <->  canonical column gate*H + 64*j + u
-    for (int n = 0; n < 4 * H; ++n) {
-        const int j = n / 256, gate = (n % 256) / 64, u = n % 64;
-        const size_t col = (size_t)gate * H + 64 * j + u;
-        for (int k = 0; k < KX; ++k) {
-            const size_t src = k < Z ? k : k + A;
-            wg[(size_t)n * KX + k] = bf(w->W_lstm[src * 4 * H + col]);
-        }
-        bg[n] = w->b_lstm[col];
-        for (int a = 0; a < A; ++a) wa[(size_t)a * 4 * H + n] = bf(w->W_lstm[(size_t)(Z + a) * 4 * H + col]);
-    }
-    // heads: tile j, local dim i, component k, part p -> row j*240 + DS*i + 3k + p
-    const size_t M = (size_t)3 * K * Z;
-    for (int d = 0; d < Z; ++d)
-        for (int part = 0; part < 3; ++part)
-            for (int k = 0; k < K; ++k) {
-                const size_t row = (size_t)(d / dpt) * HEAD_TILE + DS * (d % dpt) + 3 * k + part;
-                const size_t col = (size_t)part * K * Z + (size_t)d * K + k;
-                for (int i = 0; i < H; ++i) wh[row * H + i] = bf(w->W_mdn[(size_t)i * M + col]);
-                bh[row] = w->b_mdn[col];
-            }
-    {
-        const size_t rr = (size_t)rd_tile * HEAD_TILE + rd_col;
-        for (int i = 0; i < H; ++i) {
-            wh[rr * H + i] = bf(w->w_rew[i]);
-            wh[(rr + 1) * H + i] = bf(w->w_done[i]);
-        }
-        bh[rr] = w->b_rew;
-        bh[rr + 1] = w->b_done;
-        if (c.reward_mode == WM_REWARD_SHAPED) {
-            for (int i = 0; i < H; ++i) {
-                wh[(rr + 2) * H + i] = bf(w->w_rt[i]);
-                wh[(rr + 3) * H + i] = bf(w->w_mem[i]);
-            }
-            bh[rr + 2] = w->b_rt;
-            bh[rr + 3] = w->b_mem;
-        }
-        if (c.value_head) {
-            for (int i = 0; i < H; ++i) wh[(rr + h->NR - 1) * H + i] = bf(w->w_val[i]);
-            bh[rr + h->NR - 1] = w->b_val;
-        }
-    }
-    cudaError_t e;
-    auto up = [&](void **dst, const void *src, size_t bytes) {
-        cudaError_t r = cudaMalloc(dst, bytes);
-        if (r == cudaSuccess) r = cudaMemcpy(*dst, src, bytes, cudaMemcpyHostToDevice);
-        return r;
+    const size_t nhr = (size_t)nht * HEAD_TILE, wgs = (size_t)4 * Hp * KX * 2, was = (size_t)A * 4 * Hp * 2;
+    cudaError_t e = cudaSuccess;
+    auto room = [&](void **dst, size_t bytes) {
+        if (e == cudaSuccess) e = cudaMalloc(dst, bytes);
     };
-    if (f32) {  // the lo parts: bf16(w - hi), from the same canonical values
-        auto lo_of = [&](std::vector<__nv_bfloat16> &hi, auto canon) {
-            std::vector<__nv_bfloat16> lo(hi.size());
-            for (size_t i = 0; i < hi.size(); ++i) lo[i] = bf(canon(i) - __bfloat162float(hi[i]));
-            return lo;
-        };
-        auto wc_lo = lo_of(wc, [&](size_t i) { const size_t a = i / KX, k = i % KX; return w->W_ctrl[k * A + a]; });
-        auto wg_lo = lo_of(wg, [&](size_t i) {
-            const size_t n = i / KX, k = i % KX;
-            const size_t j = n / 256, gate = (n % 256) / 64, u = n % 64, col = gate * H + 64 * j + u;
-            const size_t src = k < (size_t)Z ? k : k + A;
-            return w->W_lstm[src * 4 * H + col];
-        });
-        auto wa_lo = lo_of(wa, [&](size_t i) {
-            const size_t a = i / (4 * H), n = i % (4 * H);
-            const size_t j = n / 256, gate = (n % 256) / 64, u = n % 64, col = gate * H + 64 * j + u;
-            return w->W_lstm[(Z + a) * 4 * H + col];
-        });
-        std::vector<float> whf(wh.size(), 0.f);  // canonical values of the packed head rows
-        for (int d = 0; d < Z; ++d)
-            for (int part = 0; part < 3; ++part)
-                for (int k = 0; k < K; ++k) {
-                    const size_t row = (size_t)(d / dpt) * HEAD_TILE + DS * (d % dpt) + 3 * k + part;
-                    const size_t col = (size_t)part * K * Z + (size_t)d * K + k;
-                    for (int i = 0; i < H; ++i) whf[row * H + i] = w->W_mdn[(size_t)i * M + col];
-                }
-        {
-            const size_t rr = (size_t)rd_tile * HEAD_TILE + rd_col;
-            for (int i = 0; i < H; ++i) {
-                whf[rr * H + i] = w->w_rew[i];
-                whf[(rr + 1) * H + i] = w->w_done[i];
-                if (c.reward_mode == WM_REWARD_SHAPED) {
-                    whf[(rr + 2) * H + i] = w->w_rt[i];
-                    whf[(rr + 3) * H + i] = w->w_mem[i];
-                }
-                if (c.value_head) whf[(rr + h->NR - 1) * H + i] = w->w_val[i];
-            }
-        }
-        auto wh_lo = lo_of(wh, [&](size_t i) { return whf[i]; });
-        if ((e = up(&T.wc_lo, wc_lo.data(), wc_lo.size() * 2)) != cudaSuccess) return e;
-        if ((e = up(&T.wg_lo, wg_lo.data(), wg_lo.size() * 2)) != cudaSuccess) return e;
-        if ((e = up(&T.wa_lo, wa_lo.data(), wa_lo.size() * 2)) != cudaSuccess) return e;
-        if ((e = up(&T.wh_lo, wh_lo.data(), wh_lo.size() * 2)) != cudaSuccess) return e;
-    }
-    {  // 128-column gate tiles: row n = 128 j + 32 gate + u <-> column gate H + 32 j + u
-        std::vector<__nv_bfloat16> wgn((size_t)4 * H * KX), wan((size_t)A * 4 * H);
-        std::vector<__nv_bfloat16> wgnl(f32 ? wgn.size() : 0), wanl(f32 ? wan.size() : 0);
-        std::vector<float> bgn(4 * H);
-        auto lo = [&](float v, __nv_bfloat16 hi) { return bf(v - __bfloat162float(hi)); };
-        for (int n = 0; n < 4 * H; ++n) {
-            const int j = n / 128, gate = (n % 128) / 32, u = n % 32;
-            const size_t col = (size_t)gate * H + 32 * j + u;
-            for (int k = 0; k < KX; ++k) {
-                const size_t src = k < Z ? k : k + A, i = (size_t)n * KX + k;
-                const float v = w->W_lstm[src * 4 * H + col];
-                wgn[i] = bf(v);
-                if (f32) wgnl[i] = lo(v, wgn[i]);
-            }
-            bgn[n] = w->b_lstm[col];
-            for (int a = 0; a < A; ++a) {
-                const size_t i = (size_t)a * 4 * H + n;
-                const float v = w->W_lstm[(size_t)(Z + a) * 4 * H + col];
-                wan[i] = bf(v);
-                if (f32) wanl[i] = lo(v, wan[i]);
-            }
-        }
-        if ((e = up(&T.wg_n, wgn.data(), wgn.size() * 2)) != cudaSuccess) return e;
-        if ((e = up(&T.wa_n, wan.data(), wan.size() * 2)) != cudaSuccess) return e;
-        if ((e = up((void **)&T.bg_n, bgn.data(), bgn.size() * 4)) != cudaSuccess) return e;
-        if (f32) {
-            if ((e = up(&T.wg_n_lo, wgnl.data(), wgnl.size() * 2)) != cudaSuccess) return e;
-            if ((e = up(&T.wa_n_lo, wanl.data(), wanl.size() * 2)) != cudaSuccess) return e;
-        }
-    }
-    if ((e = up(&T.wc, wc.data(), wc.size() * 2)) != cudaSuccess) return e;
-    if ((e = up(&T.wg, wg.data(), wg.size() * 2)) != cudaSuccess) return e;
-    if ((e = up(&T.wa, wa.data(), wa.size() * 2)) != cudaSuccess) return e;
-    if ((e = up(&T.wh, wh.data(), wh.size() * 2)) != cudaSuccess) return e;
-    if ((e = up((void **)&T.bc, bc.data(), bc.size() * 4)) != cudaSuccess) return e;
-    if ((e = up((void **)&T.bg, bg.data(), bg.size() * 4)) != cudaSuccess) return e;
-    if ((e = up((void **)&T.bh, bh.data(), bh.size() * 4)) != cudaSuccess) return e;
+    for (void **d : {&T.wg, &T.wg_n, f32 ? &T.wg_lo : nullptr, f32 ? &T.wg_n_lo : nullptr})
+        if (d) room(d, wgs);
+    for (void **d : {&T.wa, &T.wa_n, f32 ? &T.wa_lo : nullptr, f32 ? &T.wa_n_lo : nullptr})
+        if (d) room(d, was);
+    room(&T.wh, nhr * Hp * 2);
+    if (f32) room(&T.wh_lo, nhr * Hp * 2);
+    room((void **)&T.bg, (size_t)4 * Hp * 4);
+    room((void **)&T.bg_n, (size_t)4 * Hp * 4);
+    room((void **)&T.bh, nhr * 4);
+    if (e != cudaSuccess) return e;
+    const PackGeo g{Z, A, H, K, Zp, Hp, dpt, DS, rd_tile, rd_col, h->NR};
+    const long lg = 4L * H + A, lh = h->M + h->NR;
+    using bf = __nv_bfloat16;
+    k_tc_pack<PACK_GATES><<<1024, 256>>>(g, 64, 4 * Hp, KX, h->step.Wg, lg, (bf *)T.wg, (bf *)T.wg_lo, h->step.bg, T.bg);
+    k_tc_pack<PACK_GATES><<<1024, 256>>>(g, 32, 4 * Hp, KX, h->step.Wg, lg, (bf *)T.wg_n, (bf *)T.wg_n_lo, h->step.bg, T.bg_n);
+    k_tc_pack<PACK_ACTIONS><<<512, 256>>>(g, 64, 4 * Hp, A, h->step.Wa, 4L * H, (bf *)T.wa, (bf *)T.wa_lo, nullptr, nullptr);
+    k_tc_pack<PACK_ACTIONS><<<512, 256>>>(g, 32, 4 * Hp, A, h->step.Wa, 4L * H, (bf *)T.wa_n, (bf *)T.wa_n_lo, nullptr, nullptr);
+    k_tc_pack<PACK_HEADS><<<1024, 256>>>(g, 0, (int)nhr, Hp, h->step.Wh, lh, (bf *)T.wh, (bf *)T.wh_lo, h->step.bh, T.bh);
+    if ((e = wm_tc_set_controllers(h, 1)) != cudaSuccess) return e;
     int dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&T.sms, cudaDevAttrMultiProcessorCount, dev);
@@ -1962,35 +1975,6 @@ cudaError_t wm_tc_pack(wm_handle *h, const wm_weights *w) {
 int wm_tc_call_ok(const wm_handle *h, unsigned long long episode_offset) {
     // a 256-row tile must not straddle two candidates of a population
     return h->P <= 1 || (h->E % 256 == 0 && episode_offset % 256 == 0);
-}
-
-cudaError_t wm_tc_set_controllers(wm_handle *h, int P, const float *W_ctrl, const float *b_ctrl) {
-    wm_tc_weights &T = h->tc;
-    const wm_config &c = h->cfg;
-    const int A = c.a_dim, KX = c.z_dim + c.h_dim;
-    const bool f32 = c.precision == WM_FP32;
-    std::vector<__nv_bfloat16> wc((size_t)P * A * KX), wcl(f32 ? wc.size() : 0);
-    for (int g = 0; g < P; ++g)
-        for (int a = 0; a < A; ++a)
-            for (int k = 0; k < KX; ++k) {
-                const size_t i = ((size_t)g * A + a) * KX + k;
-                const float v = W_ctrl[((size_t)g * KX + k) * A + a];
-                wc[i] = __float2bfloat16_rn(v);
-                if (f32) wcl[i] = __float2bfloat16_rn(v - __bfloat162float(wc[i]));
-            }
-    cudaFree(T.wc);
-    cudaFree(T.wc_lo);
-    cudaFree(T.bc);
-    T.wc = nullptr;
-    T.wc_lo = nullptr;
-    T.bc = nullptr;
-    cudaError_t e = cudaMalloc(&T.wc, wc.size() * 2);
-    if (e == cudaSuccess) e = cudaMemcpy(T.wc, wc.data(), wc.size() * 2, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess && f32) e = cudaMalloc(&T.wc_lo, wcl.size() * 2);
-    if (e == cudaSuccess && f32) e = cudaMemcpy(T.wc_lo, wcl.data(), wcl.size() * 2, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMalloc((void **)&T.bc, (size_t)P * A * 4);
-    if (e == cudaSuccess) e = cudaMemcpy(T.bc, b_ctrl, (size_t)P * A * 4, cudaMemcpyHostToDevice);
-    return e;
 }
 
 void wm_tc_free(wm_handle *h) {
@@ -2012,11 +1996,12 @@ static cudaError_t tc_run(const wm_handle *h, int teacher, const wm_rollout_dev 
     const wm_config &c = h->cfg;
     const wm_tc_weights &T = h->tc;
     const int B = teacher ? na->N : ra->B, Tn = teacher ? na->T : ra->T;
-    const int Z = c.z_dim, A = c.a_dim, H = c.h_dim, KX = Z + H;
+    const int Z = c.z_dim, A = c.a_dim, H = c.h_dim, Zp = T.Zp, Hp = T.Hp, Ap = T.Ap, KX = Zp + Hp;
     if (B == 0) { h->last_launches = 0; return cudaSuccess; }
     TcWs w = carve_ws(h, B, ws, teacher ? Tn : -1);
     StepIO io{};
     io.B = B; io.Z = Z; io.A = A; io.H = H; io.K = c.k_mix; io.T = Tn;
+    io.Zp = Zp; io.Hp = Hp; io.Ap = Ap;
     io.seed = c.seed; io.teacher = teacher;
     io.ctrl_sample = c.ctrl_sample; io.ctrl_tau = c.ctrl_tau; io.mdn_tau = c.mdn_tau;
     io.sigma_sqrt_tau = c.sigma_sqrt_tau; io.done_terminates = c.done_terminates;
@@ -2069,7 +2054,8 @@ static cudaError_t tc_run(const wm_handle *h, int teacher, const wm_rollout_dev 
         k_tc_init<<<init_grid, 256, 0, s>>>(io, teacher ? nullptr : ra->z0, teacher ? nullptr : ra->h0,
                                             teacher ? nullptr : ra->c0,
                                             (teacher || compact) ? nullptr : ra->done0,
-                                            teacher ? w.xall : w.x[0], teacher ? w.xall_lo : w.x_lo[0], w.fz[0], w.fz[1],
+                                            teacher ? w.xall : w.x[0], teacher ? w.xall_lo : w.x_lo[0],
+                                            teacher ? nullptr : w.x[1], w.fz[0], w.fz[1],
                                             T.n_head_tiles, compact ? w.dstep : nullptr,
                                             compact ? w.cnt : nullptr);
     }
@@ -2080,21 +2066,24 @@ static cudaError_t tc_run(const wm_handle *h, int teacher, const wm_rollout_dev 
         if (he != cudaSuccess) return he;
     }
     const bool f32 = c.precision == WM_FP32;  // the split path: second operand maps and lo outputs
+    // The calls that AUTO would give to the stepwise family if this one took aligned sizes and
+    // B >= 256 only (padded sizes, small bf16 batches) keep that family's accurate nonlinearities.
+    const bool acc = !f32 && (!T.aligned || (c.path == WM_PATH_AUTO && B < 256));
     CUtensorMap mx[2], mxs[2], mwc, mwg, mwh, mc, mc2, mxl[2], mxsl[2], mwcl, mwgl, mwhl;
     // B-operand boxes are half an instantiated BN (each CTA of a pair loads half the rows;
     // rows past A read as zero)
-    const uint32_t ctrl_box = A > 128 ? 128u : 64u;
+    const uint32_t ctrl_box = Ap > 128 ? 128u : 64u;
     if (!make_map(&mx[0], w.x[0], B, KX, BM) || !make_map(&mx[1], w.x[1], B, KX, BM) ||
         !make_map(&mxs[0], w.x[0], B, KX, 32) || !make_map(&mxs[1], w.x[1], B, KX, 32) ||
-        !make_map(&mc, w.c, B, H, 32, true) || (compact && !make_map(&mc2, w.c2, B, H, 32, true)) ||
-        !make_map(&mwc, T.wc, (uint64_t)h->P * A, KX, ctrl_box) || !make_map(&mwg, T.wg, 4 * H, KX, 128) ||
-        !make_map(&mwh, T.wh, (uint64_t)T.n_head_tiles * HEAD_TILE, H, HEAD_TILE / 2))
+        !make_map(&mc, w.c, B, Hp, 32, true) || (compact && !make_map(&mc2, w.c2, B, Hp, 32, true)) ||
+        !make_map(&mwc, T.wc, (uint64_t)h->P * Ap, KX, ctrl_box) || !make_map(&mwg, T.wg, 4 * Hp, KX, 128) ||
+        !make_map(&mwh, T.wh, (uint64_t)T.n_head_tiles * HEAD_TILE, Hp, HEAD_TILE / 2))
         return cudaErrorInvalidValue;
     if (f32) {
         if (!make_map(&mxl[0], w.x_lo[0], B, KX, BM) || !make_map(&mxl[1], w.x_lo[1], B, KX, BM) ||
             !make_map(&mxsl[0], w.x_lo[0], B, KX, 32) || !make_map(&mxsl[1], w.x_lo[1], B, KX, 32) ||
-            !make_map(&mwcl, T.wc_lo, (uint64_t)h->P * A, KX, ctrl_box) || !make_map(&mwgl, T.wg_lo, 4 * H, KX, 128) ||
-            !make_map(&mwhl, T.wh_lo, (uint64_t)T.n_head_tiles * HEAD_TILE, H, HEAD_TILE / 2))
+            !make_map(&mwcl, T.wc_lo, (uint64_t)h->P * Ap, KX, ctrl_box) || !make_map(&mwgl, T.wg_lo, 4 * Hp, KX, 128) ||
+            !make_map(&mwhl, T.wh_lo, (uint64_t)T.n_head_tiles * HEAD_TILE, Hp, HEAD_TILE / 2))
             return cudaErrorInvalidValue;
     } else {  // unused by the bf16 kernels
         mxl[0] = mx[0]; mxl[1] = mx[1]; mxsl[0] = mxs[0]; mxsl[1] = mxs[1];
@@ -2109,19 +2098,19 @@ static cudaError_t tc_run(const wm_handle *h, int teacher, const wm_rollout_dev 
     // tiles, or compacted live rows (bf16, flat actions); on the fp32 path, scoring
     const int pairs = T.sms / 2;
     const bool narrow = !hier && T.wg_n &&
-                        (f32 ? teacher && T.wg_n_lo : (compact || teacher || m_tiles * (H / 64) < pairs));
+                        (f32 ? teacher && T.wg_n_lo : (compact || teacher || m_tiles * (Hp / 64) < pairs));
     CUtensorMap mwgn, mwgnl, mxsn[2];
-    if (narrow && (!make_map(&mwgn, T.wg_n, 4 * H, KX, 64) || !make_map_x32(&mxsn[0], w.x[0], B, KX) ||
+    if (narrow && (!make_map(&mwgn, T.wg_n, 4 * Hp, KX, 64) || !make_map_x32(&mxsn[0], w.x[0], B, KX) ||
                    !make_map_x32(&mxsn[1], w.x[1], B, KX)))
         return cudaErrorInvalidValue;
-    if (narrow && f32 && !make_map(&mwgnl, T.wg_n_lo, 4 * H, KX, 64)) return cudaErrorInvalidValue;
+    if (narrow && f32 && !make_map(&mwgnl, T.wg_n_lo, 4 * Hp, KX, 64)) return cudaErrorInvalidValue;
     StepIO gio_n;  // the gate launches' parameters with the 128-column packing
     if (teacher) {  // batched scoring: the recurrence step by step, then one head GEMM
         const size_t fr = (size_t)B * KX;  // elements of one frame of operand rows
         cudaError_t e = cudaSuccess;
         if (Tn > 0) {
             wm_ktime kt(h, WM_KERNEL_AUX, s);
-            k_tc_frames<<<init_grid, 256, 0, s>>>(B, Tn, Z, KX, na->z_seq, w.xall, w.xall_lo);
+            k_tc_frames<<<init_grid, 256, 0, s>>>(B, Tn, Z, Zp, KX, na->z_seq, w.xall, w.xall_lo);
             ++launches;
         }
         io.x_cur = io.x_next = io.x_next_lo = nullptr;
@@ -2139,7 +2128,7 @@ static cudaError_t tc_run(const wm_handle *h, int teacher, const wm_rollout_dev 
                 mal = ma;
                 msl = ms;
             }
-            GemmGrid g2{m_tiles, H / 64, (KX + BK - 1) / BK, 0, h->status};
+            GemmGrid g2{m_tiles, Hp / 64, (KX + BK - 1) / BK, 0, h->status};
             if (t == 0) {  // an injected wait (wm_inject_wait_timeout) goes to the first GEMM
                 g2.test_wait = h->test_wait;
                 h->test_wait = 0;
@@ -2153,7 +2142,7 @@ static cudaError_t tc_run(const wm_handle *h, int teacher, const wm_rollout_dev 
                 gio_n.wa = (const __nv_bfloat16 *)T.wa_n;
                 gio_n.b_gate = T.bg_n;
                 GemmGrid g2n = g2;
-                g2n.n_tiles = H / 32;
+                g2n.n_tiles = Hp / 32;
                 wm_ktime kt(h, WM_KERNEL_TC_GATES, s);
                 if (f32) {
                     gio_n.wa_lo = (const __nv_bfloat16 *)T.wa_n_lo;
@@ -2161,11 +2150,13 @@ static cudaError_t tc_run(const wm_handle *h, int teacher, const wm_rollout_dev 
                     e = launch_gemm<128, 1, 3, EpiGates32N, 2, 3>(opn, mc, msn, msnl, g2n, gio_n, T.sms, s, pdl);
                 } else {
                     const OpMaps opn{&ma, &mwgn, &ma, &mwgn};
-                    e = launch_gemm<128, 1, 3, EpiGatesN, 2>(opn, mc, msn, msn, g2n, gio_n, T.sms, s, pdl);
+                    e = acc ? launch_gemm<128, 1, 3, EpiGatesNA, 2>(opn, mc, msn, msn, g2n, gio_n, T.sms, s, pdl)
+                            : launch_gemm<128, 1, 3, EpiGatesN, 2>(opn, mc, msn, msn, g2n, gio_n, T.sms, s, pdl);
                 }
             } else {
                 wm_ktime kt(h, WM_KERNEL_TC_GATES, s);
                 if (f32) e = launch_gemm<256, 1, 2, EpiGates32, 2, 3>(opg, mc, ms, msl, g2, io, T.sms, s, pdl);
+                else if (acc) e = launch_gemm<256, 1, 2, EpiGatesA, 2>(opg, mc, ms, ms, g2, io, T.sms, s, pdl);
                 else e = launch_gemm<256, 1, 2, EpiGates, 2>(opg, mc, ms, ms, g2, io, T.sms, s, pdl);
             }
             ++launches;
@@ -2187,7 +2178,7 @@ static cudaError_t tc_run(const wm_handle *h, int teacher, const wm_rollout_dev 
             hio.nseq = B;
             hio.z_tgt = na->z_seq + (size_t)B * Z;
             hio.nll_part = w.part;
-            const GemmGrid g3{(rows + 2 * BM - 1) / (2 * BM), T.n_head_tiles, (H + BK - 1) / BK, Z, h->status};
+            const GemmGrid g3{(rows + 2 * BM - 1) / (2 * BM), T.n_head_tiles, (Hp + BK - 1) / BK, Zp, h->status};
             const OpMaps oph{&mh, &mwh, &mhl, &mwhl};
             wm_ktime kt(h, WM_KERNEL_TC_HEADS, s);
             if (f32) e = launch_gemm<HEAD_TILE, 1, 3, EpiHeads, 2, 3>(oph, mc, mc, mc, g3, hio, T.sms, s, pdl);
@@ -2237,7 +2228,7 @@ static cudaError_t tc_run(const wm_handle *h, int teacher, const wm_rollout_dev 
     if (compact) {
         q.dead_flag = early ? h->dead_dev : nullptr;
         q.call_id = ++h->call_seq;
-        q.B = B; q.Z = Z; q.H = H; q.KX = KX; q.M = 3 * c.k_mix * Z; q.T = Tn;
+        q.B = B; q.Z = Z; q.H = H; q.Hp = Hp; q.KX = KX; q.M = 3 * c.k_mix * Z; q.T = Tn;
         q.fill = staged;  // staged outputs leave step by step: fill each step's
         q.dstep = w.dstep; q.h32 = w.h32;
         q.hfin = w.hfin; q.cfin = w.cfin; q.rt = w.rt; q.mem = w.mem;
@@ -2305,7 +2296,7 @@ static cudaError_t tc_run(const wm_handle *h, int teacher, const wm_rollout_dev 
             if (e != cudaSuccess) break;
         }
         // the controller's weight rows: the tile's candidate's, when there is a population
-        GemmGrid g1{m_tiles, 1, (KX + BK - 1) / BK, 0, h->status, teacher ? 0ull : ra->ep0, h->P, h->E, A};
+        GemmGrid g1{m_tiles, 1, (KX + BK - 1) / BK, 0, h->status, teacher ? 0ull : ra->ep0, h->P, h->E, Ap};
         g1.n_rows = io.n_rows;
         // an injected wait (wm_inject_wait_timeout) goes to the call's first GEMM launch
         uint32_t test_wait = 0;
@@ -2319,12 +2310,12 @@ static cudaError_t tc_run(const wm_handle *h, int teacher, const wm_rollout_dev 
         if (!teacher && !hier) {
             wm_ktime kt(h, WM_KERNEL_TC_CTRL, s);
             if (f32) {
-                if (A > 256) e = launch_gemm<256, 2, 2, EpiCtrl, 2, 3>(opc, mc, mc, mc, g1, io, T.sms, s, pdl);
-                else if (A > 128) e = launch_gemm<256, 1, 3, EpiCtrl, 2, 3>(opc, mc, mc, mc, g1, io, T.sms, s, pdl);
+                if (Ap > 256) e = launch_gemm<256, 2, 2, EpiCtrl, 2, 3>(opc, mc, mc, mc, g1, io, T.sms, s, pdl);
+                else if (Ap > 128) e = launch_gemm<256, 1, 3, EpiCtrl, 2, 3>(opc, mc, mc, mc, g1, io, T.sms, s, pdl);
                 else e = launch_gemm<128, 1, 3, EpiCtrl, 2, 3>(opc, mc, mc, mc, g1, io, T.sms, s, pdl);
             } else {
-                if (A > 256) e = launch_gemm<256, 2, 2, EpiCtrl, 2>(opc, mc, mc, mc, g1, io, T.sms, s, pdl);
-                else if (A > 128) e = launch_gemm<256, 1, 3, EpiCtrl, 2>(opc, mc, mc, mc, g1, io, T.sms, s, pdl);
+                if (Ap > 256) e = launch_gemm<256, 2, 2, EpiCtrl, 2>(opc, mc, mc, mc, g1, io, T.sms, s, pdl);
+                else if (Ap > 128) e = launch_gemm<256, 1, 3, EpiCtrl, 2>(opc, mc, mc, mc, g1, io, T.sms, s, pdl);
                 else e = launch_gemm<128, 1, 3, EpiCtrl, 2>(opc, mc, mc, mc, g1, io, T.sms, s, pdl);
             }
             ++launches;
@@ -2332,8 +2323,8 @@ static cudaError_t tc_run(const wm_handle *h, int teacher, const wm_rollout_dev 
         } else if (hier) {  // the logits, then the two-stage choice (Sec. 3.1.3); bf16 models only
             {
                 wm_ktime kt(h, WM_KERNEL_TC_CTRL, s);
-                if (A > 256) e = launch_gemm<256, 2, 2, EpiLogits, 2>(opc, mc, mc, mc, g1, io, T.sms, s, pdl);
-                else if (A > 128) e = launch_gemm<256, 1, 3, EpiLogits, 2>(opc, mc, mc, mc, g1, io, T.sms, s, pdl);
+                if (Ap > 256) e = launch_gemm<256, 2, 2, EpiLogits, 2>(opc, mc, mc, mc, g1, io, T.sms, s, pdl);
+                else if (Ap > 128) e = launch_gemm<256, 1, 3, EpiLogits, 2>(opc, mc, mc, mc, g1, io, T.sms, s, pdl);
                 else e = launch_gemm<128, 1, 3, EpiLogits, 2>(opc, mc, mc, mc, g1, io, T.sms, s, pdl);
             }
             ++launches;
@@ -2344,7 +2335,7 @@ static cudaError_t tc_run(const wm_handle *h, int teacher, const wm_rollout_dev 
             }
             ++launches;
         }
-        GemmGrid g2{m_tiles, H / 64, (KX + BK - 1) / BK, 0, h->status};
+        GemmGrid g2{m_tiles, Hp / 64, (KX + BK - 1) / BK, 0, h->status};
         g2.n_rows = io.n_rows;
         if (teacher) g2.test_wait = test_wait;
         if (narrow) {
@@ -2352,23 +2343,27 @@ static cudaError_t tc_run(const wm_handle *h, int teacher, const wm_rollout_dev 
             gio_n.wa = (const __nv_bfloat16 *)T.wa_n;
             gio_n.b_gate = T.bg_n;
             GemmGrid g2n = g2;
-            g2n.n_tiles = H / 32;
+            g2n.n_tiles = Hp / 32;
             const OpMaps opn{&mx[xa], &mwgn, &mx[xa], &mwgn};
             wm_ktime kt(h, WM_KERNEL_TC_GATES, s);
-            e = launch_gemm<128, 1, 3, EpiGatesN, 2>(opn, mC, mxsn[xn], mxsn[xn], g2n, gio_n, T.sms, s, pdl);
+            e = acc ? launch_gemm<128, 1, 3, EpiGatesNA, 2>(opn, mC, mxsn[xn], mxsn[xn], g2n, gio_n, T.sms, s, pdl)
+                    : launch_gemm<128, 1, 3, EpiGatesN, 2>(opn, mC, mxsn[xn], mxsn[xn], g2n, gio_n, T.sms, s, pdl);
         } else {
             wm_ktime kt(h, WM_KERNEL_TC_GATES, s);
             if (f32) e = launch_gemm<256, 1, 2, EpiGates32, 2, 3>(opg, mC, mxs[xn], mxsl[xn], g2, io, T.sms, s, pdl);
+            else if (hier && acc) e = launch_gemm<256, 1, 2, EpiGates2A, 2>(opg, mC, mxs[xn], mxs[xn], g2, io, T.sms, s, pdl);
+            else if (acc) e = launch_gemm<256, 1, 2, EpiGatesA, 2>(opg, mC, mxs[xn], mxs[xn], g2, io, T.sms, s, pdl);
             else if (hier) e = launch_gemm<256, 1, 2, EpiGates2, 2>(opg, mC, mxs[xn], mxs[xn], g2, io, T.sms, s, pdl);
             else e = launch_gemm<256, 1, 2, EpiGates, 2>(opg, mC, mxs[xn], mxs[xn], g2, io, T.sms, s, pdl);
         }
         ++launches;
         if (e != cudaSuccess) break;
-        GemmGrid g3{m_tiles, T.n_head_tiles, (H + BK - 1) / BK, Z, h->status};
+        GemmGrid g3{m_tiles, T.n_head_tiles, (Hp + BK - 1) / BK, Zp, h->status};
         g3.n_rows = io.n_rows;
         {
             wm_ktime kt(h, WM_KERNEL_TC_HEADS, s);
             if (f32) e = launch_gemm<HEAD_TILE, 1, 3, EpiHeads, 2, 3>(oph, mc, mc, mc, g3, io, T.sms, s, pdl);
+            else if (acc) e = launch_gemm<HEAD_TILE, 1, 3, EpiHeadsA, 2>(oph, mc, mc, mc, g3, io, T.sms, s, pdl);
             else e = launch_gemm<HEAD_TILE, 1, 3, EpiHeads, 2>(oph, mc, mc, mc, g3, io, T.sms, s, pdl);
         }
         ++launches;
@@ -2385,14 +2380,14 @@ static cudaError_t tc_run(const wm_handle *h, int teacher, const wm_rollout_dev 
         if (ra->h_final || ra->c_final) {
             wm_ktime kt(h, WM_KERNEL_AUX, s);
             const int tl = t_end - 1;  // the last issued step
-            k_tc_finish_compact<<<init_grid, 256, 0, s>>>(B, H, Tn, w.dstep, w.rows[tl & 1], w.cnt + (tl & 3),
+            k_tc_finish_compact<<<init_grid, 256, 0, s>>>(B, H, Hp, Tn, w.dstep, w.rows[tl & 1], w.cnt + (tl & 3),
                                                           w.h32, cbuf[Tn & 1], w.hfin, w.cfin, ra->h_final,
                                                           ra->c_final);
             ++launches;
         }
     } else {
         wm_ktime kt(h, WM_KERNEL_AUX, s);
-        k_tc_finish<<<init_grid, 256, 0, s>>>(B, H, w.h32, w.c, teacher ? nullptr : ra->h_final,
+        k_tc_finish<<<init_grid, 256, 0, s>>>(B, H, Hp, w.h32, w.c, teacher ? nullptr : ra->h_final,
                                               teacher ? nullptr : ra->c_final, w.nll_part, 4 * T.n_head_tiles,
                                               teacher ? na->nll : nullptr);
         ++launches;

@@ -1,0 +1,93 @@
+"""The tensor-core family on sizes it pads (AUTO's choice for bf16 models the fused family does
+not take): tile edges, single columns and the largest of each range, against the oracle and
+against the stepwise family that served these calls before."""
+import numpy as np
+import pytest
+import torch
+
+import synth
+from parity import check_rollout, check_teacher, np_
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def wm():
+    import paper_2205_01435_gb300 as pkg
+    return pkg.load()
+
+
+def _cuda(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+def _cfg(Z, A, H, K, **flags):
+    return dict(synth.model_config("small_bf16"), z_dim=Z, a_dim=A, h_dim=H, k_mix=K, **flags)
+
+
+# Z, A, H, K, B, flags: one below / at / above the granularity of 8 (Z), 64 and 256 (A), 64 (H), 256 (B)
+ROLLOUT = [(1, 1, 1, 1, 1, {}), (7, 63, 63, 3, 255, {}), (8, 65, 65, 8, 257, dict(ctrl_sample=1)),
+           (33, 129, 130, 5, 300, dict(done_terminates=1)), (50, 257, 300, 6, 64, dict(ctrl_sample=1, value_head=1)),
+           (24, 512, 128, 8, 100, dict(reward_mode=1)), (81, 200, 190, 7, 513, dict(noop_terminates=1)),
+           (31, 90, 100, 4, 260, dict(n_xfers=23)), (64, 256, 512, 8, 60, {})]
+
+
+@pytest.mark.parametrize("Z,A,H,K,B,flags", ROLLOUT)
+def test_rollout(wm, orc, Z, A, H, K, B, flags):
+    cfg, T = _cfg(Z, A, H, K, **flags), 4
+    w = synth.weights(cfg, seed=31)
+    z0, x = synth.z0(B, Z, seed=31), {}
+    NX = cfg["n_xfers"]
+    if NX:
+        mask, x["loc_mask"] = synth.hier_masks(T, B, NX, A - NX, 0.5, seed=31)
+    else:
+        mask = synth.mask(T, B, A, 0.4, seed=31)
+        mask[..., -1] |= np.uint32(0xFFFFFFFF << (A % 32) & 0xFFFFFFFF if A % 32 else 0)  # bits past A mean nothing
+    if cfg["reward_mode"]:
+        x["rt0"], x["mem0"] = synth.shaping_state(B, seed=31)
+    h0 = np.tanh(synth.z0(B, H, seed=32)).astype(np.float32)
+    c0 = synth.z0(B, H, seed=33)
+    dev = {k: _cuda(v) for k, v in x.items()}
+    kw = dict(h0=_cuda(h0), c0=_cuda(c0), want_seq=True, want_logp=True, **dev)  # log-probs: not the fused family
+    m = wm.WorldModel(cfg, w)
+    g = m.rollout(_cuda(z0), T, mask=_cuda(mask), **kw)
+    m.sync()
+    assert m.last_path == "tensor"
+    r = check_rollout(g, cfg, w, z0, mask, h0=h0, c0=c0, orc=orc, **x)
+    assert r["compared"] > 0 or B == 1
+    nomask = m.rollout(_cuda(z0), T, **kw)
+    assert int(nomask["actions"].max()) < (NX or A)
+    # a workspace of another batch size before, and host arrays staged step by step, change nothing
+    n = B // 2 + 1
+    m.rollout(_cuda(z0[:n]), 2, **{k: dev[k][:n].contiguous() for k in ("rt0", "mem0") if k in dev})
+    pin = {k: torch.from_numpy(np.ascontiguousarray(v)).pin_memory() for k, v in dict(x, h0=h0, c0=c0).items()}
+    gh = m.rollout(torch.from_numpy(z0).pin_memory(), T, mask=torch.from_numpy(mask).pin_memory(), want_seq=True,
+                   want_logp=True, **pin)
+    for k in ("z", "actions", "rewards", "done", "h_final", "c_final", "h_seq", "logp_seq"):
+        assert torch.equal(gh[k], g[k].cpu()), k
+
+
+@pytest.mark.parametrize("Z,A,H,K,N,T", [(5, 45, 333, 3, 700, 3), (50, 101, 300, 6, 600, 5), (64, 256, 512, 5, 60, 4)])
+def test_scoring_and_training(wm, orc, Z, A, H, K, N, T):
+    cfg = _cfg(Z, A, H, K)
+    w = synth.weights(cfg, seed=34)
+    zs, acts, lens = synth.teacher_inputs(N, T, Z, A, seed=34, ragged=True)
+    acts[::2, ::3] = -1
+    m = wm.WorldModel(cfg, w)
+    g = m.mdn_nll(_cuda(zs), _cuda(acts), lengths=_cuda(lens), want_seq=True)
+    m.sync()
+    assert m.last_path == "tensor"
+    check_teacher({k: np_(v) for k, v in g.items()}, orc.mdn_nll(cfg, w, zs, acts, lengths=lens, want_seq=True), "bf16")
+    a = m.mdn_nll_backward(_cuda(zs), _cuda(acts), lengths=_cuda(lens))
+    s = wm.WorldModel(dict(cfg, path="stepwise"), w).mdn_nll_backward(_cuda(zs), _cuda(acts), lengths=_cuda(lens))
+    for k in ("W_lstm", "b_lstm", "W_mdn", "b_mdn", "nll"):
+        # both forwards round the same operands to bf16 (2^-9 each) and sum in fp32
+        assert float((a[k] - s[k]).norm() / s[k].norm()) < 1e-2, k
+
+
+def test_forced_path_still_refuses_unaligned_sizes(wm):
+    cfg = _cfg(50, 101, 300, 6, path="tensor")
+    m = wm.WorldModel(cfg, synth.weights(cfg))
+    with pytest.raises(wm.WMError) as e:
+        m.rollout(torch.zeros(300, 50, device="cuda"), 1)
+    assert e.value.status == wm.WM_ERR_UNSUPPORTED
