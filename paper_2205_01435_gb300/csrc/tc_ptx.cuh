@@ -9,6 +9,7 @@
 // descriptor's leading byte offset) is R*16 bytes and the row-direction stride
 // (stride byte offset) is 128 bytes.
 #pragma once
+#include <cuda.h>
 #include <stdint.h>
 
 namespace tc {
@@ -123,11 +124,36 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t saddr, uint32_t b
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" :: "r"(saddr), "r"(bytes)
                  : "memory");
 }
+// True in one lane of a full warp, and known to the compiler to be: a warp that runs its loop as a whole
+// and issues under this predicate keeps addresses and descriptors in uniform registers.  (A loop in
+// `if (lane == 0)` is divergent code: every TMA, MMA and loop turn then took 60 to 400 cycles more.)
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
 // Bounded wait: returns false if the phase did not complete within max_iter polls.
 __device__ __forceinline__ bool mbar_wait_bounded(uint32_t saddr, uint32_t parity, uint32_t max_iter) {
     for (uint32_t i = 0; i < max_iter; ++i)
         if (mbar_try_wait(saddr, parity)) return true;
     return false;
+}
+
+// ---- TMA tensor tiles (K-major bf16 operands, 128-byte swizzle) ---------------------
+__device__ __forceinline__ uint64_t desc_sw128(uint32_t saddr) {
+    uint64_t d = 0;
+    d |= (uint64_t)((saddr >> 4) & 0x3FFFu);
+    d |= (uint64_t)1u << 16;            // leading byte offset: unused for swizzled K-major
+    d |= (uint64_t)(1024u >> 4) << 32;  // stride byte offset: 8 rows x 128 B
+    d |= (uint64_t)1u << 46;            // descriptor version
+    d |= (uint64_t)2u << 61;            // 128-byte swizzle
+    return d;
+}
+
+__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map, int x, int y, uint32_t mbar) {
+    asm volatile(
+        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+        :: "r"(dst), "l"(map), "r"(x), "r"(y), "r"(mbar) : "memory");
 }
 
 // ---- clusters / distributed shared memory ------------------------------------

@@ -1,6 +1,7 @@
 // wm_internal.h -- handle layout and kernel-family launchers behind the C ABI
 // of include/wm.h.  Not part of the public interface.
 #pragma once
+#include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stddef.h>
 #include <stdint.h>
@@ -203,6 +204,30 @@ cudaError_t wm_tc_nll(const wm_handle *h, const wm_nll_dev &a, void *ws, cudaStr
 cudaError_t wm_tc_set_controllers(wm_handle *h, int P);
 // whether the tensor family can run a rollout call starting at this episode (population tiles)
 int wm_tc_call_ok(const wm_handle *h, unsigned long long episode_offset);
+
+// ---- the teacher-forced recurrence in one launch (wm_recur.cu) -----------------------
+// Row tiles a CTA takes in turn, at most (more: one launch per step keeps up).
+enum { RECUR_MAX_GROUPS = 4 };
+struct wm_recur_args {
+    int N, T, A, H, Zp, Hp, KX;
+    const int32_t *act;          // [T, N]
+    __nv_bfloat16 *x, *x_lo;     // [(T + 1) N, KX] operand rows of every frame (fp32 path: and lo parts)
+    const __nv_bfloat16 *wa, *wa_lo;  // [A, 4Hp] action rows, and the bias, in the 128-column packing
+    const float *bias;
+    float *h_seq, *c_seq;        // [T, N, H] or null
+    int *count;                  // [m_tiles] zero on entry
+    int *status;
+    uint32_t test_wait;
+    // the plan
+    int units, n_tiles, m_tiles, m_groups, groups, cluster, k_steps, stages, kps;
+    size_t smem;
+};
+// Whether (and how) N sequences run as one launch.
+bool wm_recur_plan(int mode, int N, int Hp, int KX, wm_recur_args *a);
+// mode: 0 bf16, 1 bf16 with accurate nonlinearities, 2 fp32 as bf16 parts.  Tensor maps: x rows in
+// boxes of 128 / cluster rows x 64, weights (128-column packing) in boxes of `units` rows x 64.
+cudaError_t wm_recur_launch(int mode, const void *x_map, const void *xl_map, const void *w_map, const void *wl_map,
+                            const wm_recur_args &a, cudaStream_t s);
 
 // ---- the fused family's small-batch member (wm_small.cu) ----------------------
 cudaError_t wm_small_prepare(wm_handle *h);

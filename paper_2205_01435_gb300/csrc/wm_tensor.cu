@@ -36,6 +36,8 @@
 #include "wm_internal.h"
 
 using namespace wmk;
+using tc::desc_sw128;
+using tc::tma_load_2d;
 
 namespace {
 
@@ -45,22 +47,6 @@ constexpr int EPI_WARPS = 16;      // 4 per TMEM lane quadrant
 constexpr int GEMM_THREADS = 64 + 32 * EPI_WARPS;
 constexpr uint32_t POLLS = 1u << 26;
 constexpr int HEAD_TILE = 240;   // head columns per tile (a multiple of 16 and of 24)
-
-__device__ __forceinline__ uint64_t desc_sw128(uint32_t saddr) {
-    uint64_t d = 0;
-    d |= (uint64_t)((saddr >> 4) & 0x3FFFu);
-    d |= (uint64_t)1u << 16;            // leading byte offset: unused for swizzled K-major
-    d |= (uint64_t)(1024u >> 4) << 32;  // stride byte offset: 8 rows x 128 B
-    d |= (uint64_t)1u << 46;            // descriptor version
-    d |= (uint64_t)2u << 61;            // 128-byte swizzle
-    return d;
-}
-
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map, int x, int y, uint32_t mbar) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-        :: "r"(dst), "l"(map), "r"(x), "r"(y), "r"(mbar) : "memory");
-}
 
 // ---- CTA-pair (2-SM) forms: a pair computes a 256-row tile with one MMA stream issued
 // by the leader CTA (cluster rank 0); each CTA holds its 128 rows of A and half of the B
@@ -1762,6 +1748,7 @@ struct TcWs {
     int *dstep;      // [B] first step at which each episode is frozen
     // batched teacher-forced scoring
     __nv_bfloat16 *xall, *xall_lo;  // [(T+1) B, KX] the operand rows of every frame
+    int *rcount;                    // [row tiles] the one-launch recurrence's counters
     float *part;                    // [4 head tiles, T B] per-(step, sequence) partials
 };
 
@@ -1800,6 +1787,7 @@ TcWs carve_ws(const wm_handle *h, int B, void *ws, int T_teacher = -1) {
         const size_t rows = (size_t)(T_teacher + 1) * B;
         w.xall = (__nv_bfloat16 *)p; p += a256(rows * KX * 2);
         if (c.precision == WM_FP32) { w.xall_lo = (__nv_bfloat16 *)p; p += a256(rows * KX * 2); }
+        w.rcount = (int *)p; p += a256((size_t)(B / BM + 1) * 4);
         w.part = (float *)p;
     }
     return w;
@@ -1872,6 +1860,7 @@ size_t wm_tc_ws(const wm_handle *h, int B, int T_teacher) {
     const size_t KX = (size_t)h->tc.Zp + h->tc.Hp, H = h->tc.Hp;
     const size_t rows = T_teacher >= 0 ? (size_t)(T_teacher + 1) * B : 0;
     const size_t teach = T_teacher >= 0 ? (c.precision == WM_FP32 ? 2 : 1) * a256(rows * KX * 2) +
+                                              a256((size_t)(B / BM + 1) * 4) +
                                               a256((size_t)4 * h->tc.n_head_tiles * T_teacher * B * 4)
                                         : 0;
     return teach + 2 * a256((size_t)B * KX * 2) + 2 * a256((size_t)B * H * 4) + a256((size_t)B * 4) + 2 * a256(B) +
@@ -2114,7 +2103,37 @@ static cudaError_t tc_run(const wm_handle *h, int teacher, const wm_rollout_dev 
             ++launches;
         }
         io.x_cur = io.x_next = io.x_next_lo = nullptr;
-        for (int t = 0; t < Tn && e == cudaSuccess; ++t) {
+        wm_recur_args ra_{};
+        const int rmode = f32 ? 2 : acc ? 1 : 0;
+        const uint64_t frames = (uint64_t)(Tn + 1) * B;
+        const bool one = Tn > 1 && frames < (1u << 30) && wm_recur_plan(rmode, B, Hp, KX, &ra_);
+        if (one) {  // the whole recurrence in one launch
+            CUtensorMap xm, xlm, wmap, wlmap;
+            if (!make_map(&xm, w.xall, frames, KX, BM / ra_.cluster) || !make_map(&wmap, T.wg_n, 4 * Hp, KX, ra_.units))
+                return cudaErrorInvalidValue;
+            if (f32) {
+                if (!make_map(&xlm, w.xall_lo, frames, KX, BM / ra_.cluster) || !make_map(&wlmap, T.wg_n_lo, 4 * Hp, KX, ra_.units))
+                    return cudaErrorInvalidValue;
+            } else {
+                xlm = xm;
+                wlmap = wmap;
+            }
+            ra_.N = B; ra_.T = Tn; ra_.A = A; ra_.H = H; ra_.Zp = Zp; ra_.Hp = Hp; ra_.KX = KX;
+            ra_.act = na->actions;
+            ra_.x = w.xall; ra_.x_lo = w.xall_lo;
+            ra_.wa = (const __nv_bfloat16 *)T.wa_n; ra_.wa_lo = (const __nv_bfloat16 *)T.wa_n_lo;
+            ra_.bias = T.bg_n;
+            ra_.h_seq = na->h_seq; ra_.c_seq = na->c_seq;
+            ra_.count = w.rcount;
+            ra_.status = h->status;
+            ra_.test_wait = h->test_wait;  // an injected wait goes to the call's first GEMM
+            h->test_wait = 0;
+            if ((e = cudaMemsetAsync(w.rcount, 0, (size_t)ra_.m_tiles * 4, s)) != cudaSuccess) return e;
+            wm_ktime kt(h, WM_KERNEL_TC_GATES, s);
+            e = wm_recur_launch(rmode, &xm, &xlm, &wmap, &wlmap, ra_, s);
+            ++launches;
+        }
+        for (int t = 0; t < Tn && e == cudaSuccess && !one; ++t) {
             io.t = t;
             io.step = (uint32_t)t;
             // this step's operand rows (frame t) and where h' goes (frame t + 1)

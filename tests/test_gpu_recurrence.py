@@ -1,0 +1,81 @@
+"""The one-launch teacher-forced recurrence: row-tile edges (128), clusters and unit tiles of every
+hidden size it splits, several row tiles per CTA, rings shorter than a tile's operands, against the
+oracle; determinism; and the calls it leaves to one launch per step."""
+import numpy as np
+import pytest
+import torch
+
+import synth
+from parity import check_teacher, np_
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def wm():
+    import paper_2205_01435_gb300 as pkg
+    return pkg.load()
+
+
+def _cuda(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+# Z, A, H, K, N, T, precision (aligned sizes: the tensor family takes both precisions)
+CASES = [(8, 64, 64, 2, 300, 5, "bf16"), (64, 64, 64, 5, 1, 4, "fp32"), (24, 128, 320, 5, 129, 6, "bf16"),
+         (64, 256, 512, 5, 127, 3, "fp32"), (64, 256, 512, 5, 257, 4, "bf16"), (64, 256, 512, 5, 1000, 4, "bf16"),
+         (64, 256, 512, 5, 640, 3, "fp32"), (128, 512, 1024, 8, 256, 3, "bf16"), (128, 512, 1024, 8, 300, 2, "bf16"),
+         (32, 64, 256, 5, 2500, 3, "bf16"), (128, 512, 1024, 8, 40, 2, "fp32")]
+
+
+@pytest.mark.parametrize("Z,A,H,K,N,T,prec", CASES)
+def test_scoring_against_oracle(wm, orc, Z, A, H, K, N, T, prec):
+    cfg = dict(synth.model_config("nll"), z_dim=Z, a_dim=A, h_dim=H, k_mix=K, precision=prec)
+    w = synth.weights(cfg, seed=41)
+    zs, acts, lens = synth.teacher_inputs(N, T, Z, A, seed=41, ragged=True)
+    acts[1::2, ::5] = -1
+    m = wm.WorldModel(dict(cfg, path="tensor"), w)
+    args = (_cuda(zs), _cuda(acts))
+    g = m.mdn_nll(*args, lengths=_cuda(lens), want_seq=True)
+    m.sync()
+    idx = np.unique(np.linspace(0, N - 1, 24).round().astype(int))
+    o = orc.mdn_nll(cfg, w, zs[:, idx], acts[:, idx], lengths=lens[idx], want_seq=True)
+    check_teacher({k: np_(v)[idx] if k == "nll" else np_(v)[:, idx] for k, v in g.items()}, o, prec)
+    again = m.mdn_nll(*args, lengths=_cuda(lens), want_seq=True)
+    plain = m.mdn_nll(*args, lengths=_cuda(lens))  # the other outputs change nothing
+    for k in g:
+        assert torch.equal(g[k], again[k]), k
+    assert torch.equal(g["nll"], plain["nll"])
+    # a sequence's likelihood does not depend on the batch around it
+    one = m.mdn_nll(_cuda(zs[:, N - 1:]), _cuda(acts[:, N - 1:]), lengths=_cuda(lens[N - 1:]), want_seq=True)
+    assert torch.equal(one["h_seq"][:, 0], g["h_seq"][:, N - 1])
+
+
+def test_bad_action_on_the_device_is_reported(wm):
+    cfg = synth.model_config("nll")
+    m = wm.WorldModel(dict(cfg, path="tensor"), synth.weights(cfg))
+    zs, acts, _ = synth.teacher_inputs(200, 4, 64, 256, seed=42)
+    acts[2, 150] = 256
+    m.mdn_nll(_cuda(zs), _cuda(acts))
+    with pytest.raises(wm.WMError) as e:
+        m.sync()
+    assert e.value.status == wm.WM_ERR_INVALID_ARG
+
+
+def test_under_stream_capture(wm):
+    """A captured call replays to the same bits."""
+    cfg = synth.model_config("nll")
+    m = wm.WorldModel(dict(cfg, path="tensor"), synth.weights(cfg))
+    zs, acts, _ = synth.teacher_inputs(300, 6, 64, 256, seed=43)
+    z, a = _cuda(zs), _cuda(acts)
+    want = m.mdn_nll(z, a, want_seq=True)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        got = m.mdn_nll(z, a, want_seq=True)
+    for k in got:
+        got[k].zero_()
+    g.replay()
+    torch.cuda.synchronize()
+    for k in want:
+        assert torch.equal(want[k], got[k]), k
