@@ -1108,7 +1108,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
         bar_never;
     __shared__ uint32_t tmem_base;
     __shared__ int s_abort;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const uint32_t rank = tc::cluster_rank();  // 0: the pair's leader
     const int pair = (int)(blockIdx.x >> 1), npairs = (int)(gridDim.x >> 1);
     const uint32_t smem_u = tc::smem_u32(smem);
@@ -1152,28 +1152,40 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
         __syncthreads();
         if (s_abort) ntiles = 0;
     }
-    auto wait = [&](uint32_t bar, uint32_t parity) {
-        if (!s_abort && !tc::mbar_wait_bounded(bar, parity, POLLS)) {
-            s_abort = 1;
-            atomicExch(g.status, (int)WM_ERR_TIMEOUT);
+    // Waits: one try in line (the usual case), then polls that also watch for another warp's giving
+    // up.  False once anybody gave up.
+    auto wait_slow = [&](uint32_t bar, uint32_t parity) {
+        for (uint32_t i = 0; i < POLLS; ++i) {
+            if (tc::mbar_try_wait(bar, parity)) return true;
+            if (*(volatile int *)&s_abort) return false;
         }
+        s_abort = 1;
+        atomicExch(g.status, (int)WM_ERR_TIMEOUT);
+        return false;
     };
+    auto wait = [&](uint32_t bar, uint32_t parity) { return tc::mbar_try_wait(bar, parity) || wait_slow(bar, parity); };
 
-    if (warp == 0) {
-        if (lane == 0) {  // ---- TMA producer (both CTAs)
-            int stage = 0;
-            uint32_t phase = 0;
-            for (int tile = pair; tile < ntiles; tile += npairs) {
-                const int m = tile / g.n_tiles, n = tile % g.n_tiles;
-                const int brow = g.pop_P > 1 ? (int)(((g.ep0 + (unsigned long long)m * (2 * BM)) /
-                                                      (unsigned long long)g.pop_E) % (unsigned long long)g.pop_P) * g.pop_rows
-                                             : 0;
-                for (int ks0 = 0; ks0 < ksteps; ks0 += KPS) {
-                    const int nk = ksteps - ks0 < KPS ? ksteps - ks0 : KPS;  // k-steps in this stage
+    // The producer's and the issuer's warps run their loops as a whole and issue from one elected lane
+    // (see tc::elect_one): as `if (lane == 0)` loops a stage's turn cost several hundred cycles.
+    if (warp == 0) {  // ---- TMA producer (both CTAs)
+        int stage = 0;
+        uint32_t phase = 0;
+        bool go = true;
+        for (int tile = pair; tile < ntiles && go; tile += npairs) {
+            const int m = tile / g.n_tiles, n = tile % g.n_tiles;
+            const int brow = g.pop_P > 1 ? (int)(((g.ep0 + (unsigned long long)m * (2 * BM)) /
+                                                  (unsigned long long)g.pop_E) % (unsigned long long)g.pop_P) * g.pop_rows
+                                         : 0;
+            for (int ks0 = 0; ks0 < ksteps; ks0 += KPS) {
+                const int nk = ksteps - ks0 < KPS ? ksteps - ks0 : KPS;  // k-steps in this stage
+                // the stage's previous MMAs are done
+                if (!(go = __all_sync(0xffffffffu, wait(empty_b(stage), phase ^ 1u)))) break;
+                if (tc::elect_one()) {
                     const uint32_t full_ldr = tc::map_rank(full_b(stage), 0);
-                    wait(empty_b(stage), phase ^ 1u);  // the stage's previous MMAs are done
-                    if (s_abort) break;
-                    for (int h = 0; h < nk; ++h) {
+                    if (rank == 0) tc::mbar_arrive_expect_tx(full_b(stage), 2 * nk * KSTEP_BYTES);
+#pragma unroll
+                    for (int h = 0; h < KPS; ++h) {
+                        if (h >= nk) break;
                         int ks = ks0 + h;
                         const CUtensorMap *ma = &tmA, *mb = &tmB;
                         if (NP > 1) {  // pass 0: A_hi B_hi, 1: A_hi B_lo, 2: A_lo B_hi
@@ -1183,52 +1195,51 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
                             if (pass == 2) ma = &tmA2;
                         }
                         const uint32_t sa = smem_u + stage * STAGE_BYTES + h * KSTEP_BYTES;
-                        if (h == 0 && rank == 0) tc::mbar_arrive_expect_tx(full_b(stage), 2 * nk * KSTEP_BYTES);
                         tma_load_2sm(sa, ma, g.a_col0 + ks * BK, (2 * m + (int)rank) * BM, full_ldr);
 #pragma unroll
                         for (int s = 0; s < NSUB; ++s)
                             tma_load_2sm(sa + A_BYTES + s * B_SUB, mb, ks * BK,
                                          brow + n * TILE_N + s * BN + (int)rank * BNH, full_ldr);
                     }
-                    if (s_abort) break;
-                    if (++stage == STAGES) { stage = 0; phase ^= 1u; }
                 }
+                if (++stage == STAGES) { stage = 0; phase ^= 1u; }
             }
         }
     } else if (warp == 1) {
-        if (lane == 0 && rank == 0) {  // ---- MMA issuer (the leader only)
+        if (rank == 0) {  // ---- MMA issuer (the leader only)
             int stage = 0, acc = 0;
             uint32_t phase = 0, acc_phase = 0;
+            bool go = true;
             const uint32_t idesc = tc::idesc_bf16_f32(2 * BM, BN);
             for (int tile = pair; tile < ntiles; tile += npairs) {
-                wait(tc::smem_u32(&bar_acce[acc]), acc_phase ^ 1u);
+                go = go && __all_sync(0xffffffffu, wait(tc::smem_u32(&bar_acce[acc]), acc_phase ^ 1u));
                 tc::fence_after_sync();
                 const uint32_t dcol = tm + acc * ACC_COLS;
-                for (int ks0 = 0; ks0 < ksteps; ks0 += KPS) {
+                for (int ks0 = 0; go && ks0 < ksteps; ks0 += KPS) {
                     const int nk = ksteps - ks0 < KPS ? ksteps - ks0 : KPS;
-                    wait(full_b(stage), phase);
-                    if (s_abort) break;
+                    if (!(go = __all_sync(0xffffffffu, wait(full_b(stage), phase)))) break;
                     tc::fence_after_sync();
-                    // the issuing thread shares its SMSP with four epilogue warps: few instructions
-                    // between MMAs (descriptors built once per k-step, stepped by 32 bytes = 2)
+                    if (tc::elect_one()) {
 #pragma unroll
-                    for (int h = 0; h < KPS; ++h) {
-                        if (h >= nk) break;
-                        const int ks = ks0 + h;
-                        const uint32_t sa = smem_u + stage * STAGE_BYTES + h * KSTEP_BYTES;
-                        const uint64_t da0 = desc_sw128(sa), db0 = desc_sw128(sa + A_BYTES);
+                        for (int h = 0; h < KPS; ++h) {
+                            if (h >= nk) break;
+                            const int ks = ks0 + h;
+                            const uint32_t sa = smem_u + stage * STAGE_BYTES + h * KSTEP_BYTES;
+                            const uint64_t da0 = desc_sw128(sa), db0 = desc_sw128(sa + A_BYTES);
 #pragma unroll
-                        for (int kk = 0; kk < BK / 16; ++kk) {
+                            for (int kk = 0; kk < BK / 16; ++kk) {
 #pragma unroll
-                            for (int s = 0; s < NSUB; ++s)
-                                mma_bf16_pair(dcol + s * BN, da0 + 2 * kk, db0 + (s * B_SUB >> 4) + 2 * kk, idesc,
-                                              (ks > 0 || kk > 0) ? 1u : 0u);
+                                for (int s = 0; s < NSUB; ++s)
+                                    mma_bf16_pair(dcol + s * BN, da0 + 2 * kk, db0 + (s * B_SUB >> 4) + 2 * kk, idesc,
+                                                  (ks > 0 || kk > 0) ? 1u : 0u);
+                            }
                         }
+                        mma_commit_pair(empty_b(stage));  // both CTAs' stage is free once these are done
                     }
-                    mma_commit_pair(empty_b(stage));  // both CTAs' stage is free once these are done
                     if (++stage == STAGES) { stage = 0; phase ^= 1u; }
                 }
-                mma_commit_pair(tc::smem_u32(&bar_accf[acc]));
+                // (also after giving up: both CTAs' epilogues go on to their ends)
+                if (tc::elect_one()) mma_commit_pair(tc::smem_u32(&bar_accf[acc]));
                 if (NACC == 2) {
                     acc ^= 1;
                     if (acc == 0) acc_phase ^= 1u;
