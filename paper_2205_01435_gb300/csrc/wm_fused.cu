@@ -189,14 +189,14 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_fused(FusedParams p) {
     __shared__ float s_done_logit[TILE];
 
     const Geo g = geometry<S>(p.Z, p.A, p.H);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const bool mma_warp = warp == MMA_WARP;
     const int row = 32 * (warp & 3) + lane, grp = mma_warp ? 0 : warp >> 2;
     const uint32_t rank = tc::cluster_rank();
     const int tile = blockIdx.x / CL;
     const int b = tile * TILE + row;
     const bool live = b < p.B && !mma_warp;
-    const int Z = p.Z, H = p.H, A = p.A, K1 = Z + H, KZ = KM * Z;
+    const int Z = p.Z, H = p.H, A = p.A, KZ = KM * Z;
     const int W = (A + 31) >> 5;
     const int u0 = UG * grp;               // first owned unit (within this rank)
     const int dim = (int)rank * ZD + grp;  // owned latent dim (groups < ZD)
@@ -276,15 +276,20 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_fused(FusedParams p) {
     // descriptor start addresses advance by 2 core matrices along K: 2*lbo bytes (>> 4)
     const uint64_t dX0 = tc::smem_desc(x_u32, lboX, 128), dW10 = tc::smem_desc(w1_u32, lbo1, 128);
     const uint64_t dW20 = tc::smem_desc(buf_u32, lbo2, 128);
-    // MMA1 over k-blocks [kb0, kb1) of 16: z part is [0, Z/16), h part [Z/16, K1/16).
+    // MMA1 over k-blocks of 16: z part is [0, ZB), h part [ZB, ZB + HB).
     // Every step accumulates the h part first, then the z part.
-    auto mma1 = [&](int kb0, int kb1, bool acc_first) {
-        uint64_t da = dX0 + (uint64_t)kb0 * (2 * lboX >> 4), db = dW10 + (uint64_t)kb0 * (2 * lbo1 >> 4);
-        for (int kb = kb0; kb < kb1; ++kb) {
-            tc::mma_bf16(tm, da, db, idesc1, (kb > kb0 || acc_first) ? 1u : 0u);
-            da += 2 * lboX >> 4;
-            db += 2 * lbo1 >> 4;
-        }
+    // The block counts are compile-time (Z = CL ZD, H = CL U) and the MMA warp runs as a whole and
+    // issues from an elected lane (see tc::elect_one), the MMAs unrolled.
+    constexpr int ZB = CL * ZD / 16, HB = CL * S::U / 16;
+    auto mma1_z = [&](bool acc) {
+#pragma unroll
+        for (int kb = 0; kb < ZB; ++kb)
+            tc::mma_bf16(tm, dX0 + kb * (2 * lboX >> 4), dW10 + kb * (2 * lbo1 >> 4), idesc1, (kb > 0 || acc) ? 1u : 0u);
+    };
+    auto mma1_h = [&] {
+#pragma unroll
+        for (int kb = ZB; kb < ZB + HB; ++kb)
+            tc::mma_bf16(tm, dX0 + kb * (2 * lboX >> 4), dW10 + kb * (2 * lbo1 >> 4), idesc1, kb > ZB ? 1u : 0u);
     };
     // bounded waits: wait_one by a single thread, wait_bar by whole warps
     auto wait_one = [&](uint32_t bar, uint32_t parity) {
@@ -297,8 +302,6 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_fused(FusedParams p) {
         wait_one(bar, parity);
         __syncwarp();
     };
-    const bool issuer = mma_warp && lane == 0;
-
     float nll_acc = 0.f;
     const int len_in = p.teacher && p.lengths ? p.lengths[live ? b : 0] : p.T;
     if (live && (len_in < 0 || len_in > p.T)) report_status(p.status, WM_ERR_INVALID_ARG);
@@ -329,11 +332,13 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_fused(FusedParams p) {
         if (s_abort) t_end = 0;
     }
 
-    if (issuer && t_end > 0) {  // MMA1 of step 0
+    if (mma_warp && t_end > 0) {  // MMA1 of step 0
         tc::fence_after_sync();
-        mma1(Z / 16, K1 / 16, false);
-        mma1(0, Z / 16, true);
-        tc::mma_commit(MB_MMA1);
+        if (tc::elect_one()) {
+            mma1_h();
+            mma1_z(true);
+            tc::mma_commit(MB_MMA1);
+        }
     }
     __syncwarp();  // the MMA warp reconverges before the next aligned barrier
 
@@ -491,25 +496,28 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_fused(FusedParams p) {
         }
 
         // ---------------- MMA2: heads (a5); then the h part of the next MMA1 ---
-        if (issuer) {
-            wait_one(MB_H, parity);  // h' of every rank is in X
-            wait_one(MB_W2, parity);  // W2 is in the buffer
-            if (!s_abort) {
+        if (mma_warp) {
+            wait_bar(MB_H, parity);   // h' of every rank is in X
+            wait_bar(MB_W2, parity);  // W2 is in the buffer
+            if (__all_sync(0xffffffffu, !s_abort)) {
                 tc::fence_after_sync();
-                uint64_t da = dX0 + ((uint64_t)Z * 256u >> 4), db = dW20;  // X_h: Z/8 k-blocks in
-                for (int kb = 0; kb < H / 16; ++kb) {
-                    tc::mma_bf16(tm + D2_COL, da, db, idesc2, kb > 0);
-                    da += 2 * lboX >> 4;
-                    db += 2 * lbo2 >> 4;
+                if (tc::elect_one()) {
+#pragma unroll
+                    for (int kb = 0; kb < HB; ++kb)  // X_h: ZB k-blocks in
+                        tc::mma_bf16(tm + D2_COL, dX0 + (ZB + kb) * (2 * lboX >> 4), dW20 + kb * (2 * lbo2 >> 4), idesc2,
+                                     kb > 0);
+                    tc::mma_commit(MB_MMA2);
+                    // same issuing thread: runs after MMA2 and overlaps the sampling
+                    if (!last) mma1_h();
                 }
-                tc::mma_commit(MB_MMA2);
-                // same issuing thread: runs after MMA2 and overlaps the sampling
-                if (!last) mma1(Z / 16, K1 / 16, false);
             }
+            __syncwarp();
             if (!last) {  // W_a back into the buffer once MMA2 has read W2
-                wait_one(MB_MMA2, parity);
-                tc::mbar_arrive_expect_tx(MB_W, WA_BYTES);
-                tc::bulk_load_global(buf_u32, img + g.iwa, WA_BYTES, MB_W);
+                wait_bar(MB_MMA2, parity);
+                if (tc::elect_one()) {
+                    tc::mbar_arrive_expect_tx(MB_W, WA_BYTES);
+                    tc::bulk_load_global(buf_u32, img + g.iwa, WA_BYTES, MB_W);
+                }
             }
         }
         __syncwarp();
@@ -654,10 +662,12 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_fused(FusedParams p) {
             tc::fence_proxy_async_smem();
             tc::fence_before_sync();
             __syncthreads();
-            if (issuer && !s_abort) {
+            if (mma_warp && __all_sync(0xffffffffu, !s_abort)) {
                 tc::fence_after_sync();
-                mma1(0, Z / 16, true);  // accumulate onto the h part issued after MMA2
-                tc::mma_commit(MB_MMA1);
+                if (tc::elect_one()) {
+                    mma1_z(true);  // accumulate onto the h part issued after MMA2
+                    tc::mma_commit(MB_MMA1);
+                }
             }
             __syncwarp();
             if (!p.teacher && !mma_warp) {  // freezing (a8)
