@@ -155,14 +155,13 @@ __device__ __forceinline__ void x_store8(unsigned char *sx, int r, int k, const 
 }
 
 // Push this CTA's block at shared address `src` (same offset in every CTA) to the
-// other CTAs of the cluster; lane 0 of warp w < nwarps serves peers w, w + nwarps, ...
+// other CTAs of the cluster; warp w serves peer w (whole warps call it, one lane issues).
 template <int CL>
 __device__ __forceinline__ void push_to_peers(uint32_t src, uint32_t bytes, uint32_t mbar, uint32_t rank,
-                                              int warp, int lane, int nwarps) {
-    if (lane == 0 && warp < nwarps)
-        for (int q = warp; q < CL; q += nwarps)
-            if ((uint32_t)q != rank)
-                tc::bulk_copy_to_peer(tc::map_rank(src, q), src, bytes, tc::map_rank(mbar, q));
+                                              int warp) {
+    static_assert(CL <= NT / 32, "a peer per warp");
+    if (warp < CL && (uint32_t)warp != rank && tc::elect_one())
+        tc::bulk_copy_to_peer(tc::map_rank(src, warp), src, bytes, tc::map_rank(mbar, warp));
 }
 
 // barrier over the 16 compute warps (the MMA warp may still be issuing)
@@ -388,7 +387,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_fused(FusedParams p) {
         tc::fence_proxy_async_smem();
         tc::fence_before_sync();
         __syncthreads();
-        push_to_peers<CL>(part_u32 + rank * PART_BYTES, PART_BYTES, MB_PART, rank, warp, lane, NT / 32);
+        push_to_peers<CL>(part_u32 + rank * PART_BYTES, PART_BYTES, MB_PART, rank, warp);
         float hn[UG];
         int a = -1;
         if (!mma_warp) {
@@ -460,7 +459,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_fused(FusedParams p) {
         tc::fence_proxy_async_smem();
         __syncthreads();  // every W_a read and h' write of this CTA is done
         const uint32_t hblk = x_u32 + tc::kmajor_offset(0, Z + rank * S::U, TILE);
-        push_to_peers<CL>(hblk, H_BYTES, MB_H, rank, warp, lane, NT / 32);
+        push_to_peers<CL>(hblk, H_BYTES, MB_H, rank, warp);
         // W2 replaces W_a in the buffer while h' travels.  The compute threads copy it (L2 ->
         // registers -> shared memory): the TMA engine, which moves every exchange, is left to
         // the h' slices (with W2 in its queue too, MMA2 waited for both).
@@ -605,7 +604,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_fused(FusedParams p) {
         tc::fence_before_sync();
         sync_compute_warps();  // z' staged, done logit published
         if (!last && !p.teacher)
-            push_to_peers<CL>(zst_u32 + rank * Z_BYTES, Z_BYTES, MB_Z, rank, warp, lane, NT / 32);
+            push_to_peers<CL>(zst_u32 + rank * Z_BYTES, Z_BYTES, MB_Z, rank, warp);
         const float dl = s_done_logit[row];
         // outputs of this step (overlap the exchange)
         if (live) {
