@@ -264,20 +264,37 @@ cudaError_t pack_step(wm_handle *h, const wm_weights *w) {
 // 2x even at B = 16).  The bf16 calls left over (sizes that are no multiple of the tiles', and
 // batches below 256) take the tensor family with padded sizes and accurate nonlinearities:
 // rollouts of 20 steps at Z, A, H, K = 50, 101, 300, 6 take 581 / 627 / 700 / 1274 us at B = 1 /
-// 600 / 2000 / 8000 against 1791 / 2615 / 3819 / 12135 us stepwise, at 128, 512, 1024, 8 and
-// B = 64 1017 against 6616 us, so no size is left to the stepwise family; it keeps fp32 models
-// of such sizes (its fp32 sums are more accurate than three bf16 products), K > 8, A > 512 and
-// populations that do not fill row tiles.  fused_ok / tc_ok: whether this call's options allow
-// those families.
-int pick_path(const wm_handle *h, int B, bool fused_ok = true, bool tc_ok = true) {
+// 600 / 2000 / 8000 against 1791 / 2615 / 3819 / 12135 us stepwise, at 64, 256, 512, 8 and B = 64
+// 722 against 3378 us.  Left to the stepwise family: fp32 models of such sizes (its fp32 sums are
+// more accurate than three bf16 products), K > 8, A > 512, populations that do not fill row tiles,
+// and rollouts of more than 4 steps with H > 512: there a trajectory is chaotic, so that the sums'
+// order alone moves it by 5 to 10% within 25 steps (rel. 2-norm of z, rewards, h; 1% at 4 steps,
+// and under 1% at H <= 512), and a small batch's results stay what they were.  fused_ok / tc_ok:
+// whether this call's options allow those families; steps: of a rollout (0: a scoring call).
+int pick_path(const wm_handle *h, int B, bool fused_ok = true, bool tc_ok = true, int steps = 0) {
     const int p = h->cfg.path;
     if (p != WM_PATH_AUTO) return p;
     const bool fu = fused_ok && wm_fused_supported(h, B), tc = tc_ok && wm_tc_supported(h);
     if (fu && B <= 2048) return WM_PATH_FUSED;
     if (tc && (B >= 256 || h->cfg.precision == WM_FP32)) return WM_PATH_TENSOR;
     if (fu) return WM_PATH_FUSED;
-    if (tc_ok && wm_tc_auto_ok(h)) return WM_PATH_TENSOR;
+    if (tc_ok && wm_tc_auto_ok(h) && (h->cfg.h_dim <= 512 || steps <= 4)) return WM_PATH_TENSOR;
     return WM_PATH_STEPWISE;
+}
+
+// Scoring (and the training step's forward): AUTO takes the tensor family for a bf16 model whenever its
+// recurrence runs as one launch, also where a member of the fused family would take the call, unless
+// that is short.  Measured (us, fused against tensor) at Z, A, H, K = 32, 64, 256, 5: 16 x 4 steps 40 / 44,
+// x 24 183 / 110, x 100 723 / 407, 1500 x 24 264 / 166; at 7, 45, 40, 3: 16 x 4 27 / 36, x 24 121 / 96;
+// at 85, 168, 94, 7: 271 x 24 1087 / 139.  The crossing lies between 6 and 10 steps.  In a training
+// step of the smallest models and batches the fused member's outputs cost less: 100 x 24 at 7, 45, 40, 3
+// 384 / 392, 600 x 24 732 / 475.
+int pick_score_path(const wm_handle *h, int N, int T, bool train) {
+    if (h->cfg.path == WM_PATH_AUTO && wm_tc_auto_ok(h) && wm_tc_scores_in_one(h, N, T)) {
+        const bool kept = T < 12 || (train && h->cfg.h_dim < 64 && N <= 400);
+        if (!(kept && wm_fused_supported(h, N))) return WM_PATH_TENSOR;
+    }
+    return pick_path(h, N);
 }
 
 template <class T>
@@ -536,7 +553,7 @@ wm_status wm_rollout(wm_handle *h, int B, int T, unsigned long long episode_offs
     // family needs a population's candidates aligned to its 256-row tiles
     const bool fused_ok = !io->logp_seq && !(c.value_head && io->value_seq) && h->P == 1 && c.n_xfers == 0;
     const bool tc_ok = wm_tc_call_ok(h, episode_offset) != 0;
-    int path = pick_path(h, B, fused_ok, tc_ok);
+    int path = pick_path(h, B, fused_ok, tc_ok, T);
     if (path == WM_PATH_FUSED && !(fused_ok && wm_fused_supported(h, B)))
         return fail(h, WM_ERR_UNSUPPORTED, "the fused family does not take this model / batch / outputs");
     if (c.path == WM_PATH_TENSOR && !(tc_ok && wm_tc_supported(h)))
@@ -675,7 +692,7 @@ wm_status wm_mdn_nll_backward(wm_handle *h, int N, int T, const float *z_seq, co
     st.add((void **)&g.b_mdn, grads->b_mdn, M * 4, true);
 
     // the forward: the teacher-forced pass, keeping h, c and the head outputs of every row
-    const int path = pick_path(h, N);
+    const int path = pick_score_path(h, N, T, true);
     if (path == WM_PATH_FUSED && !wm_fused_supported(h, N))
         return fail(h, WM_ERR_UNSUPPORTED, "the fused family does not take this model / batch");
     if (c.path == WM_PATH_TENSOR && !wm_tc_supported(h))
@@ -743,7 +760,7 @@ wm_status wm_mdn_nll(wm_handle *h, int N, int T, const float *z_seq, const int32
     st.add((void **)&a.c_seq, c_seq, t * n * H * 4, true);
     st.add((void **)&a.mdn_seq, mdn_seq, t * n * M * 4, true);
 
-    int path = pick_path(h, N);
+    int path = pick_score_path(h, N, T, false);
     if (path == WM_PATH_FUSED && !wm_fused_supported(h, N))
         return fail(h, WM_ERR_UNSUPPORTED, "the fused family does not take this model / batch");
     if (c.path == WM_PATH_TENSOR && !wm_tc_supported(h))

@@ -194,6 +194,7 @@ class wm_ktime {
 // ---- tensor-core family (wm_tensor.cu) ----------------------------------------
 int wm_tc_supported(const wm_handle *h);  // the model's sizes are multiples of the tiles'
 int wm_tc_auto_ok(const wm_handle *h);    // a bf16 model it runs with its sizes padded
+bool wm_tc_scores_in_one(const wm_handle *h, int N, int T);  // a scoring call's recurrence is one launch
 // workspace of a call of B rows; T_teacher >= 0: teacher-forced scoring of T_teacher steps
 // (its operand rows of all T_teacher + 1 frames), -1: a rollout
 size_t wm_tc_ws(const wm_handle *h, int B, int T_teacher = -1);

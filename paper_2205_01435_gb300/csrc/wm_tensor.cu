@@ -1318,26 +1318,26 @@ __global__ void k_tc_init(StepIO p, const float *z0, const float *h0, const floa
                           int n_head_tiles, int *dstep, int *cnt) {
     if (cnt && blockIdx.x == 0 && threadIdx.x < 4) cnt[threadIdx.x] = 0;
     const int Zp = p.Zp, Hp = p.Hp, KX = Zp + Hp;
-    for (size_t b = blockIdx.x; b < (size_t)p.B; b += gridDim.x) {  // a block per row: no divisions
-        for (int k = threadIdx.x; k < KX; k += blockDim.x) {
-            const size_t i = b * KX + k;
-            const int u = k - Zp;  // hidden unit (k >= Zp)
-            const bool is_z = k < p.Z, is_h = u >= 0 && u < p.H;
-            float v = 0.f;  // the padded columns are 0
-            if (is_z) v = p.teacher ? p.z_seq[b * p.Z + k] : z0[b * p.Z + k];
-            else if (is_h && h0) v = h0[b * p.H + u];
-            const __nv_bfloat16 vh = __float2bfloat16_rn(v);
-            x0[i] = vh;
-            if (x0_lo) x0_lo[i] = __float2bfloat16_rn(v - __bfloat162float(vh));
-            // the other operand buffer's padded z columns, which no epilogue writes
-            if (x1 && k >= p.Z && k < Zp) x1[i] = vh;
-            if (u >= 0) {
-                const size_t j = b * Hp + u;
-                p.h32[j] = v;
-                p.c[j] = c0 && is_h ? c0[b * p.H + u] : 0.f;
-            } else if (is_z && !p.teacher) {
-                p.z_out[b * p.Z + k] = v;
-            }
+    const size_t nx = (size_t)p.B * KX;
+    const bool small = nx < 0xFFFFFFFFull;  // (a 32-bit division is a quarter of a 64-bit one)
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < nx; i += (size_t)gridDim.x * blockDim.x) {
+        const size_t b = small ? (uint32_t)i / (uint32_t)KX : i / KX;
+        const int k = (int)(i - b * KX), u = k - Zp;  // operand column; hidden unit (k >= Zp)
+        const bool is_z = k < p.Z, is_h = u >= 0 && u < p.H;
+        float v = 0.f;  // the padded columns are 0
+        if (is_z) v = p.teacher ? p.z_seq[b * p.Z + k] : z0[b * p.Z + k];
+        else if (is_h && h0) v = h0[b * p.H + u];
+        const __nv_bfloat16 vh = __float2bfloat16_rn(v);
+        x0[i] = vh;
+        if (x0_lo) x0_lo[i] = __float2bfloat16_rn(v - __bfloat162float(vh));
+        // the other operand buffer's padded z columns, which no epilogue writes
+        if (x1 && k >= p.Z && k < Zp) x1[i] = vh;
+        if (u >= 0) {
+            const size_t j = b * Hp + u;
+            p.h32[j] = v;
+            p.c[j] = c0 && is_h ? c0[b * p.H + u] : 0.f;
+        } else if (is_z && !p.teacher) {
+            p.z_out[b * p.Z + k] = v;
         }
     }
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < (size_t)p.B; i += (size_t)gridDim.x * blockDim.x) {
@@ -1990,6 +1990,27 @@ void wm_tc_free(wm_handle *h) {
     memset(&T, 0, sizeof(T));
 }
 
+// The calls that AUTO would give to a SIMT family (stepwise, the fused family's small-batch member)
+// if this one took aligned sizes and B >= 256 only keep those families' accurate nonlinearities.
+static bool accurate(const wm_handle *h, int B, int teacher) {
+    if (h->cfg.precision != WM_BF16) return false;
+    return !h->tc.aligned ||
+           (h->cfg.path == WM_PATH_AUTO && (B < 256 || (teacher && wm_small_supported(h, B))));
+}
+
+// How a scoring call's recurrence runs as one launch; false: one launch per step.
+static bool one_launch(const wm_handle *h, int N, int T, wm_recur_args *a, int *mode) {
+    const wm_tc_weights &w = h->tc;
+    *mode = h->cfg.precision == WM_FP32 ? 2 : accurate(h, N, 1) ? 1 : 0;
+    return T > 1 && (uint64_t)(T + 1) * N < (1u << 30) && wm_recur_plan(*mode, N, w.Hp, w.Zp + w.Hp, a);
+}
+
+bool wm_tc_scores_in_one(const wm_handle *h, int N, int T) {
+    wm_recur_args a{};
+    int mode;
+    return h->tc.ok && N > 0 && one_launch(h, N, T, &a, &mode);
+}
+
 // One call: rollout (teacher = 0) or teacher-forced scoring (teacher = 1).
 static cudaError_t tc_run(const wm_handle *h, int teacher, const wm_rollout_dev *ra, const wm_nll_dev *na,
                           void *ws, cudaStream_t s) {
@@ -2066,9 +2087,7 @@ static cudaError_t tc_run(const wm_handle *h, int teacher, const wm_rollout_dev 
         if (he != cudaSuccess) return he;
     }
     const bool f32 = c.precision == WM_FP32;  // the split path: second operand maps and lo outputs
-    // The calls that AUTO would give to the stepwise family if this one took aligned sizes and
-    // B >= 256 only (padded sizes, small bf16 batches) keep that family's accurate nonlinearities.
-    const bool acc = !f32 && (!T.aligned || (c.path == WM_PATH_AUTO && B < 256));
+    const bool acc = accurate(h, B, teacher);
     CUtensorMap mx[2], mxs[2], mwc, mwg, mwh, mc, mc2, mxl[2], mxsl[2], mwcl, mwgl, mwhl;
     // B-operand boxes are half an instantiated BN (each CTA of a pair loads half the rows;
     // rows past A read as zero)
@@ -2115,9 +2134,9 @@ static cudaError_t tc_run(const wm_handle *h, int teacher, const wm_rollout_dev 
         }
         io.x_cur = io.x_next = io.x_next_lo = nullptr;
         wm_recur_args ra_{};
-        const int rmode = f32 ? 2 : acc ? 1 : 0;
+        int rmode = 0;
         const uint64_t frames = (uint64_t)(Tn + 1) * B;
-        const bool one = Tn > 1 && frames < (1u << 30) && wm_recur_plan(rmode, B, Hp, KX, &ra_);
+        const bool one = one_launch(h, B, Tn, &ra_, &rmode);
         if (one) {  // the whole recurrence in one launch
             CUtensorMap xm, xlm, wmap, wlmap;
             if (!make_map(&xm, w.xall, frames, KX, BM / ra_.cluster) || !make_map(&wmap, T.wg_n, 4 * Hp, KX, ra_.units))
