@@ -705,10 +705,16 @@ wm_status wm_mdn_nll_backward(wm_handle *h, int N, int T, const float *z_seq, co
     if ((e = st.begin(h, T, false, s)) != cudaSuccess) return cuda_fail(h, e, "staging inputs");
     wm_nll_dev a{};
     a.N = N; a.T = T; a.z_seq = zs; a.actions = ac; a.lengths = ln;
-    float *nll_ws;
     void *tail;
-    wm_bw_carve(h, N, T, h->bws, &a.h_seq, &a.c_seq, &a.mdn_seq, &nll_ws, &tail);
-    a.nll = nl ? nl : nll_ws;
+    wm_bw_fwd f{};
+    wm_bw_carve(h, N, T, h->bws, &f, &tail);
+    a.h_seq = f.hs; a.c_seq = f.cs; a.mdn_seq = f.md;
+    a.nll = nl ? nl : f.nll;
+    if (path == WM_PATH_TENSOR && N > 0 && T > 0) {
+        f.have_g = wm_tc_scores_in_one(h, N, T) && wm_bw_takes_gates(h, N, T);
+        if (f.have_g) a.g_seq = f.G;
+        if (c.precision == WM_BF16) f.frames = wm_tc_frames(h, N, T, h->ws, &f.ld, &f.h_col);
+    }
     int fwd_launches = 0;
     if (N > 0 && T > 0) {
         if (path == WM_PATH_FUSED) e = wm_fused_nll(h, a, h->ws, s);
@@ -721,7 +727,7 @@ wm_status wm_mdn_nll_backward(wm_handle *h, int N, int T, const float *z_seq, co
     }
     h->last_path = path;
     h->last_launches = fwd_launches;
-    e = wm_bw_launch(h, N, T, zs, ac, ln, g, a.h_seq, a.c_seq, a.mdn_seq, tail, s);
+    e = wm_bw_launch(h, N, T, zs, ac, ln, g, f, tail, s);
     if (e != cudaSuccess) return cuda_fail(h, e, "training-step backward");
     if ((e = st.end(s)) != cudaSuccess) return cuda_fail(h, e, "staging outputs");
     return WM_OK;

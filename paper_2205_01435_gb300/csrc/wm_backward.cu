@@ -23,6 +23,7 @@
 // over the operands' hi and lo parts, see k_bw_split3); the rest are the kernels below.
 // Every reduction has a fixed order, so results are bit-reproducible.
 #include <cublas_v2.h>
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <math.h>
 
@@ -131,10 +132,9 @@ __global__ void k_bw_mdn(int N, int TT, int Z, int K, const float *__restrict__ 
 // The cell's backward step at t for N rows: dh = dY_t + dH (from step t + 1), and
 //   dc = dh o (1 - tanh^2 c_t) + dc_carried;  dG = [dc g i(1-i) | dc c_{t-1} f(1-f) |
 //   dc i (1-g^2) | dh tanh(c_t) o(1-o)];  dc_carried <- dc f.
-template <class T>
 __global__ void k_bw_cell(int N, int H, int t, int first, const float *__restrict__ act, const float *__restrict__ cs,
                           const float *__restrict__ dY, const float *__restrict__ dH, float *__restrict__ dC,
-                          float *__restrict__ dG, T *__restrict__ dG_op, __nv_bfloat16 *__restrict__ dG3) {
+                          float *__restrict__ dG, __nv_bfloat16 *__restrict__ dG_op, __nv_bfloat16 *__restrict__ dG3) {
     const size_t base = (size_t)t * N;
     const int u = blockIdx.x * blockDim.x + threadIdx.x;  // unit; rows n over the grid's y
     if (u >= H) return;
@@ -150,9 +150,12 @@ __global__ void k_bw_cell(int N, int H, int t, int first, const float *__restric
         const float g0 = dc * gg * ig * (1.f - ig), g1 = dc * cp * fg * (1.f - fg);
         const float g2 = dc * ig * (1.f - gg * gg), g3 = dh * tc * og * (1.f - og);
         float *o = dG + r * 4 * H;
-        T *oo = dG_op + r * 4 * H;
         o[u] = g0; o[H + u] = g1; o[2 * H + u] = g2; o[3 * H + u] = g3;
-        oo[u] = to_op<T>(g0); oo[H + u] = to_op<T>(g1); oo[2 * H + u] = to_op<T>(g2); oo[3 * H + u] = to_op<T>(g3);
+        if (dG_op) {  // bf16 path: the GEMMs' operand
+            __nv_bfloat16 *oo = dG_op + r * 4 * H;
+            oo[u] = __float2bfloat16_rn(g0); oo[H + u] = __float2bfloat16_rn(g1);
+            oo[2 * H + u] = __float2bfloat16_rn(g2); oo[3 * H + u] = __float2bfloat16_rn(g3);
+        }
         if (dG3) {  // this step's row as [hi | hi | lo] for the three-product recurrence GEMM
             __nv_bfloat16 *q = dG3 + n * 12 * H;
             const float gv[4] = {g0, g1, g2, g3};
@@ -307,12 +310,12 @@ inline size_t al(size_t x) { return (x + 255) & ~(size_t)255; }
 // fp32 emulation on the tensor cores (each operand split into three bf16 parts, fp32-accurate
 // products), or plain fp32 where the library does not offer it.
 cublasStatus_t gemm(cublasHandle_t hb, bool bf16, bool ta, bool tb, int m, int n, int k, const void *A, long lda,
-                    const void *B, long ldb, float *C, long ldc) {
-    const float one = 1.f, zero = 0.f;
+                    const void *B, long ldb, float *C, long ldc, float beta = 0.f) {
+    const float one = 1.f;
     const cudaDataType_t dt = bf16 ? CUDA_R_16BF : CUDA_R_32F;
     auto run = [&](cublasComputeType_t ct) {
         return cublasGemmEx(hb, tb ? CUBLAS_OP_T : CUBLAS_OP_N, ta ? CUBLAS_OP_T : CUBLAS_OP_N, n, m, k, &one, B, dt,
-                            (int)ldb, A, dt, (int)lda, &zero, C, CUDA_R_32F, (int)ldc, ct, CUBLAS_GEMM_DEFAULT);
+                            (int)ldb, A, dt, (int)lda, &beta, C, CUDA_R_32F, (int)ldc, ct, CUBLAS_GEMM_DEFAULT);
     };
     if (bf16) return run(CUBLAS_COMPUTE_32F);
     const cublasStatus_t st = run(CUBLAS_COMPUTE_32F_EMULATED_16BFX9);
@@ -328,15 +331,20 @@ cudaError_t cublas_err(cublasStatus_t st) {
 }  // namespace
 
 // The forward's outputs at the front of the backward's workspace, then its own buffers.
-void wm_bw_carve(const wm_handle *h, int N, int T, void *base, float **hs, float **cs, float **md, float **nll,
-                 void **tail) {
+void wm_bw_carve(const wm_handle *h, int N, int T, void *base, wm_bw_fwd *f, void **tail) {
     const size_t NT = (size_t)N * T, H = h->cfg.h_dim, M = h->M;
     char *p = (char *)base;
-    *hs = (float *)p; p += al(NT * H * 4);
-    *cs = (float *)p; p += al(NT * H * 4);
-    *md = (float *)p; p += al(NT * M * 4);
-    *nll = (float *)p; p += al((size_t)N * 4);
+    f->hs = (float *)p; p += al(NT * H * 4);
+    f->cs = (float *)p; p += al(NT * H * 4);
+    f->md = (float *)p; p += al(NT * M * 4);
+    f->nll = (float *)p; p += al((size_t)N * 4);
+    f->G = (float *)p; p += al(NT * 4 * H * 4);
     *tail = p;
+}
+
+bool wm_bw_takes_gates(const wm_handle *h, int N, int T) {
+    wm_brecur_args a{};
+    return T > 1 && (size_t)N * T < (1u << 30) && wm_brecur_plan(h->cfg.precision != WM_BF16, N, h->cfg.h_dim, &a);
 }
 
 size_t wm_bw_ws(const wm_handle *h, int N, int T) {
@@ -349,11 +357,12 @@ size_t wm_bw_ws(const wm_handle *h, int N, int T) {
            + al(NT * H4 * 4)                                                   // gate activations
            + al(NT * M * 4) + al(NT * M * es)                                  // dMD
            + al(NT * H * 4)                                                    // dY
-           + al(NT * H4 * 4) + al(NT * H4 * es)                                // dG
+           + al(NT * H4 * 4) + (es == 2 ? al(NT * H4 * 2) : 0)                 // dG
            + 2 * al((size_t)N * H * 4)                                         // dH, dc
            + al((size_t)COLSUM_CHUNKS * part_cols * 4) + al((size_t)CHUNKS * A * H4 * 4)  // partials
            + al(NT * 4) + al((size_t)CHUNKS * (A + 1) * 4)                       // rows sorted by action
-           + (es == 4 ? al((size_t)N * 3 * H4 * 2) : 0) + 256;                   // fp32: dG_t as bf16 parts
+           + (es == 4 ? al((size_t)N * 4 * H4 * 2) : 0)                          // fp32: dG_t as bf16 parts
+           + al((size_t)(N / 128 + 1) * 4) + 256;                                // row-tile counters
 }
 
 cudaError_t wm_bw_prepare(wm_handle *h) {
@@ -412,8 +421,7 @@ void wm_bw_free(wm_handle *h) {
 
 template <class T>
 static cudaError_t bw_run(const wm_handle *h, int N, int TT, const float *z_seq, const int32_t *actions,
-                          const int32_t *lengths, const wm_grads &g, const float *hs, const float *cs,
-                          const float *md, char *p, cudaStream_t s) {
+                          const int32_t *lengths, const wm_grads &g, const wm_bw_fwd &f, char *p, cudaStream_t s) {
     const wm_config &c = h->cfg;
     const bool bf = c.precision == WM_BF16;
     const int Z = c.z_dim, A = c.a_dim, H = c.h_dim, M = h->M, KX = Z + H, H4 = 4 * H;
@@ -421,21 +429,29 @@ static cudaError_t bw_run(const wm_handle *h, int N, int TT, const float *z_seq,
     cublasHandle_t hb = (cublasHandle_t)h->cublas;
     cublasStatus_t st = cublasSetStream(hb, s);
     if (st != CUBLAS_STATUS_SUCCESS) return cublas_err(st);
+    const float *hs = f.hs, *cs = f.cs, *md = f.md;
+    float *G = f.G;
+    // X and Y are built unless the forward left them: its operand rows (bf16), or z_seq and h_t as they
+    // are (fp32, when no product with W_zh is left to do: h_{t-1} is then h_t's row N rows up)
+    const bool built = bf ? !f.frames : !f.have_g;
     T *X = (T *)p; p += al(NT * KX * sizeof(T));
     T *Y = (T *)p; p += al(NT * H * sizeof(T));
-    float *G = (float *)p; p += al(NT * H4 * 4);
     float *dMD = (float *)p; p += al(NT * M * 4);
     T *dMDo = (T *)p; p += al(NT * M * sizeof(T));
     float *dY = (float *)p; p += al(NT * H * 4);
     float *dG = (float *)p; p += al(NT * H4 * 4);
-    T *dGo = (T *)p; p += al(NT * H4 * sizeof(T));
+    __nv_bfloat16 *dGo = bf ? (__nv_bfloat16 *)p : nullptr;  // bf16 path: dG as the GEMMs' operand
+    if (bf) p += al(NT * H4 * 2);
     float *dH = (float *)p; p += al((size_t)N * H * 4);
     float *dC = (float *)p; p += al((size_t)N * H * 4);
     float *part = (float *)p; p += al((size_t)COLSUM_CHUNKS * (H4 > M ? H4 : M) * 4);
     float *apart = (float *)p; p += al((size_t)CHUNKS * A * H4 * 4);
     int32_t *srows = (int32_t *)p; p += al(NT * 4);
     int32_t *soff = (int32_t *)p; p += al((size_t)CHUNKS * (A + 1) * 4);
-    __nv_bfloat16 *dG3 = bf ? nullptr : (__nv_bfloat16 *)p;  // fp32: dG_t as [hi | hi | lo]
+    // fp32: dG_t as [hi | hi | lo], or, in the one-launch recurrence, two steps' rows [hi | lo]
+    __nv_bfloat16 *dG3 = bf ? nullptr : (__nv_bfloat16 *)p;
+    if (!bf) p += al((size_t)N * 4 * H4 * 2);
+    int *count = (int *)p;
     // weights of the GEMMs: W_zh = the z and h rows of the gate matrix, W_mdn, W_h = W_zh's h rows
     const void *Wzh = bf ? (const void *)h->bw_wzh : (const void *)h->step.Wg;
     const long ldw = bf ? H4 : H4 + A;
@@ -444,20 +460,30 @@ static cudaError_t bw_run(const wm_handle *h, int N, int TT, const float *z_seq,
     const void *Wh = bf ? (const void *)((const __nv_bfloat16 *)h->bw_wzh + (size_t)Z * H4)
                         : (const void *)(h->step.Wg + (size_t)Z * (H4 + A));
     int launches = 0;
-    {
+    if (built) {
         wm_ktime kt(h, WM_KERNEL_BW, s);
         k_bw_build<T><<<(unsigned)(NT < 8192 ? NT : 8192), 256, 0, s>>>(N, TT, Z, H, z_seq, hs, X, Y);
         ++launches;
     }
-    {
+    const void *Xz = built ? (const void *)X : bf ? (const void *)f.frames : (const void *)z_seq;
+    const long ldx = built ? KX : bf ? f.ld : Z;
+    if (!f.have_g) {
         wm_ktime kt(h, WM_KERNEL_BW_GEMM, s);
-        st = gemm(hb, bf, false, false, (int)NT, H4, KX, X, KX, Wzh, ldw, G, H4);
+        if (built) {
+            st = gemm(hb, bf, false, false, (int)NT, H4, KX, X, KX, Wzh, ldw, G, H4);
+        } else {  // z columns, then h columns on top (the rows' padding between them is skipped)
+            st = gemm(hb, true, false, false, (int)NT, H4, Z, f.frames, f.ld, Wzh, ldw, G, H4);
+            if (st == CUBLAS_STATUS_SUCCESS)
+                st = gemm(hb, true, false, false, (int)NT, H4, H, f.frames + f.h_col, f.ld,
+                          (const __nv_bfloat16 *)h->bw_wzh + (size_t)Z * H4, ldw, G, H4, 1.f);
+        }
         ++launches;
     }
     if (st != CUBLAS_STATUS_SUCCESS) return cublas_err(st);
     {
         wm_ktime kt(h, WM_KERNEL_BW, s);
-        k_bw_gates<<<(unsigned)(NT < 8192 ? NT : 8192), 256, 0, s>>>(NT, N, H, A, G, actions, h->step.Wa, h->step.bg);
+        if (!f.have_g)
+            k_bw_gates<<<(unsigned)(NT < 8192 ? NT : 8192), 256, 0, s>>>(NT, N, H, A, G, actions, h->step.Wa, h->step.bg);
         k_bw_mdn<T><<<grid_of(NT * Z), 256, 0, s>>>(N, TT, Z, c.k_mix, md, z_seq, lengths, dMD, dMDo);
         launches += 2;
     }
@@ -467,11 +493,29 @@ static cudaError_t bw_run(const wm_handle *h, int N, int TT, const float *z_seq,
         ++launches;
     }
     if (st != CUBLAS_STATUS_SUCCESS) return cublas_err(st);
-    for (int t = TT - 1; t >= 0; --t) {
+    wm_brecur_args ra{};
+    const bool one = TT > 1 && NT < (1u << 30) && wm_brecur_plan(!bf, N, H, &ra);
+    if (one) {
+        CUtensorMap gm, wmap;
+        // (bw_wzh: rows z | h of 4H columns; bw_w3: rows [hi | lo | hi])
+        if (!(bf ? wm_tc_make_map(&gm, dGo, NT, H4, 128) && wm_tc_make_map(&wmap, h->bw_wzh, KX, H4, 64)
+                 : wm_tc_make_map(&gm, dG3, 2 * (size_t)N, 2 * H4, 128) && wm_tc_make_map(&wmap, h->bw_w3, H, 3 * H4, 64)))
+            return cudaErrorInvalidValue;
+        ra.N = N; ra.T = TT; ra.H = H;
+        ra.act = G; ra.cs = cs; ra.dY = dY; ra.pre = f.have_g;
+        ra.dG = dG; ra.dGo = dGo; ra.parts = dG3;
+        ra.count = count; ra.status = h->status; ra.w_row0 = bf ? Z : 0;
+        cudaError_t e = cudaMemsetAsync(count, 0, (size_t)ra.m_tiles * 4, s);
+        if (e != cudaSuccess) return e;
+        wm_ktime kt(h, WM_KERNEL_BW, s);
+        if ((e = wm_brecur_launch(!bf, &gm, &wmap, ra, s)) != cudaSuccess) return e;
+        launches += (ra.m_tiles + ra.m_per_launch - 1) / ra.m_per_launch;
+    }
+    for (int t = TT - 1; t >= 0 && !one; --t) {
         {
             wm_ktime kt(h, WM_KERNEL_BW, s);
             const dim3 grid((unsigned)((H + 255) / 256), (unsigned)(N < 65535 ? N : 65535));
-            k_bw_cell<T><<<grid, 256, 0, s>>>(N, H, t, t == TT - 1, G, cs, dY, dH, dC, dG, dGo, t > 0 ? dG3 : nullptr);
+            k_bw_cell<<<grid, 256, 0, s>>>(N, H, t, t == TT - 1, G, cs, dY, dH, dC, dG, dGo, t > 0 ? dG3 : nullptr);
             ++launches;
         }
         if (t > 0) {
@@ -486,10 +530,16 @@ static cudaError_t bw_run(const wm_handle *h, int N, int TT, const float *z_seq,
     {
         wm_ktime kt(h, WM_KERNEL_BW_GEMM, s);
         // z rows and h rows of dW_lstm: X^T dG, straight into the output's row blocks
-        st = gemm(hb, bf, true, false, Z, H4, (int)NT, X, KX, dGo, H4, g.W_lstm, H4);
+        const void *dGx = bf ? (const void *)dGo : (const void *)dG;  // fp32: dG itself
+        st = gemm(hb, bf, true, false, Z, H4, (int)NT, Xz, ldx, dGx, H4, g.W_lstm, H4);
+        float *dWh = g.W_lstm + (size_t)(Z + A) * H4;
         if (st == CUBLAS_STATUS_SUCCESS)
-            st = gemm(hb, bf, true, false, H, H4, (int)NT, X + Z, KX, dGo, H4, g.W_lstm + (size_t)(Z + A) * H4, H4);
-        if (st == CUBLAS_STATUS_SUCCESS) st = gemm(hb, bf, true, false, H, M, (int)NT, Y, H, dMDo, M, g.W_mdn, M);
+            st = built ? gemm(hb, bf, true, false, H, H4, (int)NT, X + Z, KX, dGx, H4, dWh, H4)
+                 : bf  ? gemm(hb, true, true, false, H, H4, (int)NT, f.frames + f.h_col, f.ld, dGx, H4, dWh, H4)
+                       : gemm(hb, false, true, false, H, H4, (int)(NT - N), hs, H, dG + (size_t)N * H4, H4, dWh, H4);
+        const void *Yx = built ? (const void *)Y : bf ? (const void *)(f.frames + (size_t)N * f.ld + f.h_col) : (const void *)hs;
+        if (st == CUBLAS_STATUS_SUCCESS)
+            st = gemm(hb, bf, true, false, H, M, (int)NT, Yx, built || !bf ? H : f.ld, dMDo, M, g.W_mdn, M);
         launches += 3;
     }
     if (st != CUBLAS_STATUS_SUCCESS) return cublas_err(st);
@@ -509,8 +559,7 @@ static cudaError_t bw_run(const wm_handle *h, int N, int TT, const float *z_seq,
 }
 
 cudaError_t wm_bw_launch(const wm_handle *h, int N, int T, const float *z_seq, const int32_t *actions,
-                         const int32_t *lengths, const wm_grads &g, const float *hs, const float *cs,
-                         const float *md, void *tail, cudaStream_t s) {
+                         const int32_t *lengths, const wm_grads &g, const wm_bw_fwd &f, void *tail, cudaStream_t s) {
     if (N == 0 || T == 0) {  // no rows: every gradient is 0
         const wm_config &c = h->cfg;
         const size_t Z = c.z_dim, A = c.a_dim, H = c.h_dim, M = h->M;
@@ -521,6 +570,6 @@ cudaError_t wm_bw_launch(const wm_handle *h, int N, int T, const float *z_seq, c
         return e;
     }
     if (h->cfg.precision == WM_BF16)
-        return bw_run<__nv_bfloat16>(h, N, T, z_seq, actions, lengths, g, hs, cs, md, (char *)tail, s);
-    return bw_run<float>(h, N, T, z_seq, actions, lengths, g, hs, cs, md, (char *)tail, s);
+        return bw_run<__nv_bfloat16>(h, N, T, z_seq, actions, lengths, g, f, (char *)tail, s);
+    return bw_run<float>(h, N, T, z_seq, actions, lengths, g, f, (char *)tail, s);
 }

@@ -52,6 +52,7 @@ struct wm_nll_dev {
     const int32_t *actions;
     const int32_t *lengths;
     float *nll, *h_seq, *c_seq, *mdn_seq;
+    float *g_seq = nullptr;  // [T, N, 4H] gate pre-activations (tensor family, recurrence in one launch)
 };
 
 // Weights of the stepwise (SIMT) family: fp32 values (bf16-rounded in WM_BF16).
@@ -195,6 +196,9 @@ class wm_ktime {
 int wm_tc_supported(const wm_handle *h);  // the model's sizes are multiples of the tiles'
 int wm_tc_auto_ok(const wm_handle *h);    // a bf16 model it runs with its sizes padded
 bool wm_tc_scores_in_one(const wm_handle *h, int N, int T);  // a scoring call's recurrence is one launch
+// the operand rows [z_t | h_t] (bf16; row t N + n) that a scoring call leaves in its workspace, their
+// stride and the first column of h
+const __nv_bfloat16 *wm_tc_frames(const wm_handle *h, int N, int T, void *ws, int *ld, int *h_col);
 // workspace of a call of B rows; T_teacher >= 0: teacher-forced scoring of T_teacher steps
 // (its operand rows of all T_teacher + 1 frames), -1: a rollout
 size_t wm_tc_ws(const wm_handle *h, int B, int T_teacher = -1);
@@ -216,6 +220,7 @@ struct wm_recur_args {
     const __nv_bfloat16 *wa, *wa_lo;  // [A, 4Hp] action rows, and the bias, in the 128-column packing
     const float *bias;
     float *h_seq, *c_seq;        // [T, N, H] or null
+    float *g_seq;                // [T, N, 4H] gate pre-activations i | f | g | o, or null
     int *count;                  // [m_tiles] zero on entry
     int *status;
     uint32_t test_wait;
@@ -230,6 +235,29 @@ bool wm_recur_plan(int mode, int N, int Hp, int KX, wm_recur_args *a);
 cudaError_t wm_recur_launch(int mode, const void *x_map, const void *xl_map, const void *w_map, const void *wl_map,
                             const wm_recur_args &a, cudaStream_t s);
 
+// ---- the backward recurrence in one launch (wm_brecur.cu) ------------------------------
+enum { BRECUR_MAX_LAUNCHES = 2 };  // row tiles go in as many launches as the SMs make it
+struct wm_brecur_args {
+    int N, T, H;
+    const float *act, *cs, *dY;  // [T N, 4H] activations i | f | g | o, [T N, H] cell states, [T N, H]
+    int pre;                     // act holds pre-activations
+    float *dG;                   // [T N, 4H]
+    __nv_bfloat16 *dGo;          // bf16 path: [T N, 4H]
+    __nv_bfloat16 *parts;        // fp32 path: [2 N, 8H] rows [hi | lo] of two steps
+    int *count;                  // [m_tiles] zero on entry
+    int *status;
+    int w_row0;                  // first row of W_h in its map
+    // the plan
+    int u_tiles, m_tiles, m_per_launch, m0, stages;
+    size_t smem;
+};
+bool wm_brecur_plan(bool f32, int N, int H, wm_brecur_args *a);
+// Maps: the product's operand rows (dGo, or parts) in boxes of 128 x 64; W_h's rows of units (4H gate
+// columns, fp32 path: then their lo parts) in boxes of 64 x 64.
+cudaError_t wm_brecur_launch(bool f32, const void *g_map, const void *w_map, wm_brecur_args a, cudaStream_t s);
+// A 128-byte-swizzled map over a row-major bf16 [rows, cols] matrix (CUtensorMap *), box_rows x 64.
+bool wm_tc_make_map(void *map, const void *base, uint64_t rows, uint64_t cols, uint32_t box_rows);
+
 // ---- the fused family's small-batch member (wm_small.cu) ----------------------
 cudaError_t wm_small_prepare(wm_handle *h);
 cudaError_t wm_small_repack(wm_handle *h);  // after the stepwise weights changed
@@ -240,14 +268,21 @@ cudaError_t wm_small_rollout(const wm_handle *h, const wm_rollout_dev &a, cudaSt
 cudaError_t wm_small_nll(const wm_handle *h, const wm_nll_dev &a, cudaStream_t s);
 
 // ---- the training step (wm_backward.cu) -----------------------------------------
+// What the backward takes from its forward: the outputs of every row and, when the tensor family's
+// one-launch recurrence ran it, the gate pre-activations and (bf16) its operand rows.
+struct wm_bw_fwd {
+    float *hs, *cs, *md, *nll, *G;
+    bool have_g;
+    const __nv_bfloat16 *frames;
+    int ld, h_col;
+};
 size_t wm_bw_ws(const wm_handle *h, int N, int T);
-void wm_bw_carve(const wm_handle *h, int N, int T, void *base, float **hs, float **cs, float **md, float **nll,
-                 void **tail);
+void wm_bw_carve(const wm_handle *h, int N, int T, void *base, wm_bw_fwd *f, void **tail);
+bool wm_bw_takes_gates(const wm_handle *h, int N, int T);  // the backward recurrence reads pre-activations
 cudaError_t wm_bw_prepare(wm_handle *h);
 void wm_bw_free(wm_handle *h);
 cudaError_t wm_bw_launch(const wm_handle *h, int N, int T, const float *z_seq, const int32_t *actions,
-                         const int32_t *lengths, const wm_grads &g, const float *hs, const float *cs,
-                         const float *md, void *tail, cudaStream_t s);
+                         const int32_t *lengths, const wm_grads &g, const wm_bw_fwd &f, void *tail, cudaStream_t s);
 
 // ---- discounted returns (wm_returns.cu) ----------------------------------------
 cudaError_t wm_returns_launch(const wm_handle *h, int B, int T, unsigned long long ep0, float gamma,

@@ -256,6 +256,23 @@ __global__ void __launch_bounds__(THREADS, 1)
             for (int j = 0; j < UT; ++j) cst[((size_t)gi * U + u0 + j) * BM + r] = 0.f;
         int acc = 0;
         uint32_t acc_phase = 0;
+        // UT units of an output row: whole 32-byte sectors where the row's start and length allow
+        const bool whole = (p.H & 7) == 0 && ((reinterpret_cast<uintptr_t>(p.h_seq) | reinterpret_cast<uintptr_t>(p.c_seq)) & 31) == 0;
+        auto store_row = [&](float *q, const float (&v)[UT], int nu) {
+#pragma unroll
+            for (int j0 = 0; j0 < UT; j0 += 8) {
+                if (whole) {
+                    if (j0 < nu)  // (nu is a multiple of 8, or not positive)
+                        asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+                                     :: "l"(q + j0), "f"(v[j0]), "f"(v[j0 + 1]), "f"(v[j0 + 2]), "f"(v[j0 + 3]), "f"(v[j0 + 4]),
+                                        "f"(v[j0 + 5]), "f"(v[j0 + 6]), "f"(v[j0 + 7]) : "memory");
+                } else {
+#pragma unroll
+                    for (int j = j0; j < j0 + 8; ++j)
+                        if (j < nu) q[j] = v[j];
+                }
+            }
+        };
         auto sig = [](float x) { return MODE ? fmaf(0.5f, tanhf(0.5f * x), 0.5f) : fmaf(0.5f, tanh_hw(0.5f * x), 0.5f); };
         auto th = [](float x) { return MODE ? tanhf(x) : tanh_hw(x); };
         // The action row's columns are gathers from L2 (32 lines per load).  They go out right after a
@@ -304,6 +321,17 @@ __global__ void __launch_bounds__(THREADS, 1)
                 float c[UT], h[UT];
                 const size_t o = row * p.H + ug;
                 const int nu = p.H - ug;  // units from ug on that are not padding
+                float pre[4][8];  // eight units' gate pre-activations (for g_seq)
+                // (asked for with H % 8 == 0 and aligned rows only)
+                auto store_pre = [&](int j0) {
+                    if (!valid || !p.g_seq || j0 >= nu) return;
+                    float *q = p.g_seq + 4 * row * p.H + ug + j0;
+#pragma unroll
+                    for (int g = 0; g < 4; ++g, q += p.H)
+                        asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+                                     :: "l"(q), "f"(pre[g][0]), "f"(pre[g][1]), "f"(pre[g][2]), "f"(pre[g][3]), "f"(pre[g][4]),
+                                        "f"(pre[g][5]), "f"(pre[g][6]), "f"(pre[g][7]) : "memory");
+                };
 #pragma unroll
                 for (int j0 = 0; j0 < UT; j0 += 8) {
                     uint32_t v[4][8];
@@ -321,6 +349,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                                 const uint32_t wl = w[PARTS - 1][g][(j0 + j) / 2];
                                 x[g] += __uint_as_float((j & 1) ? wl & 0xffff0000u : wl << 16);
                             }
+                            pre[g][j] = x[g];
                         }
                         float &cs = cst[((size_t)gi * U + u0 + j0 + j) * BM + r];
                         const float cv = sig(x[1]) * cs + sig(x[0]) * th(x[2]);
@@ -328,6 +357,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                         c[j0 + j] = cv;
                         h[j0 + j] = sig(x[3]) * th(cv);
                     }
+                    if (UT > 8) store_pre(j0);  // (held past the counter they would spill)
                 }
                 tc::fence_before_sync();
                 __syncwarp();
@@ -360,14 +390,9 @@ __global__ void __launch_bounds__(THREADS, 1)
                 advance();
                 a1 = act_of(t1, m1);
                 // the optional outputs, off the chain
-                if (valid && p.h_seq)
-#pragma unroll
-                    for (int j = 0; j < UT; ++j)
-                        if (j < nu) p.h_seq[o + j] = h[j];
-                if (valid && p.c_seq)
-#pragma unroll
-                    for (int j = 0; j < UT; ++j)
-                        if (j < nu) p.c_seq[o + j] = c[j];
+                if (UT == 8) store_pre(0);
+                if (valid && p.h_seq) store_row(p.h_seq + o, h, nu);
+                if (valid && p.c_seq) store_row(p.c_seq + o, c, nu);
                 acc ^= 1;
                 if (acc == 0) acc_phase ^= 1u;
             }

@@ -1863,6 +1863,10 @@ __global__ void k_tc_pack(PackGeo g, int units, int rows, int cols, const float 
 // ---------------------------------------------------------------------------
 // Host side: packing, support test, per-call orchestration.
 
+bool wm_tc_make_map(void *map, const void *base, uint64_t rows, uint64_t cols, uint32_t box_rows) {
+    return make_map((CUtensorMap *)map, base, rows, cols, box_rows);
+}
+
 int wm_tc_supported(const wm_handle *h) { return h->tc.ok && h->tc.aligned; }
 int wm_tc_auto_ok(const wm_handle *h) { return h->tc.ok && h->cfg.precision == WM_BF16; }
 
@@ -2003,6 +2007,12 @@ static bool one_launch(const wm_handle *h, int N, int T, wm_recur_args *a, int *
     const wm_tc_weights &w = h->tc;
     *mode = h->cfg.precision == WM_FP32 ? 2 : accurate(h, N, 1) ? 1 : 0;
     return T > 1 && (uint64_t)(T + 1) * N < (1u << 30) && wm_recur_plan(*mode, N, w.Hp, w.Zp + w.Hp, a);
+}
+
+const __nv_bfloat16 *wm_tc_frames(const wm_handle *h, int N, int T, void *ws, int *ld, int *h_col) {
+    *ld = h->tc.Zp + h->tc.Hp;
+    *h_col = h->tc.Zp;
+    return carve_ws(h, N, ws, T).xall;
 }
 
 bool wm_tc_scores_in_one(const wm_handle *h, int N, int T) {
@@ -2153,7 +2163,7 @@ static cudaError_t tc_run(const wm_handle *h, int teacher, const wm_rollout_dev 
             ra_.x = w.xall; ra_.x_lo = w.xall_lo;
             ra_.wa = (const __nv_bfloat16 *)T.wa_n; ra_.wa_lo = (const __nv_bfloat16 *)T.wa_n_lo;
             ra_.bias = T.bg_n;
-            ra_.h_seq = na->h_seq; ra_.c_seq = na->c_seq;
+            ra_.h_seq = na->h_seq; ra_.c_seq = na->c_seq; ra_.g_seq = na->g_seq;
             ra_.count = w.rcount;
             ra_.status = h->status;
             ra_.test_wait = h->test_wait;  // an injected wait goes to the call's first GEMM

@@ -79,3 +79,32 @@ def test_under_stream_capture(wm):
     torch.cuda.synchronize()
     for k in want:
         assert torch.equal(want[k], got[k]), k
+
+
+# the backward recurrence: cluster edges of every hidden size (64 units), row-tile edges, two launches
+# (more row tiles than the SMs hold), one step (no recurrence), the fp32 parts, sizes it leaves
+BACKWARD = [(8, 64, 64, 3, 129, 3, "bf16"), (16, 64, 64, 2, 1, 2, "fp32"), (64, 256, 512, 5, 130, 4, "bf16"),
+            (64, 256, 512, 5, 200, 3, "fp32"), (16, 64, 512, 2, 700, 3, "bf16"), (16, 64, 512, 2, 600, 2, "fp32"),
+            (32, 128, 1024, 3, 140, 2, "bf16"), (16, 64, 1024, 2, 20, 2, "fp32"), (24, 128, 320, 5, 60, 4, "bf16"),
+            (16, 64, 128, 2, 50, 1, "bf16"), (11, 45, 100, 3, 40, 5, "bf16")]
+
+
+@pytest.mark.parametrize("Z,A,H,K,N,T,prec", BACKWARD)
+def test_gradient_against_oracle(wm, orc, Z, A, H, K, N, T, prec):
+    cfg = dict(synth.model_config("nll"), z_dim=Z, a_dim=A, h_dim=H, k_mix=K, precision=prec)
+    w = synth.weights(cfg, seed=44)
+    zs, acts, lens = synth.teacher_inputs(N, T, Z, A, seed=44, ragged=True)
+    acts[1::2, ::5] = -1
+    m = wm.WorldModel(cfg, w)
+    args = (_cuda(zs), _cuda(acts), _cuda(lens))
+    g = m.mdn_nll_backward(*args)
+    m.sync()
+    o = orc.mdn_nll_grad(cfg, w, zs, acts, lens, nthreads=16)
+    # relative Frobenius norms: about 100 fp32 roundoffs, 4 bf16 roundoffs (the operands are rounded once)
+    tol = {"fp32": 1e-5, "bf16": 1e-2}[prec]
+    for k in ("W_lstm", "b_lstm", "W_mdn", "b_mdn"):
+        ref = np.asarray(o[k], np.float64)
+        assert np.linalg.norm(np_(g[k]) - ref) <= tol * max(np.linalg.norm(ref), 1e-30), k
+    again = m.mdn_nll_backward(*args)
+    for k in g:
+        assert torch.equal(g[k], again[k]), k
