@@ -713,6 +713,9 @@ wm_status wm_mdn_nll_backward(wm_handle *h, int N, int T, const float *z_seq, co
     if (path == WM_PATH_TENSOR && N > 0 && T > 0) {
         f.have_g = wm_tc_scores_in_one(h, N, T) && wm_bw_takes_gates(h, N, T);
         if (f.have_g) a.g_seq = f.G;
+        f.have_dmd = true;  // the head GEMM's epilogue forms it: no head outputs are stored
+        a.dmd = f.dMD; a.dmd_op = f.dMDo;
+        a.mdn_seq = nullptr;
         if (c.precision == WM_BF16) f.frames = wm_tc_frames(h, N, T, h->ws, &f.ld, &f.h_col);
     }
     int fwd_launches = 0;

@@ -81,9 +81,9 @@ __global__ void k_bw_gates(size_t NT, int N, int H, int A, float *__restrict__ G
 }
 
 // d NLL / d [logit | mu | log sigma] of one row's latent dim d (0 past the row's length)
-template <class T>
+// (where the forward's head GEMM did not form it)
 __global__ void k_bw_mdn(int N, int TT, int Z, int K, const float *__restrict__ md, const float *__restrict__ z_seq,
-                         const int32_t *__restrict__ lengths, float *__restrict__ dmd, T *__restrict__ dmd_op) {
+                         const int32_t *__restrict__ lengths, float *__restrict__ dmd, __nv_bfloat16 *__restrict__ dmd_op) {
     const int KZ = K * Z, M = 3 * KZ;
     const size_t NT = (size_t)N * TT;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < NT * Z; i += (size_t)gridDim.x * blockDim.x) {
@@ -93,12 +93,12 @@ __global__ void k_bw_mdn(int N, int TT, int Z, int K, const float *__restrict__ 
         len = len < 0 ? 0 : (len > TT ? TT : len);
         const float *row = md + r * M;
         float *out = dmd + r * M;
-        T *oop = dmd_op + r * M;
+        __nv_bfloat16 *oop = dmd_op ? dmd_op + r * M : nullptr;  // bf16 path: the GEMMs' operand
         if (t >= len) {
             for (int k = 0; k < K; ++k)
                 for (int p = 0; p < 3; ++p) {
                     out[p * KZ + d * K + k] = 0.f;
-                    oop[p * KZ + d * K + k] = to_op<T>(0.f);
+                    if (oop) oop[p * KZ + d * K + k] = __float2bfloat16_rn(0.f);
                 }
             continue;
         }
@@ -122,9 +122,10 @@ __global__ void k_bw_mdn(int N, int TT, int Z, int K, const float *__restrict__ 
             out[d * K + k] = v0;
             out[KZ + d * K + k] = v1;
             out[2 * KZ + d * K + k] = v2;
-            oop[d * K + k] = to_op<T>(v0);
-            oop[KZ + d * K + k] = to_op<T>(v1);
-            oop[2 * KZ + d * K + k] = to_op<T>(v2);
+            if (!oop) continue;
+            oop[d * K + k] = __float2bfloat16_rn(v0);
+            oop[KZ + d * K + k] = __float2bfloat16_rn(v1);
+            oop[2 * KZ + d * K + k] = __float2bfloat16_rn(v2);
         }
     }
 }
@@ -339,6 +340,9 @@ void wm_bw_carve(const wm_handle *h, int N, int T, void *base, wm_bw_fwd *f, voi
     f->md = (float *)p; p += al(NT * M * 4);
     f->nll = (float *)p; p += al((size_t)N * 4);
     f->G = (float *)p; p += al(NT * 4 * H * 4);
+    f->dMD = (float *)p; p += al(NT * M * 4);
+    f->dMDo = nullptr;
+    if (h->cfg.precision == WM_BF16) { f->dMDo = (__nv_bfloat16 *)p; p += al(NT * M * 2); }
     *tail = p;
 }
 
@@ -355,7 +359,7 @@ size_t wm_bw_ws(const wm_handle *h, int N, int T) {
     return al(NT * H * 4) * 2 + al(NT * M * 4) + al((size_t)N * 4)             // h, c, head outputs, nll
            + al(NT * KX * es) + al(NT * H * es)                                // X, Y
            + al(NT * H4 * 4)                                                   // gate activations
-           + al(NT * M * 4) + al(NT * M * es)                                  // dMD
+           + al(NT * M * 4) + (es == 2 ? al(NT * M * 2) : 0)                   // dMD
            + al(NT * H * 4)                                                    // dY
            + al(NT * H4 * 4) + (es == 2 ? al(NT * H4 * 2) : 0)                 // dG
            + 2 * al((size_t)N * H * 4)                                         // dH, dc
@@ -429,15 +433,15 @@ static cudaError_t bw_run(const wm_handle *h, int N, int TT, const float *z_seq,
     cublasHandle_t hb = (cublasHandle_t)h->cublas;
     cublasStatus_t st = cublasSetStream(hb, s);
     if (st != CUBLAS_STATUS_SUCCESS) return cublas_err(st);
-    const float *hs = f.hs, *cs = f.cs, *md = f.md;
+    const float *hs = f.hs, *cs = f.cs;
     float *G = f.G;
     // X and Y are built unless the forward left them: its operand rows (bf16), or z_seq and h_t as they
     // are (fp32, when no product with W_zh is left to do: h_{t-1} is then h_t's row N rows up)
     const bool built = bf ? !f.frames : !f.have_g;
     T *X = (T *)p; p += al(NT * KX * sizeof(T));
     T *Y = (T *)p; p += al(NT * H * sizeof(T));
-    float *dMD = (float *)p; p += al(NT * M * 4);
-    T *dMDo = (T *)p; p += al(NT * M * sizeof(T));
+    float *dMD = f.dMD;
+    const void *dMDo = bf ? (const void *)f.dMDo : (const void *)dMD;  // the GEMMs' operand
     float *dY = (float *)p; p += al(NT * H * 4);
     float *dG = (float *)p; p += al(NT * H4 * 4);
     __nv_bfloat16 *dGo = bf ? (__nv_bfloat16 *)p : nullptr;  // bf16 path: dG as the GEMMs' operand
@@ -480,11 +484,11 @@ static cudaError_t bw_run(const wm_handle *h, int N, int TT, const float *z_seq,
         ++launches;
     }
     if (st != CUBLAS_STATUS_SUCCESS) return cublas_err(st);
-    {
+    if (!f.have_g || !f.have_dmd) {
         wm_ktime kt(h, WM_KERNEL_BW, s);
         if (!f.have_g)
             k_bw_gates<<<(unsigned)(NT < 8192 ? NT : 8192), 256, 0, s>>>(NT, N, H, A, G, actions, h->step.Wa, h->step.bg);
-        k_bw_mdn<T><<<grid_of(NT * Z), 256, 0, s>>>(N, TT, Z, c.k_mix, md, z_seq, lengths, dMD, dMDo);
+        if (!f.have_dmd) k_bw_mdn<<<grid_of(NT * Z), 256, 0, s>>>(N, TT, Z, c.k_mix, f.md, z_seq, lengths, dMD, f.dMDo);
         launches += 2;
     }
     {

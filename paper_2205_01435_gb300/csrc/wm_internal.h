@@ -53,6 +53,9 @@ struct wm_nll_dev {
     const int32_t *lengths;
     float *nll, *h_seq, *c_seq, *mdn_seq;
     float *g_seq = nullptr;  // [T, N, 4H] gate pre-activations (tensor family, recurrence in one launch)
+    // tensor family: the NLL's gradient with respect to the head outputs [T, N, M], and its bf16 copy
+    float *dmd = nullptr;
+    __nv_bfloat16 *dmd_op = nullptr;
 };
 
 // Weights of the stepwise (SIMT) family: fp32 values (bf16-rounded in WM_BF16).
@@ -271,8 +274,9 @@ cudaError_t wm_small_nll(const wm_handle *h, const wm_nll_dev &a, cudaStream_t s
 // What the backward takes from its forward: the outputs of every row and, when the tensor family's
 // one-launch recurrence ran it, the gate pre-activations and (bf16) its operand rows.
 struct wm_bw_fwd {
-    float *hs, *cs, *md, *nll, *G;
-    bool have_g;
+    float *hs, *cs, *md, *nll, *G, *dMD;
+    __nv_bfloat16 *dMDo;  // bf16: dMD's copy
+    bool have_g, have_dmd;
     const __nv_bfloat16 *frames;
     int ld, h_col;
 };

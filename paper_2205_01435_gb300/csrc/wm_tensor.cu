@@ -166,6 +166,8 @@ struct StepIO {
     float *h_seq, *c_seq, *mdn_seq;
     uint8_t *comp_seq;
     float *nll_part;                // [n_head_tiles, B]
+    float *dmd;                     // teacher: d NLL / d head outputs [T N, M] (in place of mdn_seq), or null
+    __nv_bfloat16 *dmd_op;          // and its bf16 copy, or null
     // shaped reward (Sec. 3.1.4, Eq. 2): columns rd_col + 2, + 3 predict runtime and memory
     // accesses; rt, mem carry each episode's last predictions
     int reward_mode;
@@ -818,7 +820,8 @@ using EpiGatesNA = EpiGatesT<0, 32, true>;
 // stored by all 128 threads in row-major order, so a warp's stores cover a few contiguous
 // row segments instead of 32 rows.
 // ACC: accurate exponentials and divisions in the draw (as EpiGatesT's ACC).
-template <bool ACC>
+// TEACH: teacher-forced scoring (one batched GEMM over all rows) instead of a rollout's step.
+template <bool ACC, bool TEACH>
 struct EpiHeadsT {
     static constexpr bool TMA_STAGE = false;
     static constexpr int ZS_PITCH = 33;
@@ -841,7 +844,7 @@ struct EpiHeadsT {
         // the row's draws for the tile's dims (a5, a7): Philox blocks of 4 dims
         const int b0 = m * BM + x.row;
         const int b = b0 < p.live_rows() ? b0 : 0;
-        if (p.teacher || !(p.mdn_tau > 0.f) || p.fz_cur[b]) return;
+        if (TEACH || !(p.mdn_tau > 0.f) || p.fz_cur[b]) return;
         const unsigned long long ep = p.ep0 + p.ep_of(b);
         const int d0 = n * p.dims_per_tile, nd = min(p.dims_per_tile, p.Z - d0);
         float *es = reinterpret_cast<float *>(x.stage), *us = reinterpret_cast<float *>(x.stage + US_OFF);
@@ -860,7 +863,138 @@ struct EpiHeadsT {
             }
         }
     }
-    static __device__ void run(const StepIO &p, uint32_t tacc, int m, int n, EpiCtx &x, const Pre &, int, int) {
+    // A dim's logits, means and log sigmas (accumulator + bias).  Its columns are component-interleaved
+    // (logit, mu, log sigma) so that every register index is static: no local-memory arrays.
+    static __device__ __forceinline__ void dim_values(uint32_t tcol, const float *bias, int K, float (&lg)[8], float (&mu)[8],
+                                                      float (&ls)[8]) {
+        float v[24];
+        {
+            uint32_t r0[8], r1[8], r2[8];
+            TC_LD8(tcol, r0);
+            TC_LD8(tcol + 8, r1);
+            TC_LD8(tcol + 16, r2);  // past the dim when 3K <= 16: unused
+            tc::tmem_ld_wait();
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                v[j] = __uint_as_float(r0[j]);
+                v[8 + j] = __uint_as_float(r1[j]);
+                v[16 + j] = __uint_as_float(r2[j]);
+            }
+        }
+        float bv[24];  // (a dim's columns start at a multiple of 8 floats: 16-byte aligned)
+        const float4 *b4 = reinterpret_cast<const float4 *>(bias);
+#pragma unroll
+        for (int j = 0; j < 6; ++j) {
+            const float4 t = b4[j];
+            bv[4 * j] = t.x; bv[4 * j + 1] = t.y; bv[4 * j + 2] = t.z; bv[4 * j + 3] = t.w;
+        }
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            lg[k] = k < K ? v[3 * k] + bv[3 * k] : -INFINITY;
+            mu[k] = k < K ? v[3 * k + 1] + bv[3 * k + 1] : 0.f;
+            ls[k] = k < K ? v[3 * k + 2] + bv[3 * k + 2] : 0.f;
+        }
+    }
+    static __device__ void run(const StepIO &p, uint32_t tacc, int m, int n, EpiCtx &x, const Pre &pr, int nm, int nn) {
+        if constexpr (TEACH) run_teacher(p, tacc, m, n, x);
+        else run_rollout(p, tacc, m, n, x, pr, nm, nn);
+    }
+    // The NLL partials of the tile's rows, and, when asked for, the head outputs (mdn_seq) or the NLL's
+    // gradient with respect to them (dmd, and its bf16 copy dmd_op).  Column group g takes dims g, g + 4,
+    // ... so that a turn covers four consecutive dims; their values go through the quadrant's stage and
+    // leave as contiguous row segments (stored from the registers, a lane per row, every store touched 32
+    // sectors: the GEMM over 65,536 rows with mdn_seq took 430 us, 118 without).
+    static __device__ void run_teacher(const StepIO &p, uint32_t tacc, int m, int n, EpiCtx &x) {
+        const int b0 = m * BM + x.row, nrows = p.B;
+        const bool valid = b0 < nrows;
+        const int e = valid ? b0 : 0;  // rows past the batch compute on row 0 and store nothing
+        const int Z = p.Z, K = p.K, KZ = K * Z;
+        const size_t M = (size_t)3 * KZ;
+        const int DS = (3 * K + 7) & ~7;
+        const int d0 = n * p.dims_per_tile, nd = min(p.dims_per_tile, Z - d0);
+        const float *bh = reinterpret_cast<const float *>(x.stage + BIAS_OFF);  // the tile's bias
+        float *st = reinterpret_cast<float *>(x.stage);                         // [parts][32][pitch]
+        const int sq = e % p.nseq, tt = e / p.nseq;                             // sequence, step
+        const int len = p.lengths ? p.lengths[sq] : p.T;
+        if (valid && tt == 0 && n == 0 && x.cg == 0 && (len < 0 || len > p.T)) report_status(x.status, WM_ERR_INVALID_ARG);
+        const bool counted = tt < len;
+        const bool out = p.mdn_seq || p.dmd;  // uniform
+        const int pitch = 4 * K + 1, per = K <= 5 ? 3 : 2;  // parts staged at once (the stage holds 2 * ZS_ALIGNED)
+        float nll = 0.f;
+        x.sync();  // the quadrant's bias copy is complete
+        for (int i0 = 0; i0 < nd; i0 += 4) {
+            const int i = i0 + x.cg, na = min(4, nd - i0);  // warp-uniform
+            float lg[8], mu[8], ls[8];
+            if (i < nd) {
+                dim_values(tacc + DS * i, bh + DS * i, K, lg, mu, ls);
+                const float xv = p.z_tgt[(size_t)e * Z + d0 + i];
+                float mx = -INFINITY;
+#pragma unroll
+                for (int k = 0; k < 8; ++k) if (k < K) mx = fmaxf(mx, lg[k]);
+                float s = 0.f;
+#pragma unroll
+                for (int k = 0; k < 8; ++k) if (k < K) s += expf(lg[k] - mx);
+                const float lse = mx + logf(s);
+                float lp[8], tmax = -INFINITY;
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    if (k < K) {
+                        const float zsd = (xv - mu[k]) * expf(-ls[k]);
+                        lp[k] = (lg[k] - lse) - 0.5f * zsd * zsd - ls[k] - 0.91893853320467274178f;
+                        tmax = fmaxf(tmax, lp[k]);
+                    }
+                }
+                float acc = 0.f;
+#pragma unroll
+                for (int k = 0; k < 8; ++k) if (k < K) acc += expf(lp[k] - tmax);
+                const float lse2 = tmax + logf(acc);
+                nll += -lse2;
+                if (p.dmd) {  // responsibilities against softmax weights; the means; the log sigmas
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) {
+                        if (k < K) {
+                            const float pi = expf(lg[k] - lse), gam = expf(lp[k] - lse2);
+                            const float is = expf(-ls[k]), zsd = (xv - mu[k]) * is;
+                            lg[k] = counted ? pi - gam : 0.f;
+                            mu[k] = counted ? -gam * zsd * is : 0.f;
+                            ls[k] = counted ? gam * (1.f - zsd * zsd) : 0.f;
+                        }
+                    }
+                }
+            }
+            if (!out) continue;
+            for (int p0 = 0; p0 < 3; p0 += per) {
+                if (i < nd) {
+#pragma unroll
+                    for (int q = 0; q < 3; ++q) {
+                        if (q < p0 || q >= p0 + per) continue;
+                        float *o = st + ((q - p0) * 32 + x.lane) * pitch + x.cg * K;
+#pragma unroll
+                        for (int k = 0; k < 8; ++k)
+                            if (k < K) o[k] = q == 0 ? lg[k] : q == 1 ? mu[k] : ls[k];
+                    }
+                }
+                x.sync();
+                const int y0 = m * BM + 32 * x.quad;
+                if (x.lane < na * K)
+                    for (int q = p0; q < 3 && q < p0 + per; ++q)
+#pragma unroll
+                        for (int rr = 0; rr < 8; ++rr) {  // a row per warp and turn, a column per lane
+                            const int r = 8 * x.cg + rr;
+                            if (y0 + r >= nrows) break;
+                            const float v = st[((q - p0) * 32 + r) * pitch + x.lane];
+                            const size_t o = (size_t)(y0 + r) * M + (size_t)q * KZ + (size_t)(d0 + i0) * K + x.lane;
+                            if (p.mdn_seq) p.mdn_seq[o] = v;
+                            if (p.dmd) p.dmd[o] = v;
+                            if (p.dmd_op) p.dmd_op[o] = __float2bfloat16_rn(v);
+                        }
+                x.sync();
+            }
+        }
+        if (valid) p.nll_part[((size_t)n * 4 + x.cg) * p.B + e] = counted ? nll : 0.f;
+        x.sync();  // the bias copy may be rewritten by the next tile
+    }
+    static __device__ void run_rollout(const StepIO &p, uint32_t tacc, int m, int n, EpiCtx &x, const Pre &, int, int) {
         const int b0 = m * BM + x.row;
         const int nrows = p.live_rows();
         const bool valid = b0 < nrows;
@@ -868,54 +1002,23 @@ struct EpiHeadsT {
         const int e = p.ep_of(b);     // the row's episode
         const int Z = p.Z, K = p.K, KZ = K * Z, M = 3 * KZ, KX = p.Zp + p.Hp;
         const int DS = (3 * K + 7) & ~7;  // columns per latent dim (8-aligned TMEM loads)
-        const bool fz = !p.teacher && p.fz_cur[b] != 0;
+        const bool fz = p.fz_cur[b] != 0;
         const size_t tb = (size_t)p.t * p.B + e;
         const int d0 = n * p.dims_per_tile;
         const int nd = min(p.dims_per_tile, Z - d0);
         const float *bh = reinterpret_cast<const float *>(x.stage + BIAS_OFF);  // the tile's bias
         float *zs = reinterpret_cast<float *>(x.stage);  // the normal draws, then z'
         const float *us = reinterpret_cast<const float *>(x.stage + US_OFF);
-        float nll = 0.f;
         x.sync();  // the quadrant's bias copy and draws are complete
         {
             for (int i = x.cg; i < nd; i += 4) {  // warp-uniform bounds
                 const int d = d0 + i;
-                float v[24];
-                {
-                    uint32_t r0[8], r1[8], r2[8];
-                    TC_LD8(tacc + DS * i, r0);
-                    TC_LD8(tacc + DS * i + 8, r1);
-                    TC_LD8(tacc + DS * i + 16, r2);  // past the dim when 3K <= 16: unused
-                    tc::tmem_ld_wait();
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        v[j] = __uint_as_float(r0[j]);
-                        v[8 + j] = __uint_as_float(r1[j]);
-                        v[16 + j] = __uint_as_float(r2[j]);
-                    }
-                }
-                // columns of a dim are component-interleaved (logit, mu, log sigma) so that every
-                // register index below is static: no local-memory arrays
                 float lg[8], mu[8], ls[8];
-                {
-                    float bv[24];  // DS * i is a multiple of 8 floats: 16-byte aligned
-                    const float4 *b4 = reinterpret_cast<const float4 *>(bh + DS * i);
-#pragma unroll
-                    for (int j = 0; j < 6; ++j) {
-                        const float4 t = b4[j];
-                        bv[4 * j] = t.x; bv[4 * j + 1] = t.y; bv[4 * j + 2] = t.z; bv[4 * j + 3] = t.w;
-                    }
-#pragma unroll
-                    for (int k = 0; k < 8; ++k) {
-                        lg[k] = k < K ? v[3 * k] + bv[3 * k] : -INFINITY;
-                        mu[k] = k < K ? v[3 * k + 1] + bv[3 * k + 1] : 0.f;
-                        ls[k] = k < K ? v[3 * k + 2] + bv[3 * k + 2] : 0.f;
-                    }
-                }
+                dim_values(tacc + DS * i, bh + DS * i, K, lg, mu, ls);
                 if (!valid) continue;
                 if (p.mdn_seq) {
                     float *ms = p.mdn_seq + tb * M;
-                    const bool zero = fz && !p.teacher;
+                    const bool zero = fz;
 #pragma unroll
                     for (int k = 0; k < 8; ++k) {
                         if (k < K) {
@@ -926,30 +1029,7 @@ struct EpiHeadsT {
                     }
                 }
                 float zn;
-                if (p.teacher) {
-                    const float xv = p.z_tgt[(size_t)e * Z + d];
-                    float mx = -INFINITY;
-#pragma unroll
-                    for (int k = 0; k < 8; ++k) if (k < K) mx = fmaxf(mx, lg[k]);
-                    float s = 0.f;
-#pragma unroll
-                    for (int k = 0; k < 8; ++k) if (k < K) s += expf(lg[k] - mx);
-                    const float lse = mx + logf(s);
-                    float lp[8], tmax = -INFINITY;
-#pragma unroll
-                    for (int k = 0; k < 8; ++k) {
-                        if (k < K) {
-                            const float zsd = (xv - mu[k]) * expf(-ls[k]);
-                            lp[k] = (lg[k] - lse) - 0.5f * zsd * zsd - ls[k] - 0.91893853320467274178f;
-                            tmax = fmaxf(tmax, lp[k]);
-                        }
-                    }
-                    float acc = 0.f;
-#pragma unroll
-                    for (int k = 0; k < 8; ++k) if (k < K) acc += expf(lp[k] - tmax);
-                    nll += -(tmax + logf(acc));
-                    zn = xv;
-                } else if (fz) {
+                if (fz) {
                     zn = p.z_out[tb * Z + d];
                     if (p.comp_seq) p.comp_seq[tb * Z + d] = 255;
                 } else {
@@ -1008,15 +1088,6 @@ struct EpiHeadsT {
                 zs[x.lane * ZS_PITCH + i] = zn;
             }
         }
-        if (p.teacher && valid) {
-            const int sq = p.nseq ? e % p.nseq : e, tt = p.nseq ? e / p.nseq : p.t;  // sequence, step
-            const int len = p.lengths ? p.lengths[sq] : p.T;
-            if (tt == 0 && n == 0 && x.cg == 0 && (len < 0 || len > p.T))
-                report_status(x.status, WM_ERR_INVALID_ARG);
-            float *part = p.nll_part + ((size_t)n * 4 + x.cg) * p.B + e;
-            if (p.nseq) *part = tt < len ? nll : 0.f;  // one row per (step, sequence)
-            else if (tt < len) *part += nll;
-        }
         if (n == p.rd_tile) {
             const bool shaped = p.reward_mode == WM_REWARD_SHAPED;  // uniform
             uint32_t r[2], q[2] = {0u, 0u};
@@ -1031,7 +1102,7 @@ struct EpiHeadsT {
                              : "=r"(vr) : "r"(tacc + p.rd_col + p.nr - 1));
             tc::tmem_ld_wait();
             const float vq = __uint_as_float(vr);
-            if (!p.teacher && valid && x.cg == 0) {
+            if (valid && x.cg == 0) {
                 float rew = __uint_as_float(r[0]) + bh[p.rd_col];
                 const float dl = __uint_as_float(r[1]) + bh[p.rd_col + 1];
                 const int a = p.act[b];
@@ -1063,19 +1134,18 @@ struct EpiHeadsT {
             const int rr = j / nd, i = j - rr * nd;
             const size_t bb = (size_t)(y0 + rr);
             const float zn = zs[rr * ZS_PITCH + i];
-            if (!p.teacher) p.z_out[((size_t)(p.t + 1) * p.B + p.ep_of((int)bb)) * Z + d0 + i] = zn;
-            if (p.x_next) {  // (a batched scoring GEMM has no next operand: the frames are staged)
-                const __nv_bfloat16 zh = __float2bfloat16_rn(zn);
-                p.x_next[bb * KX + d0 + i] = zh;
-                if (p.x_next_lo) p.x_next_lo[bb * KX + d0 + i] = __float2bfloat16_rn(zn - __bfloat162float(zh));
-            }
+            p.z_out[((size_t)(p.t + 1) * p.B + p.ep_of((int)bb)) * Z + d0 + i] = zn;
+            const __nv_bfloat16 zh = __float2bfloat16_rn(zn);
+            p.x_next[bb * KX + d0 + i] = zh;
+            if (p.x_next_lo) p.x_next_lo[bb * KX + d0 + i] = __float2bfloat16_rn(zn - __bfloat162float(zh));
         }
         x.sync();  // the staging may be rewritten by the next tile
     }
 };
 
-using EpiHeads = EpiHeadsT<false>;
-using EpiHeadsA = EpiHeadsT<true>;
+using EpiHeads = EpiHeadsT<false, false>;
+using EpiHeadsA = EpiHeadsT<true, false>;
+using EpiHeadsScore = EpiHeadsT<false, true>;
 
 // ---------------------------------------------------------------------------
 // The persistent warp-specialised GEMM on CTA pairs.  A pair computes 256-row tiles of
@@ -2237,11 +2307,13 @@ static cudaError_t tc_run(const wm_handle *h, int teacher, const wm_rollout_dev 
             hio.nseq = B;
             hio.z_tgt = na->z_seq + (size_t)B * Z;
             hio.nll_part = w.part;
+            hio.dmd = na->dmd;
+            hio.dmd_op = na->dmd_op;
             const GemmGrid g3{(rows + 2 * BM - 1) / (2 * BM), T.n_head_tiles, (Hp + BK - 1) / BK, Zp, h->status};
             const OpMaps oph{&mh, &mwh, &mhl, &mwhl};
             wm_ktime kt(h, WM_KERNEL_TC_HEADS, s);
-            if (f32) e = launch_gemm<HEAD_TILE, 1, 3, EpiHeads, 2, 3>(oph, mc, mc, mc, g3, hio, T.sms, s, pdl);
-            else e = launch_gemm<HEAD_TILE, 1, 3, EpiHeads, 2>(oph, mc, mc, mc, g3, hio, T.sms, s, pdl);
+            if (f32) e = launch_gemm<HEAD_TILE, 1, 3, EpiHeadsScore, 2, 3>(oph, mc, mc, mc, g3, hio, T.sms, s, pdl);
+            else e = launch_gemm<HEAD_TILE, 1, 3, EpiHeadsScore, 2>(oph, mc, mc, mc, g3, hio, T.sms, s, pdl);
             ++launches;
             if (e != cudaSuccess) return e;
         }
