@@ -172,23 +172,50 @@ __global__ void k_bw_cell(int N, int H, int t, int first, const float *__restric
     }
 }
 
+// Compensated (Kahan) fp32 sum: the error stays near one rounding however many terms.
+struct Kahan {
+    float s = 0.f, comp = 0.f;
+    __device__ __forceinline__ void add(float v) {
+        const float y = v - comp, t = s + y;
+        comp = (t - s) - y;
+        s = t;
+    }
+};
+
 // Column sums of a [R, C] matrix, two levels: chunk c of the rows (COLSUM_CHUNKS of them)
-// into part[c][C], then the chunks' partials in order.  One thread per column, rows in
-// order, a compensated (Kahan) fp32 sum: the error stays near one rounding whatever R,
-// and the order, so the result, is fixed.
+// into part[c][C], then the chunks' partials in order.  The order, so the result, is fixed.
+// C % 4 == 0: a thread takes four columns and every fourth row of the chunk, and the four row
+// lanes are combined in order (one column a thread and all rows: 106 us for 65,536 x 960, bound by
+// the loads in flight).  Other C: one thread per column, rows in order.
 constexpr int COLSUM_CHUNKS = 64;
+__global__ void __launch_bounds__(256) k_bw_colsum4(size_t R, int C, const float *__restrict__ in, float *__restrict__ part) {
+    __shared__ float4 lanes[3][64];
+    const int q = threadIdx.x & 63, l = threadIdx.x >> 6, col = 4 * (blockIdx.x * 64 + q), c = blockIdx.y;
+    const size_t r0 = R * c / COLSUM_CHUNKS, r1 = R * (c + 1) / COLSUM_CHUNKS;
+    Kahan k[4];
+    if (col < C) {
+#pragma unroll 8
+        for (size_t r = r0 + l; r < r1; r += 4) {
+            const float4 v = *reinterpret_cast<const float4 *>(in + r * C + col);
+            k[0].add(v.x); k[1].add(v.y); k[2].add(v.z); k[3].add(v.w);
+        }
+    }
+    if (l) lanes[l - 1][q] = make_float4(k[0].s, k[1].s, k[2].s, k[3].s);
+    __syncthreads();
+    if (l || col >= C) return;
+    for (int i = 0; i < 3; ++i) {
+        const float4 v = lanes[i][q];
+        k[0].add(v.x); k[1].add(v.y); k[2].add(v.z); k[3].add(v.w);
+    }
+    *reinterpret_cast<float4 *>(part + (size_t)c * C + col) = make_float4(k[0].s, k[1].s, k[2].s, k[3].s);
+}
 __global__ void k_bw_colsum(size_t R, int C, const float *__restrict__ in, float *__restrict__ part) {
     const int col = blockIdx.x * blockDim.x + threadIdx.x, c = blockIdx.y;
     if (col >= C) return;
     const size_t r0 = R * c / COLSUM_CHUNKS, r1 = R * (c + 1) / COLSUM_CHUNKS;
-    float s = 0.f, comp = 0.f;
-    for (size_t r = r0; r < r1; ++r) {
-        const float y = in[r * C + col] - comp;
-        const float t = s + y;
-        comp = (t - s) - y;
-        s = t;
-    }
-    part[(size_t)c * C + col] = s;
+    Kahan k;
+    for (size_t r = r0; r < r1; ++r) k.add(in[r * C + col]);
+    part[(size_t)c * C + col] = k.s;
 }
 __global__ void k_bw_colsum_fin(int C, const float *__restrict__ part, float *__restrict__ out) {
     const int col = blockIdx.x * blockDim.x + threadIdx.x;
@@ -198,76 +225,85 @@ __global__ void k_bw_colsum_fin(int C, const float *__restrict__ part, float *__
     out[col] = (float)s;
 }
 
-// The action rows of dW_lstm: dW_a[a] = sum of the dG rows whose action is a.  Each row
-// chunk is first sorted stably by action (k_bw_rowsort: one block per chunk, rows taken in
-// order by one warp 32 at a time, each lane's place among the lanes with the same action
-// from a match mask), then block (a, c) sums, in row order, only the rows of chunk c with
-// action a, into part[c][a][4H]; then the CHUNKS partials in order.
+// The action rows of dW_lstm: dW_a[a] = sum of the dG rows whose action is a, and bucket A the rows
+// without an action.  Each row chunk is first sorted stably by bucket (k_bw_rowsort: one block per
+// chunk, rows taken in order by one warp 32 at a time, each lane's place among the lanes with the same
+// bucket from a match mask), then block (a, c) sums, in row order, only the rows of chunk c in bucket a,
+// into part[c][a][4H]; then the CHUNKS partials in order.  db_lstm is the sum of all buckets'
+// partials: dG (fp32, half a gigabyte at 65,536 rows of H = 512) is read once for both.
 __global__ void k_bw_rowsort(size_t R, int A, const int32_t *__restrict__ act, int32_t *__restrict__ srows,
                              int32_t *__restrict__ soff) {
-    extern __shared__ int s_cnt[];  // [A] counts, then running cursors
+    extern __shared__ int s_cnt[];  // [A + 1] counts, then running cursors
     const int c = blockIdx.x;
     const size_t r0 = R * c / CHUNKS, r1 = R * (c + 1) / CHUNKS;
-    for (int a = threadIdx.x; a < A; a += blockDim.x) s_cnt[a] = 0;
+    for (int a = threadIdx.x; a <= A; a += blockDim.x) s_cnt[a] = 0;
     __syncthreads();
     for (size_t r = r0 + threadIdx.x; r < r1; r += blockDim.x) {
         const int a = act[r];
-        if (a >= 0 && a < A) atomicAdd(&s_cnt[a], 1);
+        atomicAdd(&s_cnt[a >= 0 && a < A ? a : A], 1);
     }
     __syncthreads();
     if (threadIdx.x == 0) {  // exclusive offsets within the chunk
         int run = 0;
-        int32_t *off = soff + (size_t)c * (A + 1);
-        for (int a = 0; a < A; ++a) {
+        int32_t *off = soff + (size_t)c * (A + 2);
+        for (int a = 0; a <= A; ++a) {
             const int n = s_cnt[a];
             off[a] = run;
             s_cnt[a] = run;
             run += n;
         }
-        off[A] = run;
+        off[A + 1] = run;
     }
     __syncthreads();
     if (threadIdx.x < 32) {
         const int lane = threadIdx.x;
-        for (size_t b = r0; b < r1; b += 32) {
-            const size_t r = b + lane;
-            const int a = r < r1 ? act[r] : -1;
-            const bool ok = a >= 0 && a < A;
-            const uint32_t same = __match_any_sync(0xffffffffu, ok ? a : -1);
-            const int rank = __popc(same & ((1u << lane) - 1u));
-            int pos = 0;
-            if (ok) pos = s_cnt[a] + rank;
-            __syncwarp();
-            if (ok && rank == 0) s_cnt[a] += __popc(same);  // the lowest lane of each action
-            __syncwarp();
-            if (ok) srows[r0 + pos] = (int32_t)r;
+        for (size_t b8 = r0; b8 < r1; b8 += 256) {  // eight loads in flight, then their rows in order
+            int av[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const size_t r = b8 + 32 * i + lane;
+                av[i] = r < r1 ? act[r] : -1;
+            }
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const size_t r = b8 + 32 * i + lane;
+                const bool ok = r < r1;
+                const int a = ok && (av[i] < 0 || av[i] >= A) ? A : av[i];
+                const uint32_t same = __match_any_sync(0xffffffffu, a);
+                const int rank = __popc(same & ((1u << lane) - 1u));
+                int pos = 0;
+                if (ok) pos = s_cnt[a] + rank;
+                __syncwarp();
+                if (ok && rank == 0) s_cnt[a] += __popc(same);  // the lowest lane of each action
+                __syncwarp();
+                if (ok) srows[r0 + pos] = (int32_t)r;
+            }
         }
     }
 }
-__global__ void k_bw_arows(size_t R, int A, int H4, const int32_t *__restrict__ srows,
-                           const int32_t *__restrict__ soff, const float *__restrict__ dG, float *__restrict__ part) {
+__global__ void __launch_bounds__(256) k_bw_arows(size_t R, int A, int H4, const int32_t *__restrict__ srows,
+                                                  const int32_t *__restrict__ soff, const float *__restrict__ dG,
+                                                  float *__restrict__ part) {
     const int a = blockIdx.x, c = blockIdx.y;
     const size_t r0 = R * c / CHUNKS;
-    const int32_t *off = soff + (size_t)c * (A + 1);
+    const int32_t *off = soff + (size_t)c * (A + 2);
     const int i0 = off[a], i1 = off[a + 1];
-    for (int col0 = 0; col0 < H4; col0 += blockDim.x * 4) {
-        float s[4] = {0.f, 0.f, 0.f, 0.f};
-        const int col = col0 + 4 * threadIdx.x;
+    for (int col = 4 * threadIdx.x; col < H4; col += 4 * blockDim.x) {  // (H4 is a multiple of 4)
+        Kahan k[4];
+#pragma unroll 8
         for (int i = i0; i < i1; ++i) {
-            const size_t r = (size_t)srows[r0 + i];
-            if (col < H4)
-                for (int j = 0; j < 4; ++j)
-                    if (col + j < H4) s[j] += dG[r * H4 + col + j];
+            const float4 v = *reinterpret_cast<const float4 *>(dG + (size_t)srows[r0 + i] * H4 + col);
+            k[0].add(v.x); k[1].add(v.y); k[2].add(v.z); k[3].add(v.w);
         }
-        for (int j = 0; j < 4; ++j)
-            if (col + j < H4) part[((size_t)c * A + a) * H4 + col + j] = s[j];
+        *reinterpret_cast<float4 *>(part + ((size_t)c * (A + 1) + a) * H4 + col) = make_float4(k[0].s, k[1].s, k[2].s, k[3].s);
     }
 }
 __global__ void k_bw_arows_fin(int A, int H4, const float *__restrict__ part, float *__restrict__ out) {
-    const size_t n = (size_t)A * H4;
+    const size_t n = (size_t)A * H4, ld = (size_t)(A + 1) * H4;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
         float s = 0.f;
-        for (int c = 0; c < CHUNKS; ++c) s += part[(size_t)c * n + i];
+#pragma unroll
+        for (int c = 0; c < CHUNKS; ++c) s += part[(size_t)c * ld + i];
         out[i] = s;
     }
 }
@@ -363,8 +399,8 @@ size_t wm_bw_ws(const wm_handle *h, int N, int T) {
            + al(NT * H * 4)                                                    // dY
            + al(NT * H4 * 4) + (es == 2 ? al(NT * H4 * 2) : 0)                 // dG
            + 2 * al((size_t)N * H * 4)                                         // dH, dc
-           + al((size_t)COLSUM_CHUNKS * part_cols * 4) + al((size_t)CHUNKS * A * H4 * 4)  // partials
-           + al(NT * 4) + al((size_t)CHUNKS * (A + 1) * 4)                       // rows sorted by action
+           + al((size_t)COLSUM_CHUNKS * part_cols * 4) + al((size_t)CHUNKS * (A + 1) * H4 * 4)  // partials
+           + al(NT * 4) + al((size_t)CHUNKS * (A + 2) * 4)                       // rows sorted by action
            + (es == 4 ? al((size_t)N * 4 * H4 * 2) : 0)                          // fp32: dG_t as bf16 parts
            + al((size_t)(N / 128 + 1) * 4) + 256;                                // row-tile counters
 }
@@ -449,9 +485,9 @@ static cudaError_t bw_run(const wm_handle *h, int N, int TT, const float *z_seq,
     float *dH = (float *)p; p += al((size_t)N * H * 4);
     float *dC = (float *)p; p += al((size_t)N * H * 4);
     float *part = (float *)p; p += al((size_t)COLSUM_CHUNKS * (H4 > M ? H4 : M) * 4);
-    float *apart = (float *)p; p += al((size_t)CHUNKS * A * H4 * 4);
+    float *apart = (float *)p; p += al((size_t)CHUNKS * (A + 1) * H4 * 4);
     int32_t *srows = (int32_t *)p; p += al(NT * 4);
-    int32_t *soff = (int32_t *)p; p += al((size_t)CHUNKS * (A + 1) * 4);
+    int32_t *soff = (int32_t *)p; p += al((size_t)CHUNKS * (A + 2) * 4);
     // fp32: dG_t as [hi | hi | lo], or, in the one-launch recurrence, two steps' rows [hi | lo]
     __nv_bfloat16 *dG3 = bf ? nullptr : (__nv_bfloat16 *)p;
     if (!bf) p += al((size_t)N * 4 * H4 * 2);
@@ -549,13 +585,21 @@ static cudaError_t bw_run(const wm_handle *h, int N, int TT, const float *z_seq,
     if (st != CUBLAS_STATUS_SUCCESS) return cublas_err(st);
     {
         wm_ktime kt(h, WM_KERNEL_BW, s);
-        k_bw_rowsort<<<CHUNKS, 256, (size_t)A * 4, s>>>(NT, A, actions, srows, soff);
-        k_bw_arows<<<dim3(A, CHUNKS), 256, 0, s>>>(NT, A, H4, srows, soff, dG, apart);
+        auto colsum = [&](size_t R, int C, const float *in, float *out) {
+            if (C % 4 == 0) k_bw_colsum4<<<dim3((C + 255) / 256, COLSUM_CHUNKS), 256, 0, s>>>(R, C, in, part);
+            else k_bw_colsum<<<dim3((C + 255) / 256, COLSUM_CHUNKS), 256, 0, s>>>(R, C, in, part);
+            k_bw_colsum_fin<<<(C + 255) / 256, 256, 0, s>>>(C, part, out);
+        };
+        const size_t counts = (size_t)(A + 1) * 4;
+        if (counts > 48 * 1024) {
+            const cudaError_t e = cudaFuncSetAttribute(k_bw_rowsort, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)counts);
+            if (e != cudaSuccess) return e;
+        }
+        k_bw_rowsort<<<CHUNKS, 256, counts, s>>>(NT, A, actions, srows, soff);
+        k_bw_arows<<<dim3(A + 1, CHUNKS), 256, 0, s>>>(NT, A, H4, srows, soff, dG, apart);
         k_bw_arows_fin<<<grid_of((size_t)A * H4), 256, 0, s>>>(A, H4, apart, g.W_lstm + (size_t)Z * H4);
-        k_bw_colsum<<<dim3((H4 + 255) / 256, COLSUM_CHUNKS), 256, 0, s>>>(NT, H4, dG, part);
-        k_bw_colsum_fin<<<(H4 + 255) / 256, 256, 0, s>>>(H4, part, g.b_lstm);
-        k_bw_colsum<<<dim3((M + 255) / 256, COLSUM_CHUNKS), 256, 0, s>>>(NT, M, dMD, part);
-        k_bw_colsum_fin<<<(M + 255) / 256, 256, 0, s>>>(M, part, g.b_mdn);
+        colsum((size_t)CHUNKS * (A + 1), H4, apart, g.b_lstm);
+        colsum(NT, M, dMD, g.b_mdn);
         launches += 7;
     }
     h->last_launches += launches;
