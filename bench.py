@@ -91,8 +91,11 @@ def nll_inputs(cfg: dict, rank: int = 0):
 
 
 def kernel_flops(cls: str, cfg: dict, B: int, T: int, launches: int) -> float:
-    """Algorithmic FLOPs of one launch of a kernel class (its contraction)."""
+    """Algorithmic FLOPs of one launch of a kernel class (its contraction).  launches: of this class
+    in one call (a scoring call's recurrence is one launch or T; its heads are one launch)."""
     Z, A, H, K = cfg["z_dim"], cfg["a_dim"], cfg["h_dim"], cfg["k_mix"]
+    if cfg.get("teacher") and cls in ("tc_gates", "tc_heads"):
+        return 2.0 * B * T * ((Z + H) * 4 * H if cls == "tc_gates" else H * (3 * K * Z + 2)) / max(1, launches)
     if cls in ("fused", "fused_small"):
         return (nll_flops_per_step(cfg) if cfg.get("teacher") else flops_per_env_step(cfg)) * B * T
     if cls == "tc_ctrl":
@@ -304,7 +307,8 @@ def run_nll(args) -> None:
     timed = {k: v for k, v in kt.items() if k in KERNELS}
     dom = max(timed, key=lambda k: timed[k][0])
     dom_ms, dom_n = timed[dom]
-    fl = kernel_flops(dom, tcfg, N, T, dom_n)
+    per_call = max(1, dom_n // args.steps)
+    fl = kernel_flops(dom, tcfg, N, T, per_call)
     achieved = fl / (dom_ms / dom_n / 1e3) / 1e12
     if cfg["precision"] == "bf16" and dom in ("fused", "tc_gates", "tc_heads"):
         bound, peak, psrc = "tensor", peaks["bf16_tflops"], peaks["source"] + " bf16 burst"
@@ -314,6 +318,8 @@ def run_nll(args) -> None:
     else:
         bound, peak, psrc = "alu", fp32_simt_peak_tflops(), "derived: 152 SM x 128 fp32 FMA x 2 FLOP x 2.07 GHz"
     kname, ksrc = KERNELS[dom]
+    if dom == "tc_gates" and per_call == 1:  # the recurrence as one launch
+        kname, ksrc = "k_recur", "wm_recur.cu"
     call_fl = nll_flops_per_step(cfg) * N * T
     roof = {"bound": bound, "achieved": round(achieved, 3), "peak": round(peak, 1), "unit": "TFLOP/s",
             "frac": round(achieved / peak, 5),

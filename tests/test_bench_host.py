@@ -37,6 +37,11 @@ def test_nll_flops_have_no_controller():
     Z, H, K = cfg["z_dim"], cfg["h_dim"], cfg["k_mix"]
     assert bench.nll_flops_per_step(cfg) == 2 * ((Z + H) * 4 * H + H * (3 * K * Z + 2))
     assert bench.kernel_flops("fused", dict(cfg, teacher=True), 10, 3, 1) == bench.nll_flops_per_step(cfg) * 30
+    # a scoring call: the recurrence in one launch or one per step, the heads in one
+    t = dict(cfg, teacher=True)
+    assert bench.kernel_flops("tc_gates", t, 10, 3, 1) == 3 * bench.kernel_flops("tc_gates", t, 10, 3, 3)
+    assert bench.kernel_flops("tc_gates", t, 10, 3, 1) + bench.kernel_flops("tc_heads", t, 10, 3, 1) == \
+        pytest.approx(bench.nll_flops_per_step(cfg) * 30, rel=1e-12)
 
 
 def test_traffic_is_read_only_for_the_captured_source(tmp_path, monkeypatch):
