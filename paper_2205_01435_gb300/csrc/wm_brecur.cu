@@ -83,7 +83,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         tc::fence_mbar_init();
         s_abort = 0;
     }
-    if (warp == 1) tc::tmem_alloc(tc::smem_u32(&tmem_base), UC);
+    if (warp == 1) tc::tmem_alloc(tc::smem_u32(&tmem_base), UC * PARTS);
     tc::fence_before_sync();
     tc::cluster_sync();  // the cluster's barriers exist before any store reaches them
     tc::fence_after_sync();
@@ -148,7 +148,8 @@ __global__ void __launch_bounds__(THREADS, 1)
         bool go = wait(&bar_w, 0);
         int stage = 0;
         uint32_t phase = 0;
-        const uint32_t idesc = tc::idesc_bf16_f32(BM, UC);
+        // (fp32 path: hi meets hi and lo in one MMA, see wm_recur.cu)
+        const uint32_t idesc = tc::idesc_bf16_f32(BM, UC), idesc2 = tc::idesc_bf16_f32(BM, UC * PARTS);
         for (int t = p.T - 2; t >= 0 && go; --t) {
             // (the accumulator is free: dG_{t+1}'s counter covers this CTA's reads of it)
             for (int i0 = 0; i0 < np; i0 += KPS) {
@@ -163,11 +164,8 @@ __global__ void __launch_bounds__(THREADS, 1)
                         const uint64_t da = da0 + h * (A_BYTES >> 4), db = db0 + h * (W_BYTES >> 4);
 #pragma unroll
                         for (int kk = 0; kk < BK / 16; ++kk)
-                            tc::mma_bf16(tm, da + 2 * kk, db + 2 * kk, idesc, (i0 + h > 0 || kk > 0) ? 1u : 0u);
+                            tc::mma_bf16(tm, da + 2 * kk, db + 2 * kk, idesc2, (i0 + h > 0 || kk > 0) ? 1u : 0u);
                         if (F32) {
-#pragma unroll
-                            for (int kk = 0; kk < BK / 16; ++kk)  // hi . lo
-                                tc::mma_bf16(tm, da + 2 * kk, db + (W_BYTES >> 4) + 2 * kk, idesc, 1u);
 #pragma unroll
                             for (int kk = 0; kk < BK / 16; ++kk)  // lo . hi
                                 tc::mma_bf16(tm, da + (A_BYTES >> 4) + 2 * kk, db + 2 * kk, idesc, 1u);
@@ -250,6 +248,13 @@ __global__ void __launch_bounds__(THREADS, 1)
                     tc::tmem_ld_wait();
 #pragma unroll
                     for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(q[j]);
+                    if (F32) {
+                        TC_LD16(ta + UC, q);
+                        TC_LD16(ta + UC + 16, (q + 16));
+                        tc::tmem_ld_wait();
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) v[j] += __uint_as_float(q[j]);
+                    }
                 }
                 tc::fence_before_sync();
 #pragma unroll
@@ -325,7 +330,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     __syncwarp();
     tc::fence_before_sync();
     tc::cluster_sync();  // peers' stores into this CTA's shared memory are done
-    if (warp == 1) tc::tmem_dealloc(tm, UC);
+    if (warp == 1) tc::tmem_dealloc(tm, UC * PARTS);
 }
 
 constexpr size_t SMEM_MAX = 227 * 1024, SMEM_STATIC = 1024;

@@ -81,6 +81,11 @@ __global__ void __launch_bounds__(THREADS, 1)
             const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmWl, wm_recur_args p) {
     constexpr bool F32 = MODE == 2;
     constexpr int PARTS = F32 ? 2 : 1, UT = U / 2, N = 4 * U;
+    // The fp32 path's weights of a block are 2N rows in shared memory, hi above lo: A's hi part meets both
+    // in one MMA of 2N columns, hi.hi and hi.lo side by side (an MMA's time here is its operands' reads,
+    // 128 bytes a cycle: 64 cycles instead of twice 48), lo.hi adds to the first half, and the
+    // epilogue adds the halves.
+    constexpr int NA = N * PARTS;  // columns of an accumulator
     constexpr uint32_t W_BYTES = N * BK * 2;  // one k-block of the CTA's weights
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *smem = reinterpret_cast<unsigned char *>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -114,7 +119,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         tc::fence_mbar_init();
         s_abort = 0;
     }
-    if (warp == 1) tc::tmem_alloc(tc::smem_u32(&tmem_base), 2 * N);
+    if (warp == 1) tc::tmem_alloc(tc::smem_u32(&tmem_base), 2 * NA);
     tc::fence_before_sync();
     tc::cluster_sync();  // the cluster's barriers exist before any copy or arrive reaches them
     tc::fence_after_sync();
@@ -201,12 +206,12 @@ __global__ void __launch_bounds__(THREADS, 1)
             bool go = wait(&bar_w, 0);
             int stage = 0, acc = 0;
             uint32_t phase = 0, acc_phase = 0;
-            const uint32_t idesc = tc::idesc_bf16_f32(BM, N);
+            const uint32_t idesc = tc::idesc_bf16_f32(BM, N), idesc2 = tc::idesc_bf16_f32(BM, NA);
             for (int t = 0; t < T && go; ++t)
                 for (int m = mg; m < p.m_tiles && go; m += p.m_groups) {
                     if (!(go = wait(&bar_acce[acc], acc_phase ^ 1u))) break;
                     tc::fence_after_sync();
-                    const uint32_t d = tm + acc * N;
+                    const uint32_t d = tm + acc * NA;
                     for (int i0 = 0; i0 < np; i0 += KPS) {
                         const int nk = np - i0 < KPS ? np - i0 : KPS;
                         if (!(go = wait(&bar_full[stage], phase))) break;
@@ -219,11 +224,8 @@ __global__ void __launch_bounds__(THREADS, 1)
                                 const uint64_t da = da0 + h * (A_BYTES >> 4), db = db0 + h * (W_BYTES >> 4);
 #pragma unroll
                                 for (int kk = 0; kk < BK / 16; ++kk)
-                                    tc::mma_bf16(d, da + 2 * kk, db + 2 * kk, idesc, (i0 + h > 0 || kk > 0) ? 1u : 0u);
+                                    tc::mma_bf16(d, da + 2 * kk, db + 2 * kk, idesc2, (i0 + h > 0 || kk > 0) ? 1u : 0u);
                                 if (F32) {
-#pragma unroll
-                                    for (int kk = 0; kk < BK / 16; ++kk)  // hi . lo
-                                        tc::mma_bf16(d, da + 2 * kk, db + (W_BYTES >> 4) + 2 * kk, idesc, 1u);
 #pragma unroll
                                     for (int kk = 0; kk < BK / 16; ++kk)  // lo . hi
                                         tc::mma_bf16(d, da + (A_BYTES >> 4) + 2 * kk, db + 2 * kk, idesc, 1u);
@@ -317,7 +319,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                 wait(&bar_accf[acc], acc_phase);
                 __syncwarp();
                 tc::fence_after_sync();
-                const uint32_t ta = tm + ((uint32_t)(32 * quad) << 16) + acc * N + u0;
+                const uint32_t ta = tm + ((uint32_t)(32 * quad) << 16) + acc * NA + u0;
                 float c[UT], h[UT];
                 const size_t o = row * p.H + ug;
                 const int nu = p.H - ug;  // units from ug on that are not padding
@@ -338,6 +340,16 @@ __global__ void __launch_bounds__(THREADS, 1)
 #pragma unroll
                     for (int g = 0; g < 4; ++g) TC_LD8(ta + U * g + j0, v[g]);
                     tc::tmem_ld_wait();
+                    if (F32) {
+#pragma unroll
+                        for (int g = 0; g < 4; ++g) {
+                            uint32_t v2[8];
+                            TC_LD8(ta + N + U * g + j0, v2);
+                            tc::tmem_ld_wait();
+#pragma unroll
+                            for (int j = 0; j < 8; ++j) v[g][j] = __float_as_uint(__uint_as_float(v[g][j]) + __uint_as_float(v2[j]));
+                        }
+                    }
 #pragma unroll
                     for (int j = 0; j < 8; ++j) {
                         float x[4];
@@ -400,7 +412,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     __syncwarp();
     tc::fence_before_sync();
     tc::cluster_sync();  // peers' copies into, and arrives on, this CTA's shared memory are done
-    if (warp == 1) tc::tmem_dealloc(tm, 2 * N);
+    if (warp == 1) tc::tmem_dealloc(tm, 2 * NA);
 }
 
 constexpr size_t SMEM_MAX = 227 * 1024, SMEM_STATIC = 1024;
