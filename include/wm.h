@@ -276,11 +276,13 @@ typedef struct {
  * within 3 * 2^-16 of the fp32 one at worst), all for finite inputs and weights
  * (non-finite values are not propagated as IEEE arithmetic would), and the
  * forward is fp32-accurate (see Precision above).  The forward runs on the
- * kernel family wm_mdn_nll would pick; the batched GEMMs of the backward
- * (gate activations over all N*T rows, the heads' and the recurrent input
- * gradients, the weight gradients) are cuBLAS calls, the rest (the mixture
- * NLL's gradient, the cell's backward step, the action-row and bias sums) are
- * the library's kernels.  Deterministic: every reduction has a fixed order.
+ * kernel family wm_mdn_nll would pick; the batched GEMMs of the backward (the
+ * heads' input gradient, the weight gradients, and the gate pre-activations
+ * where the forward did not leave them) are cuBLAS calls, the rest (the mixture
+ * NLL's gradient, the recurrence, the action-row and bias sums) are the
+ * library's kernels, but for sizes the one-launch recurrence does not take
+ * (H % 64 != 0, or more row tiles than two launches hold), whose recurrent
+ * input gradient is a cuBLAS call per step.  Deterministic: every reduction has a fixed order.
  * Returns WM_ERR_UNSUPPORTED for hierarchical models. */
 wm_status wm_mdn_nll_backward(wm_handle *h, int N, int T, const float *z_seq, const int32_t *actions,
                               const int32_t *lengths, float *nll, const wm_grads *grads,

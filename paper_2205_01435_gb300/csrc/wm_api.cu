@@ -271,14 +271,14 @@ cudaError_t pack_step(wm_handle *h, const wm_weights *w) {
 // order alone moves it by 5 to 10% within 25 steps (rel. 2-norm of z, rewards, h; 1% at 4 steps,
 // and under 1% at H <= 512), and a small batch's results stay what they were.  fused_ok / tc_ok:
 // whether this call's options allow those families; steps: of a rollout (0: a scoring call).
-int pick_path(const wm_handle *h, int B, bool fused_ok = true, bool tc_ok = true, int steps = 0) {
+int pick_path(const wm_handle *h, int B, bool fused_ok = true, bool tc_ok = true, int steps = 0, bool pad_ok = true) {
     const int p = h->cfg.path;
     if (p != WM_PATH_AUTO) return p;
     const bool fu = fused_ok && wm_fused_supported(h, B), tc = tc_ok && wm_tc_supported(h);
     if (fu && B <= 2048) return WM_PATH_FUSED;
     if (tc && (B >= 256 || h->cfg.precision == WM_FP32)) return WM_PATH_TENSOR;
     if (fu) return WM_PATH_FUSED;
-    if (tc_ok && wm_tc_auto_ok(h) && (h->cfg.h_dim <= 512 || steps <= 4)) return WM_PATH_TENSOR;
+    if (tc_ok && pad_ok && wm_tc_auto_ok(h) && (h->cfg.h_dim <= 512 || steps <= 4)) return WM_PATH_TENSOR;
     return WM_PATH_STEPWISE;
 }
 
@@ -288,13 +288,15 @@ int pick_path(const wm_handle *h, int B, bool fused_ok = true, bool tc_ok = true
 // x 24 183 / 110, x 100 723 / 407, 1500 x 24 264 / 166; at 7, 45, 40, 3: 16 x 4 27 / 36, x 24 121 / 96;
 // at 85, 168, 94, 7: 271 x 24 1087 / 139.  The crossing lies between 6 and 10 steps.  In a training
 // step of the smallest models and batches the fused member's outputs cost less: 100 x 24 at 7, 45, 40, 3
-// 384 / 392, 600 x 24 732 / 475.
+// 384 / 392, 600 x 24 732 / 475.  The tensor family holds the operand rows of all steps: a call that
+// another family can run on N rows' scratch goes to it when those pass 8 GB.
 int pick_score_path(const wm_handle *h, int N, int T, bool train) {
-    if (h->cfg.path == WM_PATH_AUTO && wm_tc_auto_ok(h) && wm_tc_scores_in_one(h, N, T)) {
+    const bool fits = wm_tc_auto_ok(h) && wm_tc_ws(h, N, T) <= (size_t)8 << 30;
+    if (h->cfg.path == WM_PATH_AUTO && fits && wm_tc_scores_in_one(h, N, T)) {
         const bool kept = T < 12 || (train && h->cfg.h_dim < 64 && N <= 400);
         if (!(kept && wm_fused_supported(h, N))) return WM_PATH_TENSOR;
     }
-    return pick_path(h, N);
+    return pick_path(h, N, true, true, 0, fits);
 }
 
 template <class T>

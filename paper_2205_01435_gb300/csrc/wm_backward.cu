@@ -6,21 +6,26 @@
 // the library.  Everything that does not depend on the recurrence is batched over all
 // N T rows:
 //   forward      the teacher-forced pass of the kernel family wm_mdn_nll picks, keeping
-//                h_t, c_t and the head outputs of every row
-//   X, Y         the GEMM operands of every row, X = [op(z_t); op(h_{t-1})], Y = op(h_t)
-//   gates        G = X W_zh (one GEMM) + b + W_a[a_t], then sigma / tanh  (k_bw_gates)
-//   dMD          d NLL / d [logit | mu | log sigma] of every counted row     (k_bw_mdn)
+//                h_t and c_t of every row
+//   X, Y         the GEMM operands of every row, X = [op(z_t); op(h_{t-1})], Y = op(h_t): the
+//                forward's own operand rows where it leaves them, else built (k_bw_build)
+//   gates        the pre-activations G = X W_zh + b + W_a[a_t]: left by the forward's one-launch
+//                recurrence, else one GEMM and, with sigma / tanh, k_bw_gates
+//   dMD          d NLL / d [logit | mu | log sigma] of every counted row: formed by the
+//                tensor family's head GEMM, else from the head outputs          (k_bw_mdn)
 //   dY           dMD W_mdn^T (one GEMM): the heads' share of d loss / d h_t
-// then the recurrence, t = T-1 .. 0:
+// then the recurrence, t = T-1 .. 0, in one launch (wm_brecur.cu) or per step:
 //   dG_t         the cell's backward step from dY_t + dH and the carried dc  (k_bw_cell)
 //   dH           dG_t W_h^T (one GEMM on N rows): d loss / d h_{t-1}
 // and the weight gradients, batched again:
 //   dW_z, dW_h   X^T dG (two GEMMs writing the z and h rows of the output)
 //   dW_a         per action, the sum of the dG rows that took it          (k_bw_arows)
-//   dW_mdn       Y^T dMD (one GEMM);  db_lstm, db_mdn  column sums          (k_bw_colsum)
+//   dW_mdn       Y^T dMD (one GEMM)
+//   db_lstm      the sum of dW_a's buckets, one of them for rows without an action
+//   db_mdn       column sums                                               (k_bw_colsum4)
 // The plain GEMMs are cuBLAS calls (bf16 operands and fp32 accumulation on the bf16 path;
-// on the fp32 path the library's fp32 emulation, and for the recurrence's dH one bf16 GEMM
-// over the operands' hi and lo parts, see k_bw_split3); the rest are the kernels below.
+// on the fp32 path the library's fp32 emulation, and for the recurrence's dH bf16 products
+// of the operands' hi and lo parts, see k_bw_split3); the rest are the kernels below.
 // Every reduction has a fixed order, so results are bit-reproducible.
 #include <cublas_v2.h>
 #include <cuda.h>

@@ -18,8 +18,10 @@
 // A step (512 sequences, H = 512, clock64 stamps of one CTA, cycles at about 2 GHz): counter to
 // accumulator 3.9K (operands land at the rate of one 16 KB part per 215 cycles after 1.2K, then
 // the last MMAs), cell 0.95K, stores to the counter's release 1.9K, release to the next step's
-// acquire 1.2K: 8K, 4 us.  A call of 512 x 128 takes 0.69 ms, 1.28 as one launch per step; on the
-// fp32 path (two parts per block through a ring that holds 4) 1.27 ms, 2.38 before.
+// acquire 1.2K: 8K, 4 us.  A call of 512 x 128 takes 0.67 ms, 1.28 as one launch per step; on the
+// fp32 path (two parts per block through a ring that holds 4; paced by the issuer's MMAs) 1.21 ms,
+// 2.38 before.  Up to RECUR_MAX_GROUPS row tiles per CTA this stays ahead of one launch per step
+// (24 steps at H = 512: 1024 / 2048 sequences 221 / 341 us against 288 / 432).
 // Every CTA waits for others: the launch is cooperative (all CTAs resident), every wait is
 // bounded, and a CTA that gives up records WM_ERR_TIMEOUT, skips its remaining work and exits.
 //

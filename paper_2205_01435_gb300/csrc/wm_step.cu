@@ -39,8 +39,8 @@ __device__ __forceinline__ uint64_t both(float v) {
 // rows come in pairs, two FMAs per instruction; the next k-block's elements are loaded into registers
 // under the current one's FMAs and go to the other half of a double buffer, one barrier per block
 // (of GBK: the small tiles, which have few FMAs to hide a load behind, take long ones).
-// (64 x 64 tiles of scalar FMAs with both loads and a second barrier in front of them: 174 us per step
-// of 495 episodes at Z, A, H, K = 56, 87, 426, 8.)
+// (A step of 495 episodes at Z, A, H, K = 56, 87, 426, 8: 87 us; 174 with 64 x 64 tiles of scalar FMAs
+// and both loads and a second barrier in front of them.  16 at 128, 512, 1024, 8: 72 us, 256.)
 template <bool ROUND, int BM, int BN, int TM, int TN, int GBK>
 __global__ void __launch_bounds__((BM / TM) * (BN / TN)) k_gemm(int M, int N, int K1, int K2,
                                                                const float *__restrict__ A1, long lda1,
@@ -509,7 +509,9 @@ void launch_gemm(const wm_handle *hd, bool round, int M, int N, int K1, int K2, 
                  const float *A2, long lda2, const float *W, long ldw, const float *bias, float *C, long ldc,
                  cudaStream_t s) {
     wm_ktime kt(hd, WM_KERNEL_STEP_GEMM, s);
-    // the largest tile that gives the 152 SMs a block each or more; a small batch takes low tiles
+    // the largest tile that gives the 152 SMs a block each or more; a small batch takes low tiles (20
+    // steps at H = 300: 1 episode 1705 us on the 64 x 64 tile, 844 on 16 x 32 with k-blocks of 16, 659
+    // with 64; 100 episodes 2351 on 64 x 64, 767 on 32 x 64)
     auto blocks = [&](int bm, int bn) { return (long)((M + bm - 1) / bm) * ((N + bn - 1) / bn); };
     if (M > 64 && blocks(128, 128) >= 2 * 152)
         launch_tile<128, 128, 8, 8, 16>(round, M, N, K1, K2, A1, lda1, A2, lda2, W, ldw, bias, C, ldc, s);

@@ -1444,8 +1444,8 @@ __global__ void k_tc_finish(int B, int H, int Hp, const float *h32, const float 
 // ---------------------------------------------------------------------------
 // Batched teacher-forced scoring: the operand rows of all T + 1 frames are staged at once
 // (frame f, sequence n at row f N + n: z part from z_seq; the h part of frame f + 1 is
-// written by step f's gate epilogue), the recurrence runs one gate GEMM per step, and one
-// head GEMM then scores all N T (step, sequence) rows.
+// written by step f), the recurrence runs as one launch (wm_recur.cu) or as one gate GEMM per
+// step, and one head GEMM then scores all N T (step, sequence) rows.
 __global__ void k_tc_frames(int N, int T, int Z, int Zp, int KX, const float *__restrict__ z_seq,
                             __nv_bfloat16 *__restrict__ x, __nv_bfloat16 *__restrict__ x_lo) {
     const size_t n = (size_t)T * N * Zp;  // frames 1..T (frame 0 is the init kernel's); padded columns 0
