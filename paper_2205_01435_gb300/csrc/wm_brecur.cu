@@ -351,7 +351,8 @@ void set_attrs(cudaLaunchConfig_t &lc, cudaLaunchAttribute (&at)[2], size_t smem
 
 template <bool F32>
 int resident_clusters() {
-    static int known = 0;
+    static int per_device[WM_MAX_DEVICES] = {};  // (the shared-memory limit is a device's, too)
+    int &known = per_device[wm_device_slot()];
     if (!known) {
         const size_t smem = SMEM_MAX - SMEM_STATIC;
         cudaLaunchConfig_t lc = {};

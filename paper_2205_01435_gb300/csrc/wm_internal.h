@@ -179,6 +179,14 @@ struct wm_handle {
     size_t bws_bytes = 0;
 };
 
+// The current device's place in tables of per-device launch attributes.
+enum { WM_MAX_DEVICES = 64 };
+inline int wm_device_slot() {
+    int d = 0;
+    cudaGetDevice(&d);
+    return d >= 0 && d < WM_MAX_DEVICES ? d : 0;
+}
+
 // Brackets the kernel launches of its scope with CUDA events on stream s when
 // timing is on for h; does nothing otherwise.
 class wm_ktime {

@@ -446,8 +446,8 @@ kern_t kernel_of(int mode, int units, int kps) {
 
 // CTAs that can be resident at once in clusters of `cluster` (one per SM)
 int resident(int mode, int units, int kps, int cluster) {
-    static int known[3][2][2][3] = {};
-    int &n = known[mode][units >> 5][kps - 2][cluster >> 1];
+    static int known[WM_MAX_DEVICES][3][2][2][3] = {};  // (the shared-memory limit is a device's, too)
+    int &n = known[wm_device_slot()][mode][units >> 5][kps - 2][cluster >> 1];
     if (!n) {
         const kern_t kern = kernel_of(mode, units, kps);
         const size_t smem = SMEM_MAX - SMEM_STATIC;

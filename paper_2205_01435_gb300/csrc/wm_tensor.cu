@@ -1796,7 +1796,9 @@ cudaError_t launch_gemm(const OpMaps &op, const CUtensorMap &mc, const CUtensorM
     at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[1].val.programmaticStreamSerializationAllowed = pdl ? 1 : 0;
     lc.numAttrs = 2;
-    static int max_pairs = 0;  // pairs resident at once (the grid is persistent)
+    // pairs resident at once (the grid is persistent), per device, as is the shared-memory limit
+    static int per_device[WM_MAX_DEVICES] = {};
+    int &max_pairs = per_device[wm_device_slot()];
     if (!max_pairs) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
