@@ -802,13 +802,16 @@ struct EpiGatesT {
 };
 
 using EpiGates = EpiGatesT<0>;
-using EpiGates2 = EpiGatesT<1>;
 using EpiGates32 = EpiGatesT<2>;
 using EpiGatesN = EpiGatesT<0, 32>;  // 128-column tiles (few row tiles)
 using EpiGates32N = EpiGatesT<2, 32>;  // the same, fp32 path (teacher-forced scoring)
 using EpiGatesA = EpiGatesT<0, 64, true>;    // accurate nonlinearities, bf16 path
-using EpiGates2A = EpiGatesT<1, 64, true>;
 using EpiGatesNA = EpiGatesT<0, 32, true>;
+// Two action rows (hierarchical actions) take 128-column tiles at every size: with 256-column
+// ones the second row's words make the epilogue spill.  16384 x 8 steps, H = 1024: gates
+// 161 -> 130 us a step, call 2550 -> 2328 us; 64 to 16384 rows, H = 512 and 1024: 1-13% less.
+using EpiGates2N = EpiGatesT<1, 32>;
+using EpiGates2NA = EpiGatesT<1, 32, true>;
 
 // ---- head epilogue: dims_per_tile latent dims, DS columns each; reward / done -----
 // Before the accumulator wait, the quadrant's 128 threads make the tile's random draws:
@@ -2196,10 +2199,11 @@ static cudaError_t tc_run(const wm_handle *h, int teacher, const wm_rollout_dev 
     // a call at B = 8192), but made the long launches of B = 65536 3% slower: on below 32768.
     const bool pdl = B < 32768;
     // 128-column gate tiles when 256-column ones would leave most CTA pairs idle: few row
-    // tiles, or compacted live rows (bf16, flat actions); on the fp32 path, scoring
+    // tiles, or compacted live rows (bf16); always for hierarchical actions (EpiGates2N); on
+    // the fp32 path, scoring
     const int pairs = T.sms / 2;
-    const bool narrow = !hier && T.wg_n &&
-                        (f32 ? teacher && T.wg_n_lo : (compact || teacher || m_tiles * (Hp / 64) < pairs));
+    const bool narrow = T.wg_n &&
+                        (f32 ? teacher && T.wg_n_lo : (compact || teacher || hier || m_tiles * (Hp / 64) < pairs));
     CUtensorMap mwgn, mwgnl, mxsn[2];
     if (narrow && (!make_map(&mwgn, T.wg_n, 4 * Hp, KX, 64) || !make_map_x32(&mxsn[0], w.x[0], B, KX) ||
                    !make_map_x32(&mxsn[1], w.x[1], B, KX)))
@@ -2479,14 +2483,14 @@ static cudaError_t tc_run(const wm_handle *h, int teacher, const wm_rollout_dev 
             g2n.n_tiles = Hp / 32;
             const OpMaps opn{&mx[xa], &mwgn, &mx[xa], &mwgn};
             wm_ktime kt(h, WM_KERNEL_TC_GATES, s);
-            e = acc ? launch_gemm<128, 1, 3, EpiGatesNA, 2>(opn, mC, mxsn[xn], mxsn[xn], g2n, gio_n, T.sms, s, pdl)
-                    : launch_gemm<128, 1, 3, EpiGatesN, 2>(opn, mC, mxsn[xn], mxsn[xn], g2n, gio_n, T.sms, s, pdl);
+            if (hier && acc) e = launch_gemm<128, 1, 3, EpiGates2NA, 2>(opn, mC, mxsn[xn], mxsn[xn], g2n, gio_n, T.sms, s, pdl);
+            else if (hier) e = launch_gemm<128, 1, 3, EpiGates2N, 2>(opn, mC, mxsn[xn], mxsn[xn], g2n, gio_n, T.sms, s, pdl);
+            else if (acc) e = launch_gemm<128, 1, 3, EpiGatesNA, 2>(opn, mC, mxsn[xn], mxsn[xn], g2n, gio_n, T.sms, s, pdl);
+            else e = launch_gemm<128, 1, 3, EpiGatesN, 2>(opn, mC, mxsn[xn], mxsn[xn], g2n, gio_n, T.sms, s, pdl);
         } else {
             wm_ktime kt(h, WM_KERNEL_TC_GATES, s);
             if (f32) e = launch_gemm<256, 1, 2, EpiGates32, 2, 3>(opg, mC, mxs[xn], mxsl[xn], g2, io, T.sms, s, pdl);
-            else if (hier && acc) e = launch_gemm<256, 1, 2, EpiGates2A, 2>(opg, mC, mxs[xn], mxs[xn], g2, io, T.sms, s, pdl);
             else if (acc) e = launch_gemm<256, 1, 2, EpiGatesA, 2>(opg, mC, mxs[xn], mxs[xn], g2, io, T.sms, s, pdl);
-            else if (hier) e = launch_gemm<256, 1, 2, EpiGates2, 2>(opg, mC, mxs[xn], mxs[xn], g2, io, T.sms, s, pdl);
             else e = launch_gemm<256, 1, 2, EpiGates, 2>(opg, mC, mxs[xn], mxs[xn], g2, io, T.sms, s, pdl);
         }
         ++launches;

@@ -67,6 +67,23 @@ def test_rollout(wm, orc, Z, A, H, K, B, flags):
         assert torch.equal(gh[k], g[k].cpu()), k
 
 
+@pytest.mark.parametrize("H,B", [(256, 9985), (512, 5001)])
+def test_hierarchical_gates_over_many_tiles(wm, H, B):
+    """More gate tiles than CTA pairs, a ragged last one: the bits of the same episodes in a
+    batch of one tile per pair (which the oracle checks)."""
+    cfg, T, NX = _cfg(32, 128, H, 5, ctrl_sample=1, n_xfers=32), 3, 32
+    z0, (xm, lm) = synth.z0(B, 32, seed=35), synth.hier_masks(T, B, NX, 96, 0.5, seed=35)
+    m = wm.WorldModel(cfg, synth.weights(cfg, seed=35))
+    g = m.rollout(_cuda(z0), T, mask=_cuda(xm), loc_mask=_cuda(lm), want_seq=True)
+    for first in (0, B - 300):
+        r = slice(first, first + 300)
+        s = m.rollout(_cuda(z0[r]), T, mask=_cuda(xm[:, r]), loc_mask=_cuda(lm[:, r]), episode_offset=first, want_seq=True)
+        assert m.last_path == "tensor"
+        for k in ("z", "h_seq", "rewards"):
+            assert torch.equal(s[k], g[k][:, r]), k
+        assert torch.equal(s["c_final"], g["c_final"][r])
+
+
 @pytest.mark.parametrize("Z,A,H,K,N,T", [(5, 45, 333, 3, 700, 3), (50, 101, 300, 6, 600, 5), (64, 256, 512, 5, 60, 4)])
 def test_scoring_and_training(wm, orc, Z, A, H, K, N, T):
     cfg = _cfg(Z, A, H, K)
