@@ -2077,6 +2077,25 @@ static bool accurate(const wm_handle *h, int B, int teacher) {
            (h->cfg.path == WM_PATH_AUTO && (B < 256 || (teacher && wm_small_supported(h, B))));
 }
 
+// Whether a rollout's gate GEMM takes 128-column tiles: `tiles` 256-column ones over `pairs`
+// CTA pairs leave the last wave at most half full (rest), which halves of tiles fill better.
+// A wave of two halves costs 2-12% more than one whole tile (each half reads its rows of x
+// again), so the rule ends after a number of whole waves:
+// bf16, 8 steps, whole -> halves: 1280 x H 1024 (80 tiles) 460 -> 425 us, 2560 (160) 575 -> 542,
+// 4096 (256) 694 -> 668, 8192 (512) 1045 -> 1060; 2560 x H 512 (80) 309 -> 301, 5632 (176)
+// 432 -> 432, 8192 (256) 495 -> 513; padded 7936 x H 300 (155) 490 -> 478, 11776 (230) 601 -> 600;
+// 8 x 768 x H 256 (96) 259 -> 255, 8 x 1280 (160) 353 -> 357.
+// On the fp32 path the 256-column epilogue spills, which weighs most where the contraction is
+// short: 65536 x H 256 (1024) 2282 -> 2179 us, 1000 x H 512 (32) 437 -> 362, 8192 (256) 896 -> 854,
+// 10000 (320) 1080 -> 1043, 12000 (376) 1154 -> 1168, 16384 (512) 1467 -> 1506; 6000 x H 1024 (384)
+// 2174 -> 2108, 8192 (512) 2527 -> 2580.
+static bool narrow_gates(bool f32, bool acc, int Hp, int tiles, int pairs) {
+    const int full = tiles / pairs, rest = tiles % pairs;
+    const bool half = rest > 0 && 2 * rest <= pairs;
+    if (f32) return Hp <= 256 || full < 4 || (half && full <= 5);
+    return full < 1 || (half && full <= (Hp >= 768 ? 3 : acc ? 2 : 1));
+}
+
 // How a scoring call's recurrence runs as one launch; false: one launch per step.
 static bool one_launch(const wm_handle *h, int N, int T, wm_recur_args *a, int *mode) {
     const wm_tc_weights &w = h->tc;
@@ -2198,17 +2217,16 @@ static cudaError_t tc_run(const wm_handle *h, int teacher, const wm_rollout_dev 
     // Programmatic dependent launch hides the ~4 us between consecutive launches (a fifth of
     // a call at B = 8192), but made the long launches of B = 65536 3% slower: on below 32768.
     const bool pdl = B < 32768;
-    // 128-column gate tiles when 256-column ones would leave most CTA pairs idle: few row
-    // tiles, or compacted live rows (bf16); always for hierarchical actions (EpiGates2N); on
-    // the fp32 path, scoring
-    const int pairs = T.sms / 2;
-    const bool narrow = T.wg_n &&
-                        (f32 ? teacher && T.wg_n_lo : (compact || teacher || hier || m_tiles * (Hp / 64) < pairs));
-    CUtensorMap mwgn, mwgnl, mxsn[2];
+    // 128-column gate tiles for compacted live rows, scoring, hierarchical actions
+    // (EpiGates2N), and as narrow_gates says for the rest
+    const bool narrow = compact || teacher || hier || narrow_gates(f32, acc, Hp, m_tiles * (Hp / 64), T.sms / 2);
+    CUtensorMap mwgn, mwgnl, mxsn[2], mxsnl[2];
     if (narrow && (!make_map(&mwgn, T.wg_n, 4 * Hp, KX, 64) || !make_map_x32(&mxsn[0], w.x[0], B, KX) ||
                    !make_map_x32(&mxsn[1], w.x[1], B, KX)))
         return cudaErrorInvalidValue;
-    if (narrow && f32 && !make_map(&mwgnl, T.wg_n_lo, 4 * Hp, KX, 64)) return cudaErrorInvalidValue;
+    if (f32 && (!make_map(&mwgnl, T.wg_n_lo, 4 * Hp, KX, 64) || !make_map_x32(&mxsnl[0], w.x_lo[0], B, KX) ||
+                !make_map_x32(&mxsnl[1], w.x_lo[1], B, KX)))
+        return cudaErrorInvalidValue;
     StepIO gio_n;  // the gate launches' parameters with the 128-column packing
     if (teacher) {  // batched scoring: the recurrence step by step, then one head GEMM
         const size_t fr = (size_t)B * KX;  // elements of one frame of operand rows
@@ -2253,46 +2271,29 @@ static cudaError_t tc_run(const wm_handle *h, int teacher, const wm_rollout_dev 
             io.t = t;
             io.step = (uint32_t)t;
             // this step's operand rows (frame t) and where h' goes (frame t + 1)
-            CUtensorMap ma, mal, ms, msl;
-            if (!make_map(&ma, w.xall + t * fr, B, KX, BM) || !make_map(&ms, w.xall + (t + 1) * fr, B, KX, 32))
+            CUtensorMap ma, mal, msn, msnl;
+            if (!make_map(&ma, w.xall + t * fr, B, KX, BM) || !make_map_x32(&msn, w.xall + (t + 1) * fr, B, KX))
                 return cudaErrorInvalidValue;
-            if (f32) {
-                if (!make_map(&mal, w.xall_lo + t * fr, B, KX, BM) || !make_map(&msl, w.xall_lo + (t + 1) * fr, B, KX, 32))
-                    return cudaErrorInvalidValue;
-            } else {
-                mal = ma;
-                msl = ms;
-            }
-            GemmGrid g2{m_tiles, Hp / 64, (KX + BK - 1) / BK, 0, h->status};
+            if (f32 && (!make_map(&mal, w.xall_lo + t * fr, B, KX, BM) ||
+                        !make_map_x32(&msnl, w.xall_lo + (t + 1) * fr, B, KX)))
+                return cudaErrorInvalidValue;
+            GemmGrid g2n{m_tiles, Hp / 32, (KX + BK - 1) / BK, 0, h->status};
             if (t == 0) {  // an injected wait (wm_inject_wait_timeout) goes to the first GEMM
-                g2.test_wait = h->test_wait;
+                g2n.test_wait = h->test_wait;
                 h->test_wait = 0;
             }
-            const OpMaps opg{&ma, &mwg, &mal, &mwgl};
-            if (narrow) {
-                CUtensorMap msn, msnl;
-                if (!make_map_x32(&msn, w.xall + (t + 1) * fr, B, KX)) return cudaErrorInvalidValue;
-                if (f32 && !make_map_x32(&msnl, w.xall_lo + (t + 1) * fr, B, KX)) return cudaErrorInvalidValue;
-                gio_n = io;
-                gio_n.wa = (const __nv_bfloat16 *)T.wa_n;
-                gio_n.b_gate = T.bg_n;
-                GemmGrid g2n = g2;
-                g2n.n_tiles = Hp / 32;
-                wm_ktime kt(h, WM_KERNEL_TC_GATES, s);
-                if (f32) {
-                    gio_n.wa_lo = (const __nv_bfloat16 *)T.wa_n_lo;
-                    const OpMaps opn{&ma, &mwgn, &mal, &mwgnl};
-                    e = launch_gemm<128, 1, 3, EpiGates32N, 2, 3>(opn, mc, msn, msnl, g2n, gio_n, T.sms, s, pdl);
-                } else {
-                    const OpMaps opn{&ma, &mwgn, &ma, &mwgn};
-                    e = acc ? launch_gemm<128, 1, 3, EpiGatesNA, 2>(opn, mc, msn, msn, g2n, gio_n, T.sms, s, pdl)
-                            : launch_gemm<128, 1, 3, EpiGatesN, 2>(opn, mc, msn, msn, g2n, gio_n, T.sms, s, pdl);
-                }
+            gio_n = io;
+            gio_n.wa = (const __nv_bfloat16 *)T.wa_n;
+            gio_n.b_gate = T.bg_n;
+            wm_ktime kt(h, WM_KERNEL_TC_GATES, s);
+            if (f32) {
+                gio_n.wa_lo = (const __nv_bfloat16 *)T.wa_n_lo;
+                const OpMaps opn{&ma, &mwgn, &mal, &mwgnl};
+                e = launch_gemm<128, 1, 3, EpiGates32N, 2, 3>(opn, mc, msn, msnl, g2n, gio_n, T.sms, s, pdl);
             } else {
-                wm_ktime kt(h, WM_KERNEL_TC_GATES, s);
-                if (f32) e = launch_gemm<256, 1, 2, EpiGates32, 2, 3>(opg, mc, ms, msl, g2, io, T.sms, s, pdl);
-                else if (acc) e = launch_gemm<256, 1, 2, EpiGatesA, 2>(opg, mc, ms, ms, g2, io, T.sms, s, pdl);
-                else e = launch_gemm<256, 1, 2, EpiGates, 2>(opg, mc, ms, ms, g2, io, T.sms, s, pdl);
+                const OpMaps opn{&ma, &mwgn, &ma, &mwgn};
+                e = acc ? launch_gemm<128, 1, 3, EpiGatesNA, 2>(opn, mc, msn, msn, g2n, gio_n, T.sms, s, pdl)
+                        : launch_gemm<128, 1, 3, EpiGatesN, 2>(opn, mc, msn, msn, g2n, gio_n, T.sms, s, pdl);
             }
             ++launches;
         }
@@ -2481,9 +2482,11 @@ static cudaError_t tc_run(const wm_handle *h, int teacher, const wm_rollout_dev 
             gio_n.b_gate = T.bg_n;
             GemmGrid g2n = g2;
             g2n.n_tiles = Hp / 32;
-            const OpMaps opn{&mx[xa], &mwgn, &mx[xa], &mwgn};
+            gio_n.wa_lo = (const __nv_bfloat16 *)T.wa_n_lo;
+            const OpMaps opn{&mx[xa], &mwgn, f32 ? &mxl[xa] : &mx[xa], f32 ? &mwgnl : &mwgn};
             wm_ktime kt(h, WM_KERNEL_TC_GATES, s);
-            if (hier && acc) e = launch_gemm<128, 1, 3, EpiGates2NA, 2>(opn, mC, mxsn[xn], mxsn[xn], g2n, gio_n, T.sms, s, pdl);
+            if (f32) e = launch_gemm<128, 1, 3, EpiGates32N, 2, 3>(opn, mC, mxsn[xn], mxsnl[xn], g2n, gio_n, T.sms, s, pdl);
+            else if (hier && acc) e = launch_gemm<128, 1, 3, EpiGates2NA, 2>(opn, mC, mxsn[xn], mxsn[xn], g2n, gio_n, T.sms, s, pdl);
             else if (hier) e = launch_gemm<128, 1, 3, EpiGates2N, 2>(opn, mC, mxsn[xn], mxsn[xn], g2n, gio_n, T.sms, s, pdl);
             else if (acc) e = launch_gemm<128, 1, 3, EpiGatesNA, 2>(opn, mC, mxsn[xn], mxsn[xn], g2n, gio_n, T.sms, s, pdl);
             else e = launch_gemm<128, 1, 3, EpiGatesN, 2>(opn, mC, mxsn[xn], mxsn[xn], g2n, gio_n, T.sms, s, pdl);

@@ -67,17 +67,24 @@ def test_rollout(wm, orc, Z, A, H, K, B, flags):
         assert torch.equal(gh[k], g[k].cpu()), k
 
 
-@pytest.mark.parametrize("H,B", [(256, 9985), (512, 5001)])
-def test_hierarchical_gates_over_many_tiles(wm, H, B):
-    """More gate tiles than CTA pairs, a ragged last one: the bits of the same episodes in a
-    batch of one tile per pair (which the oracle checks)."""
-    cfg, T, NX = _cfg(32, 128, H, 5, ctrl_sample=1, n_xfers=32), 3, 32
-    z0, (xm, lm) = synth.z0(B, 32, seed=35), synth.hier_masks(T, B, NX, 96, 0.5, seed=35)
+# more gate tiles of 256 columns than 76 CTA pairs: two action rows; bf16 with a last wave half full
+# (80, 114) and just over (115); fp32 over the whole range of its rule (40, 320, 330, 512)
+@pytest.mark.parametrize("H,B,precision,NX", [
+    (256, 9985, "bf16", 32), (512, 5001, "bf16", 32), (512, 2500, "bf16", 0), (1216, 1281, "bf16", 0),
+    (320, 5800, "bf16", 0), (1024, 2500, "bf16", 0), (512, 1100, "fp32", 0), (256, 20001, "fp32", 0),
+    (512, 10200, "fp32", 0), (704, 7600, "fp32", 0), (512, 16300, "fp32", 0)])
+def test_gates_over_many_tiles(wm, H, B, precision, NX):
+    """The bits of the same episodes in a batch of few tiles (which the oracle checks)."""
+    cfg, T = dict(_cfg(32, 128, H, 5, ctrl_sample=1, n_xfers=NX), precision=precision), 3
+    z0, x = synth.z0(B, 32, seed=35), {}
+    if NX:
+        x["mask"], x["loc_mask"] = synth.hier_masks(T, B, NX, 128 - NX, 0.5, seed=35)
     m = wm.WorldModel(cfg, synth.weights(cfg, seed=35))
-    g = m.rollout(_cuda(z0), T, mask=_cuda(xm), loc_mask=_cuda(lm), want_seq=True)
+    g = m.rollout(_cuda(z0), T, want_seq=True, want_logp=True, **{k: _cuda(v) for k, v in x.items()})
     for first in (0, B - 300):
         r = slice(first, first + 300)
-        s = m.rollout(_cuda(z0[r]), T, mask=_cuda(xm[:, r]), loc_mask=_cuda(lm[:, r]), episode_offset=first, want_seq=True)
+        s = m.rollout(_cuda(z0[r]), T, episode_offset=first, want_seq=True, want_logp=True,
+                      **{k: _cuda(v[:, r]) for k, v in x.items()})
         assert m.last_path == "tensor"
         for k in ("z", "h_seq", "rewards"):
             assert torch.equal(s[k], g[k][:, r]), k
