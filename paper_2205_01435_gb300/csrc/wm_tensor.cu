@@ -1783,7 +1783,7 @@ struct OpMaps {
 
 template <int BN, int NSUB, int STAGES, class Epi, int KPS = 1, int NP = 1>
 cudaError_t launch_gemm(const OpMaps &op, const CUtensorMap &mc, const CUtensorMap &mxs, const CUtensorMap &mxs2,
-                        GemmGrid g, const StepIO &io, int sms, cudaStream_t s, bool pdl) {
+                        GemmGrid g, const StepIO &io, int sms, cudaStream_t s) {
     const size_t smem = gemm_smem<BN, NSUB, STAGES, Epi, KPS>();
     auto kern = k_tc_gemm<BN, NSUB, STAGES, Epi, KPS, NP>;
     cudaLaunchConfig_t lc = {};
@@ -1796,8 +1796,11 @@ cudaError_t launch_gemm(const OpMaps &op, const CUtensorMap &mc, const CUtensorM
     lc.dynamicSmemBytes = smem;
     lc.stream = s;
     lc.attrs = at;
+    // Programmatic dependent launch hides the ~4 us between consecutive launches: a fifth of a
+    // call at B = 8192, and with the warps' elected issue also at the largest batches (65536
+    // rows: H = 1024 0.2-1.4%, H = 512 16 steps 5370 -> 5251 us; 33000 2945 -> 2807).
     at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[1].val.programmaticStreamSerializationAllowed = pdl ? 1 : 0;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     lc.numAttrs = 2;
     // pairs resident at once (the grid is persistent), per device, as is the shared-memory limit
     static int per_device[WM_MAX_DEVICES] = {};
@@ -2214,9 +2217,6 @@ static cudaError_t tc_run(const wm_handle *h, int teacher, const wm_rollout_dev 
     }
     io.wa_lo = (const __nv_bfloat16 *)T.wa_lo;
     const int m_tiles = (B + 2 * BM - 1) / (2 * BM);  // 256-row tiles, one per CTA pair
-    // Programmatic dependent launch hides the ~4 us between consecutive launches (a fifth of
-    // a call at B = 8192), but made the long launches of B = 65536 3% slower: on below 32768.
-    const bool pdl = B < 32768;
     // 128-column gate tiles for compacted live rows, scoring, hierarchical actions
     // (EpiGates2N), and as narrow_gates says for the rest
     const bool narrow = compact || teacher || hier || narrow_gates(f32, acc, Hp, m_tiles * (Hp / 64), T.sms / 2);
@@ -2289,11 +2289,11 @@ static cudaError_t tc_run(const wm_handle *h, int teacher, const wm_rollout_dev 
             if (f32) {
                 gio_n.wa_lo = (const __nv_bfloat16 *)T.wa_n_lo;
                 const OpMaps opn{&ma, &mwgn, &mal, &mwgnl};
-                e = launch_gemm<128, 1, 3, EpiGates32N, 2, 3>(opn, mc, msn, msnl, g2n, gio_n, T.sms, s, pdl);
+                e = launch_gemm<128, 1, 3, EpiGates32N, 2, 3>(opn, mc, msn, msnl, g2n, gio_n, T.sms, s);
             } else {
                 const OpMaps opn{&ma, &mwgn, &ma, &mwgn};
-                e = acc ? launch_gemm<128, 1, 3, EpiGatesNA, 2>(opn, mc, msn, msn, g2n, gio_n, T.sms, s, pdl)
-                        : launch_gemm<128, 1, 3, EpiGatesN, 2>(opn, mc, msn, msn, g2n, gio_n, T.sms, s, pdl);
+                e = acc ? launch_gemm<128, 1, 3, EpiGatesNA, 2>(opn, mc, msn, msn, g2n, gio_n, T.sms, s)
+                        : launch_gemm<128, 1, 3, EpiGatesN, 2>(opn, mc, msn, msn, g2n, gio_n, T.sms, s);
             }
             ++launches;
         }
@@ -2319,8 +2319,8 @@ static cudaError_t tc_run(const wm_handle *h, int teacher, const wm_rollout_dev 
             const GemmGrid g3{(rows + 2 * BM - 1) / (2 * BM), T.n_head_tiles, (Hp + BK - 1) / BK, Zp, h->status};
             const OpMaps oph{&mh, &mwh, &mhl, &mwhl};
             wm_ktime kt(h, WM_KERNEL_TC_HEADS, s);
-            if (f32) e = launch_gemm<HEAD_TILE, 1, 3, EpiHeadsScore, 2, 3>(oph, mc, mc, mc, g3, hio, T.sms, s, pdl);
-            else e = launch_gemm<HEAD_TILE, 1, 3, EpiHeadsScore, 2>(oph, mc, mc, mc, g3, hio, T.sms, s, pdl);
+            if (f32) e = launch_gemm<HEAD_TILE, 1, 3, EpiHeadsScore, 2, 3>(oph, mc, mc, mc, g3, hio, T.sms, s);
+            else e = launch_gemm<HEAD_TILE, 1, 3, EpiHeadsScore, 2>(oph, mc, mc, mc, g3, hio, T.sms, s);
             ++launches;
             if (e != cudaSuccess) return e;
         }
@@ -2414,7 +2414,7 @@ static cudaError_t tc_run(const wm_handle *h, int teacher, const wm_rollout_dev 
             cudaLaunchConfig_t lc = {};
             cudaLaunchAttribute at[1];
             at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-            at[0].val.programmaticStreamSerializationAllowed = pdl ? 1 : 0;
+            at[0].val.programmaticStreamSerializationAllowed = 1;
             {  // a block per CROWS rows, and enough threads for the frozen episodes' outputs
                 const size_t fe = q.fill ? (size_t)Z + ((q.h_seq || q.c_seq) ? H : 0) + (q.mdn_seq ? q.M : 0) + 1 : 0;
                 const size_t rows_blocks = ((size_t)B + CROWS - 1) / CROWS;
@@ -2448,22 +2448,22 @@ static cudaError_t tc_run(const wm_handle *h, int teacher, const wm_rollout_dev 
         if (!teacher && !hier) {
             wm_ktime kt(h, WM_KERNEL_TC_CTRL, s);
             if (f32) {
-                if (Ap > 256) e = launch_gemm<256, 2, 2, EpiCtrl, 2, 3>(opc, mc, mc, mc, g1, io, T.sms, s, pdl);
-                else if (Ap > 128) e = launch_gemm<256, 1, 3, EpiCtrl, 2, 3>(opc, mc, mc, mc, g1, io, T.sms, s, pdl);
-                else e = launch_gemm<128, 1, 3, EpiCtrl, 2, 3>(opc, mc, mc, mc, g1, io, T.sms, s, pdl);
+                if (Ap > 256) e = launch_gemm<256, 2, 2, EpiCtrl, 2, 3>(opc, mc, mc, mc, g1, io, T.sms, s);
+                else if (Ap > 128) e = launch_gemm<256, 1, 3, EpiCtrl, 2, 3>(opc, mc, mc, mc, g1, io, T.sms, s);
+                else e = launch_gemm<128, 1, 3, EpiCtrl, 2, 3>(opc, mc, mc, mc, g1, io, T.sms, s);
             } else {
-                if (Ap > 256) e = launch_gemm<256, 2, 2, EpiCtrl, 2>(opc, mc, mc, mc, g1, io, T.sms, s, pdl);
-                else if (Ap > 128) e = launch_gemm<256, 1, 3, EpiCtrl, 2>(opc, mc, mc, mc, g1, io, T.sms, s, pdl);
-                else e = launch_gemm<128, 1, 3, EpiCtrl, 2>(opc, mc, mc, mc, g1, io, T.sms, s, pdl);
+                if (Ap > 256) e = launch_gemm<256, 2, 2, EpiCtrl, 2>(opc, mc, mc, mc, g1, io, T.sms, s);
+                else if (Ap > 128) e = launch_gemm<256, 1, 3, EpiCtrl, 2>(opc, mc, mc, mc, g1, io, T.sms, s);
+                else e = launch_gemm<128, 1, 3, EpiCtrl, 2>(opc, mc, mc, mc, g1, io, T.sms, s);
             }
             ++launches;
             if (e != cudaSuccess) break;
         } else if (hier) {  // the logits, then the two-stage choice (Sec. 3.1.3); bf16 models only
             {
                 wm_ktime kt(h, WM_KERNEL_TC_CTRL, s);
-                if (Ap > 256) e = launch_gemm<256, 2, 2, EpiLogits, 2>(opc, mc, mc, mc, g1, io, T.sms, s, pdl);
-                else if (Ap > 128) e = launch_gemm<256, 1, 3, EpiLogits, 2>(opc, mc, mc, mc, g1, io, T.sms, s, pdl);
-                else e = launch_gemm<128, 1, 3, EpiLogits, 2>(opc, mc, mc, mc, g1, io, T.sms, s, pdl);
+                if (Ap > 256) e = launch_gemm<256, 2, 2, EpiLogits, 2>(opc, mc, mc, mc, g1, io, T.sms, s);
+                else if (Ap > 128) e = launch_gemm<256, 1, 3, EpiLogits, 2>(opc, mc, mc, mc, g1, io, T.sms, s);
+                else e = launch_gemm<128, 1, 3, EpiLogits, 2>(opc, mc, mc, mc, g1, io, T.sms, s);
             }
             ++launches;
             if (e != cudaSuccess) break;
@@ -2485,16 +2485,16 @@ static cudaError_t tc_run(const wm_handle *h, int teacher, const wm_rollout_dev 
             gio_n.wa_lo = (const __nv_bfloat16 *)T.wa_n_lo;
             const OpMaps opn{&mx[xa], &mwgn, f32 ? &mxl[xa] : &mx[xa], f32 ? &mwgnl : &mwgn};
             wm_ktime kt(h, WM_KERNEL_TC_GATES, s);
-            if (f32) e = launch_gemm<128, 1, 3, EpiGates32N, 2, 3>(opn, mC, mxsn[xn], mxsnl[xn], g2n, gio_n, T.sms, s, pdl);
-            else if (hier && acc) e = launch_gemm<128, 1, 3, EpiGates2NA, 2>(opn, mC, mxsn[xn], mxsn[xn], g2n, gio_n, T.sms, s, pdl);
-            else if (hier) e = launch_gemm<128, 1, 3, EpiGates2N, 2>(opn, mC, mxsn[xn], mxsn[xn], g2n, gio_n, T.sms, s, pdl);
-            else if (acc) e = launch_gemm<128, 1, 3, EpiGatesNA, 2>(opn, mC, mxsn[xn], mxsn[xn], g2n, gio_n, T.sms, s, pdl);
-            else e = launch_gemm<128, 1, 3, EpiGatesN, 2>(opn, mC, mxsn[xn], mxsn[xn], g2n, gio_n, T.sms, s, pdl);
+            if (f32) e = launch_gemm<128, 1, 3, EpiGates32N, 2, 3>(opn, mC, mxsn[xn], mxsnl[xn], g2n, gio_n, T.sms, s);
+            else if (hier && acc) e = launch_gemm<128, 1, 3, EpiGates2NA, 2>(opn, mC, mxsn[xn], mxsn[xn], g2n, gio_n, T.sms, s);
+            else if (hier) e = launch_gemm<128, 1, 3, EpiGates2N, 2>(opn, mC, mxsn[xn], mxsn[xn], g2n, gio_n, T.sms, s);
+            else if (acc) e = launch_gemm<128, 1, 3, EpiGatesNA, 2>(opn, mC, mxsn[xn], mxsn[xn], g2n, gio_n, T.sms, s);
+            else e = launch_gemm<128, 1, 3, EpiGatesN, 2>(opn, mC, mxsn[xn], mxsn[xn], g2n, gio_n, T.sms, s);
         } else {
             wm_ktime kt(h, WM_KERNEL_TC_GATES, s);
-            if (f32) e = launch_gemm<256, 1, 2, EpiGates32, 2, 3>(opg, mC, mxs[xn], mxsl[xn], g2, io, T.sms, s, pdl);
-            else if (acc) e = launch_gemm<256, 1, 2, EpiGatesA, 2>(opg, mC, mxs[xn], mxs[xn], g2, io, T.sms, s, pdl);
-            else e = launch_gemm<256, 1, 2, EpiGates, 2>(opg, mC, mxs[xn], mxs[xn], g2, io, T.sms, s, pdl);
+            if (f32) e = launch_gemm<256, 1, 2, EpiGates32, 2, 3>(opg, mC, mxs[xn], mxsl[xn], g2, io, T.sms, s);
+            else if (acc) e = launch_gemm<256, 1, 2, EpiGatesA, 2>(opg, mC, mxs[xn], mxs[xn], g2, io, T.sms, s);
+            else e = launch_gemm<256, 1, 2, EpiGates, 2>(opg, mC, mxs[xn], mxs[xn], g2, io, T.sms, s);
         }
         ++launches;
         if (e != cudaSuccess) break;
@@ -2502,9 +2502,9 @@ static cudaError_t tc_run(const wm_handle *h, int teacher, const wm_rollout_dev 
         g3.n_rows = io.n_rows;
         {
             wm_ktime kt(h, WM_KERNEL_TC_HEADS, s);
-            if (f32) e = launch_gemm<HEAD_TILE, 1, 3, EpiHeads, 2, 3>(oph, mc, mc, mc, g3, io, T.sms, s, pdl);
-            else if (acc) e = launch_gemm<HEAD_TILE, 1, 3, EpiHeadsA, 2>(oph, mc, mc, mc, g3, io, T.sms, s, pdl);
-            else e = launch_gemm<HEAD_TILE, 1, 3, EpiHeads, 2>(oph, mc, mc, mc, g3, io, T.sms, s, pdl);
+            if (f32) e = launch_gemm<HEAD_TILE, 1, 3, EpiHeads, 2, 3>(oph, mc, mc, mc, g3, io, T.sms, s);
+            else if (acc) e = launch_gemm<HEAD_TILE, 1, 3, EpiHeadsA, 2>(oph, mc, mc, mc, g3, io, T.sms, s);
+            else e = launch_gemm<HEAD_TILE, 1, 3, EpiHeads, 2>(oph, mc, mc, mc, g3, io, T.sms, s);
         }
         ++launches;
         if (e == cudaSuccess && hooks) e = hooks->after_step(t, s);

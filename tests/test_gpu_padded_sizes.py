@@ -68,10 +68,10 @@ def test_rollout(wm, orc, Z, A, H, K, B, flags):
 
 
 # more gate tiles of 256 columns than 76 CTA pairs: two action rows; bf16 with a last wave half full
-# (80, 114) and just over (115); fp32 over the whole range of its rule (40, 320, 330, 512)
+# (80, 114, 115, 160) and many waves; fp32 on both sides of its rule (40, 316, 320, 330, 512)
 @pytest.mark.parametrize("H,B,precision,NX", [
     (256, 9985, "bf16", 32), (512, 5001, "bf16", 32), (512, 2500, "bf16", 0), (1216, 1281, "bf16", 0),
-    (320, 5800, "bf16", 0), (1024, 2500, "bf16", 0), (512, 1100, "fp32", 0), (256, 20001, "fp32", 0),
+    (320, 5800, "bf16", 0), (1024, 2500, "bf16", 0), (512, 40001, "bf16", 0), (512, 1100, "fp32", 0), (256, 20001, "fp32", 0),
     (512, 10200, "fp32", 0), (704, 7600, "fp32", 0), (512, 16300, "fp32", 0)])
 def test_gates_over_many_tiles(wm, H, B, precision, NX):
     """The bits of the same episodes in a batch of few tiles (which the oracle checks)."""
