@@ -236,13 +236,13 @@ struct wm_recur_args {
     int *status;
     uint32_t test_wait;
     // the plan
-    int units, n_tiles, m_tiles, m_groups, groups, cluster, k_steps, stages, kps;
+    int units, n_tiles, m_tiles, m_groups, groups, k_steps, stages, kps;
     size_t smem;
 };
 // Whether (and how) N sequences run as one launch.
 bool wm_recur_plan(int mode, int N, int Hp, int KX, wm_recur_args *a);
 // mode: 0 bf16, 1 bf16 with accurate nonlinearities, 2 fp32 as bf16 parts.  Tensor maps: x rows in
-// boxes of 128 / cluster rows x 64, weights (128-column packing) in boxes of `units` rows x 64.
+// boxes of 128 rows x 64, weights (128-column packing) in boxes of `units` rows x 64.
 cudaError_t wm_recur_launch(int mode, const void *x_map, const void *xl_map, const void *w_map, const void *wl_map,
                             const wm_recur_args &a, cudaStream_t s);
 

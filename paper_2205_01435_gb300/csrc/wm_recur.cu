@@ -12,16 +12,14 @@
 //   - h_{t+1} goes to the operand rows of frame t + 1 in global memory (L2), then the CTA adds
 //     one to the row tile's counter (release); the CTAs of that row tile load their rows by TMA
 //     once the counter shows all unit tiles of step t (acquire).  Frames are distinct rows, so
-//     nothing is overwritten and one counter is the only dependency;
-//   - the 2 or 4 CTAs of a cluster share a row tile and multicast a part of every block to each
-//     other.
-// A step (512 sequences, H = 512, clock64 stamps of one CTA, cycles at about 2 GHz): counter to
-// accumulator 3.9K (operands land at the rate of one 16 KB part per 215 cycles after 1.2K, then
-// the last MMAs), cell 0.95K, stores to the counter's release 1.9K, release to the next step's
-// acquire 1.2K: 8K, 4 us.  A call of 512 x 128 takes 0.67 ms, 1.28 as one launch per step; on the
-// fp32 path (two parts per block through a ring that holds 4; paced by the issuer's MMAs) 1.21 ms,
-// 2.38 before.  Up to RECUR_MAX_GROUPS row tiles per CTA this stays ahead of one launch per step
-// (24 steps at H = 512: 1024 / 2048 sequences 221 / 341 us against 288 / 432).
+//     nothing is overwritten and one counter is the only dependency.  Every CTA loads its whole
+//     operand blocks itself.
+// A step (512 sequences, H = 512) takes about 4 us: operands through L2, MMAs, cell, stores and the
+// hand-off are one chain.  A call of 512 x 128 takes 0.64 ms, 1.28 as one launch per step; on the
+// fp32 path (two parts per block through a ring that holds 4; paced by the issuer's MMAs) 1.22 ms,
+// 2.38 before.  (With the loads of a row tile shared by a cluster of four CTAs: 0.67 and 1.21.)  Up
+// to RECUR_MAX_GROUPS row tiles per CTA this stays ahead of one launch per step (24 steps at H = 512:
+// 1024 / 2048 sequences 221 / 341 us against 288 / 432).
 // Every CTA waits for others: the launch is cooperative (all CTAs resident), every wait is
 // bounded, and a CTA that gives up records WM_ERR_TIMEOUT, skips its remaining work and exits.
 //
@@ -53,20 +51,6 @@ __device__ __forceinline__ int ld_acquire(const int *p) {
 // generic-proxy global accesses ordered before / after TMA's (async-proxy) ones
 __device__ __forceinline__ void fence_proxy_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
 
-// TMA tile load into the same shared-memory offset (and onto the same mbarrier) of every CTA in mask
-__device__ __forceinline__ void tma_load_multicast(uint32_t dst, const CUtensorMap *map, int x, int y, uint32_t mbar,
-                                                   uint16_t mask) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster [%0], [%1, {%2, %3}], [%4], %5;"
-        :: "r"(dst), "l"(map), "r"(x), "r"(y), "r"(mbar), "h"(mask) : "memory");
-}
-// arrive on this mbarrier of every CTA in mask when this thread's MMAs so far have completed
-__device__ __forceinline__ void mma_commit_multicast(uint32_t mbar, uint16_t mask) {
-    asm volatile(
-        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-        :: "r"(mbar), "h"(mask) : "memory");
-}
-
 __device__ __forceinline__ float tanh_hw(float x) {
     float y;
     asm("tanh.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -97,11 +81,6 @@ __global__ void __launch_bounds__(THREADS, 1)
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int n = blockIdx.x % p.n_tiles, mg = blockIdx.x / p.n_tiles;
     const int ks = p.k_steps, S = p.stages;
-    // The CTAs of a cluster share a row tile: each loads 1 / CL of every operand block and multicasts
-    // it, so the block leaves L2 once per cluster.
-    const int CL = p.cluster;
-    const uint32_t rank = tc::cluster_rank();
-    const uint16_t all = (uint16_t)((1u << CL) - 1u);
     const uint32_t sw = tc::smem_u32(smem), sa = sw + (uint32_t)ks * PARTS * W_BYTES;
     float *cst = reinterpret_cast<float *>(smem + (size_t)ks * PARTS * W_BYTES + (size_t)S * KPS * A_BYTES);
     auto bar = [](uint64_t *b) { return tc::smem_u32(b); };
@@ -109,7 +88,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     if (tid == 0) {
         for (int s = 0; s < S; ++s) {
             tc::mbar_init(bar(&bar_full[s]), 1);
-            tc::mbar_init(bar(&bar_empty[s]), CL);  // every CTA of the cluster has consumed the stage
+            tc::mbar_init(bar(&bar_empty[s]), 1);
         }
         for (int a = 0; a < 2; ++a) {
             tc::mbar_init(bar(&bar_accf[a]), 1);
@@ -123,7 +102,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     }
     if (warp == 1) tc::tmem_alloc(tc::smem_u32(&tmem_base), 2 * NA);
     tc::fence_before_sync();
-    tc::cluster_sync();  // the cluster's barriers exist before any copy or arrive reaches them
+    __syncthreads();
     tc::fence_after_sync();
     const uint32_t tm = tmem_base;
     int T = p.T;
@@ -176,32 +155,27 @@ __global__ void __launch_bounds__(THREADS, 1)
                         if (!__all_sync(0xffffffffu, ok)) break;
                         fence_proxy_async_global();
                     }
-                    const int rows = BM / CL, y = t * p.N + m * BM + (int)rank * rows;
-                    const uint32_t slice = sa + rank * rows * (BK * 2);
+                    const int y = t * p.N + m * BM;
                     for (int i0 = 0; i0 < np; i0 += KPS) {
                         const int nk = np - i0 < KPS ? np - i0 : KPS;
                         if (!(go = wait(&bar_empty[stage], phase ^ 1u))) break;
                         if (tc::elect_one()) {
-                            const uint32_t full = bar(&bar_full[stage]), dst = slice + stage * KPS * A_BYTES;
+                            const uint32_t full = bar(&bar_full[stage]), dst = sa + stage * KPS * A_BYTES;
                             tc::mbar_arrive_expect_tx(full, nk * A_BYTES);
 #pragma unroll
                             for (int h = 0; h < KPS; ++h)
                                 if (h < nk)
-                                    tma_load_multicast(dst + h * A_BYTES, F32 && (h & 1) ? &tmXl : &tmX, (i0 + h) / PARTS * BK, y,
-                                                       full, all);
+                                    tc::tma_load_2d(dst + h * A_BYTES, F32 && (h & 1) ? &tmXl : &tmX, (i0 + h) / PARTS * BK, y, full);
                         }
                         ++used;
                         if (++stage == S) { stage = 0; phase ^= 1u; }
                     }
                 }
-            // nothing may be in flight into the cluster's shared memory when a CTA exits (after a normal
-            // end everything has landed long since; after giving up, also leave peers' copies time)
+            // nothing may be in flight into shared memory when the CTA exits
             __syncwarp();
-            const bool gave_up = s_abort != 0;
             tc::mbar_wait_bounded(bar(&bar_w), 0, POLLS);
             for (int i = used > S ? used - S : 0; i < used; ++i)
-                tc::mbar_wait_bounded(bar(&bar_full[i % S]), (uint32_t)(i / S) & 1u, gave_up ? 1u << 16 : POLLS);
-            if (gave_up) tc::mbar_wait_bounded(bar(&bar_never), 0, 1u << 14);
+                tc::mbar_wait_bounded(bar(&bar_full[i % S]), (uint32_t)(i / S) & 1u, POLLS);
         }
     } else if (warp == 1) {
         if (T > 0) {  // ---- MMA issuer (likewise)
@@ -233,7 +207,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                                         tc::mma_bf16(d, da + (A_BYTES >> 4) + 2 * kk, db + 2 * kk, idesc, 1u);
                                 }
                             }
-                            mma_commit_multicast(bar(&bar_empty[stage]), all);
+                            tc::mma_commit(bar(&bar_empty[stage]));
                         }
                         if (++stage == S) { stage = 0; phase ^= 1u; }
                     }
@@ -413,7 +387,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     }
     __syncwarp();
     tc::fence_before_sync();
-    tc::cluster_sync();  // peers' copies into, and arrives on, this CTA's shared memory are done
+    __syncthreads();
     if (warp == 1) tc::tmem_dealloc(tm, 2 * NA);
 }
 
@@ -424,18 +398,6 @@ size_t fixed_smem(bool f32, int U, int ks, int groups) {
     return 1024 + (size_t)ks * (f32 ? 2 : 1) * 4 * U * BK * 2 + (size_t)groups * U * BM * 4;
 }
 
-void set_attrs(cudaLaunchConfig_t &lc, cudaLaunchAttribute (&at)[2], int cluster, size_t smem) {
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = (unsigned)cluster;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    at[1].id = cudaLaunchAttributeCooperative;  // every CTA resident: they wait for one another
-    at[1].val.cooperative = 1;
-    lc.blockDim = dim3(THREADS);
-    lc.dynamicSmemBytes = smem;
-    lc.attrs = at;
-    lc.numAttrs = 2;
-}
-
 using kern_t = void (*)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap, wm_recur_args);
 kern_t kernel_of(int mode, int units, int kps) {
     if (mode == 2) return units == 16 ? k_recur<2, 16, 2> : k_recur<2, 32, 2>;
@@ -444,25 +406,22 @@ kern_t kernel_of(int mode, int units, int kps) {
     return units == 16 ? (kps == 3 ? k_recur<0, 16, 3> : k_recur<0, 16, 2>) : (kps == 3 ? k_recur<0, 32, 3> : k_recur<0, 32, 2>);
 }
 
-// CTAs that can be resident at once in clusters of `cluster` (one per SM)
-int resident(int mode, int units, int kps, int cluster) {
-    static int known[WM_MAX_DEVICES][3][2][2][3] = {};  // (the shared-memory limit is a device's, too)
-    int &n = known[wm_device_slot()][mode][units >> 5][kps - 2][cluster >> 1];
+// CTAs that can be resident at once (one per SM)
+int resident(int mode, int units, int kps) {
+    static int known[WM_MAX_DEVICES][3][2][2] = {};  // (the shared-memory limit is a device's, too)
+    int &n = known[wm_device_slot()][mode][units >> 5][kps - 2];
     if (!n) {
         const kern_t kern = kernel_of(mode, units, kps);
         const size_t smem = SMEM_MAX - SMEM_STATIC;
-        cudaLaunchConfig_t lc = {};
-        cudaLaunchAttribute at[2];
-        set_attrs(lc, at, cluster, smem);
-        lc.gridDim = dim3((unsigned)cluster);
-        lc.numAttrs = 1;
-        int c = 0;
+        int dev = 0, sms = 0, c = 0;
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
-            cudaOccupancyMaxActiveClusters(&c, kern, &lc) != cudaSuccess) {
+            cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c, kern, THREADS, smem) != cudaSuccess) {
             cudaGetLastError();
             c = 0;
         }
-        n = c > 0 ? c * cluster : -1;
+        n = c > 0 ? c * sms : -1;
     }
     return n;
 }
@@ -474,12 +433,12 @@ bool wm_recur_plan(int mode, int N, int Hp, int KX, wm_recur_args *a) {
     const int ks = (KX + BK - 1) / BK, mt = (N + BM - 1) / BM;
     bool found = false;
     for (int U : {16, 32}) {
-        const int nt = Hp / U, cl = nt % 4 == 0 ? 4 : 2;
+        const int nt = Hp / U;
         // the ring's depth follows from what the weights and the cell states leave
         int mg = 0, groups = 0, kps = 0, stages = 0;
         size_t fixed = 0;
         for (int pass = 0; pass < 2; ++pass) {  // (the states' share depends on the resident CTAs, found with kps = 2)
-            const int ctas = resident(mode, U, pass ? kps : 2, cl);
+            const int ctas = resident(mode, U, pass ? kps : 2);
             if (nt > ctas) { stages = 0; break; }
             mg = mt < ctas / nt ? mt : ctas / nt;
             groups = (mt + mg - 1) / mg;
@@ -495,7 +454,6 @@ bool wm_recur_plan(int mode, int N, int Hp, int KX, wm_recur_args *a) {
         a->m_tiles = mt;
         a->m_groups = mg;
         a->groups = groups;
-        a->cluster = cl;
         a->k_steps = ks;
         a->stages = stages;
         a->kps = kps;
@@ -507,10 +465,15 @@ bool wm_recur_plan(int mode, int N, int Hp, int KX, wm_recur_args *a) {
 cudaError_t wm_recur_launch(int mode, const void *x_map, const void *xl_map, const void *w_map, const void *wl_map,
                             const wm_recur_args &a, cudaStream_t s) {
     cudaLaunchConfig_t lc = {};
-    cudaLaunchAttribute at[2];
-    set_attrs(lc, at, a.cluster, a.smem);
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeCooperative;  // every CTA resident: they wait for one another
+    at[0].val.cooperative = 1;
     lc.gridDim = dim3((unsigned)(a.n_tiles * a.m_groups));
+    lc.blockDim = dim3(THREADS);
+    lc.dynamicSmemBytes = a.smem;
     lc.stream = s;
+    lc.attrs = at;
+    lc.numAttrs = 1;
     return cudaLaunchKernelEx(&lc, kernel_of(mode, a.units, a.kps), *(const CUtensorMap *)x_map, *(const CUtensorMap *)xl_map,
                               *(const CUtensorMap *)w_map, *(const CUtensorMap *)wl_map, a);
 }

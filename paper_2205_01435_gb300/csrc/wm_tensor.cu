@@ -2243,10 +2243,10 @@ static cudaError_t tc_run(const wm_handle *h, int teacher, const wm_rollout_dev 
         const bool one = one_launch(h, B, Tn, &ra_, &rmode);
         if (one) {  // the whole recurrence in one launch
             CUtensorMap xm, xlm, wmap, wlmap;
-            if (!make_map(&xm, w.xall, frames, KX, BM / ra_.cluster) || !make_map(&wmap, T.wg_n, 4 * Hp, KX, ra_.units))
+            if (!make_map(&xm, w.xall, frames, KX, BM) || !make_map(&wmap, T.wg_n, 4 * Hp, KX, ra_.units))
                 return cudaErrorInvalidValue;
             if (f32) {
-                if (!make_map(&xlm, w.xall_lo, frames, KX, BM / ra_.cluster) || !make_map(&wlmap, T.wg_n_lo, 4 * Hp, KX, ra_.units))
+                if (!make_map(&xlm, w.xall_lo, frames, KX, BM) || !make_map(&wlmap, T.wg_n_lo, 4 * Hp, KX, ra_.units))
                     return cudaErrorInvalidValue;
             } else {
                 xlm = xm;
