@@ -267,18 +267,19 @@ cudaError_t pack_step(wm_handle *h, const wm_weights *w) {
 // 600 / 2000 / 8000 against 1791 / 2615 / 3819 / 12135 us stepwise, at 64, 256, 512, 8 and B = 64
 // 722 against 3378 us.  Left to the stepwise family: fp32 models of such sizes (its fp32 sums are
 // more accurate than three bf16 products), K > 8, A > 512, populations that do not fill row tiles,
-// and rollouts of more than 4 steps with H > 512: there a trajectory is chaotic, so that the sums'
-// order alone moves it by 5 to 10% within 25 steps (rel. 2-norm of z, rewards, h; 1% at 4 steps,
-// and under 1% at H <= 512), and a small batch's results stay what they were.  fused_ok / tc_ok:
-// whether this call's options allow those families; steps: of a rollout (0: a scoring call).
-int pick_path(const wm_handle *h, int B, bool fused_ok = true, bool tc_ok = true, int steps = 0, bool pad_ok = true) {
+// and rollouts with H > 512: there a trajectory is chaotic, so that the sums' order alone moves it by
+// 5 to 10% within 25 steps (rel. 2-norm of z, rewards, h; under 1% at H <= 512), and these calls'
+// results stay what they were.  A rollout's family does not depend on its number of steps: one split
+// over calls has the unsplit one's bits.  fused_ok / tc_ok / pad_ok: whether this call may take
+// those families, and the tensor family outside its own sizes and batches.
+int pick_path(const wm_handle *h, int B, bool fused_ok, bool tc_ok, bool pad_ok) {
     const int p = h->cfg.path;
     if (p != WM_PATH_AUTO) return p;
     const bool fu = fused_ok && wm_fused_supported(h, B), tc = tc_ok && wm_tc_supported(h);
     if (fu && B <= 2048) return WM_PATH_FUSED;
     if (tc && (B >= 256 || h->cfg.precision == WM_FP32)) return WM_PATH_TENSOR;
     if (fu) return WM_PATH_FUSED;
-    if (tc_ok && pad_ok && wm_tc_auto_ok(h) && (h->cfg.h_dim <= 512 || steps <= 4)) return WM_PATH_TENSOR;
+    if (tc_ok && pad_ok && wm_tc_auto_ok(h)) return WM_PATH_TENSOR;
     return WM_PATH_STEPWISE;
 }
 
@@ -296,7 +297,7 @@ int pick_score_path(const wm_handle *h, int N, int T, bool train) {
         const bool kept = T < 12 || (train && h->cfg.h_dim < 64 && N <= 400);
         if (!(kept && wm_fused_supported(h, N))) return WM_PATH_TENSOR;
     }
-    return pick_path(h, N, true, true, 0, fits);
+    return pick_path(h, N, true, true, fits);
 }
 
 template <class T>
@@ -555,7 +556,7 @@ wm_status wm_rollout(wm_handle *h, int B, int T, unsigned long long episode_offs
     // family needs a population's candidates aligned to its 256-row tiles
     const bool fused_ok = !io->logp_seq && !(c.value_head && io->value_seq) && h->P == 1 && c.n_xfers == 0;
     const bool tc_ok = wm_tc_call_ok(h, episode_offset) != 0;
-    int path = pick_path(h, B, fused_ok, tc_ok, T);
+    int path = pick_path(h, B, fused_ok, tc_ok, c.h_dim <= 512);
     if (path == WM_PATH_FUSED && !(fused_ok && wm_fused_supported(h, B)))
         return fail(h, WM_ERR_UNSUPPORTED, "the fused family does not take this model / batch / outputs");
     if (c.path == WM_PATH_TENSOR && !(tc_ok && wm_tc_supported(h)))

@@ -298,6 +298,26 @@ def test_resume_is_bit_exact(wm, name, path):
         assert torch.equal(torch.cat([a[k], b[k]]), full[k]), k
 
 
+# one model per choice of AUTO beside those: padded sizes, small batches, H > 512 (few steps or many)
+@pytest.mark.parametrize("Z,A,H,K,B,prec,path", [
+    (50, 101, 300, 6, 40, "bf16", "tensor"), (64, 256, 512, 8, 60, "bf16", "tensor"), (32, 128, 1024, 8, 64, "bf16", "stepwise"),
+    (20, 100, 600, 4, 300, "bf16", "stepwise"), (64, 256, 512, 8, 300, "bf16", "tensor"), (64, 256, 512, 8, 30, "fp32", "tensor"),
+    (20, 100, 300, 4, 30, "fp32", "stepwise")])
+def test_resume_is_bit_exact_on_every_family(wm, Z, A, H, K, B, prec, path):
+    cfg = dict(synth.model_config("small_bf16"), z_dim=Z, a_dim=A, h_dim=H, k_mix=K, precision=prec, ctrl_sample=1)
+    m, T = wm.WorldModel(cfg, synth.weights(cfg, seed=8)), 8
+    z0, mask = _cuda(synth.z0(B, Z, seed=8)), _cuda(synth.mask(T, B, A, 0.4, seed=8))
+    full = m.rollout(z0, T, mask=mask, want_logp=True)  # log-probs: not the fused family
+    assert m.last_path == path
+    a = m.rollout(z0, 4, mask=mask[:4].contiguous(), want_logp=True)
+    b = m.rollout(a["z"][4].contiguous(), 4, mask=mask[4:].contiguous(), t0=4, h0=a["h_final"], c0=a["c_final"], want_logp=True)
+    assert m.last_path == path
+    assert torch.equal(torch.cat([a["z"], b["z"][1:]]), full["z"])
+    for k in ("actions", "rewards", "done", "logp_seq"):
+        assert torch.equal(torch.cat([a[k], b[k]]), full[k]), k
+    assert torch.equal(b["h_final"], full["h_final"])
+
+
 @pytest.mark.parametrize("kind", ["pinned", "pageable"])
 @pytest.mark.parametrize("path,B,T,seq,done", [("auto", None, 6, False, 0),  # fused: copied whole around the call
                                                ("tensor", 700, 6, True, 0),   # per-step staging, every output kind
