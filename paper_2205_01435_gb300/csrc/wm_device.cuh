@@ -178,4 +178,14 @@ __device__ __forceinline__ float round_bf16(float x) { return __bfloat162float(_
 
 __device__ __forceinline__ float sigmoidf_(float x) { return 1.0f / (1.0f + expf(-x)); }
 
+// The same without the division: the hardware's reciprocal and one step of Newton's iteration, which
+// leaves about half a roundoff (60 sequences x 128 steps at H = 512: the recurrence 678 us with the
+// division, 535 so).  Below 2^-126 (x < -87.3) it is 0.
+__device__ __forceinline__ float sigmoid_newton(float x) {
+    float d = 1.f + expf(-x), r;
+    asm("min.NaN.f32 %0, %0, 0f7F7FFFFF;" : "+f"(d));  // (of infinity the step would make a NaN)
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
+    return fmaf(r, fmaf(-d, r, 1.f), r);
+}
+
 }  // namespace wmk

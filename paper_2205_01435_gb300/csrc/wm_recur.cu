@@ -57,8 +57,9 @@ __device__ __forceinline__ float tanh_hw(float x) {
     return y;
 }
 
-// MODE 0: bf16 operands, hardware tanh; 1: bf16 operands, accurate tanh; 2: the fp32 path, each
-// operand as bf16 hi and lo parts (products hi.hi + hi.lo + lo.hi), accurate tanh.
+// MODE 0: bf16 operands, hardware tanh; 1: bf16 operands, the stepwise family's accurate
+// nonlinearities; 2: the fp32 path, each operand as bf16 hi and lo parts (products hi.hi + hi.lo +
+// lo.hi), accurate tanh.
 // KPS operand parts (16 KB) make a ring stage: the producer's and the issuer's turns cost 200 to 300
 // cycles a stage beside the copies (30 each) and MMAs (70 a part), and a part lands every 215.
 template <int MODE, int U, int KPS>
@@ -251,7 +252,9 @@ __global__ void __launch_bounds__(THREADS, 1)
                 }
             }
         };
-        auto sig = [](float x) { return MODE ? fmaf(0.5f, tanhf(0.5f * x), 0.5f) : fmaf(0.5f, tanh_hw(0.5f * x), 0.5f); };
+        auto sig = [](float x) {
+            return MODE == 1 ? sigmoid_newton(x) : MODE ? fmaf(0.5f, tanhf(0.5f * x), 0.5f) : fmaf(0.5f, tanh_hw(0.5f * x), 0.5f);
+        };
         auto th = [](float x) { return MODE ? tanhf(x) : tanh_hw(x); };
         // The action row's columns are gathers from L2 (32 lines per load).  They go out right after a
         // tile's h' (its action was loaded one tile before that), so that they are done before the next

@@ -242,7 +242,9 @@ struct EpiCtx {
 // the bias is read from a copy in shared memory.  The tempered draw keeps each
 // chunk's sum of weights, so only the chunk that holds the drawn point is read a
 // third time.
-struct EpiCtrl {
+// ACC: accurate exponentials and divisions in the draw (as EpiGatesT's ACC).
+template <bool ACC>
+struct EpiCtrlT {
     static constexpr bool TMA_STAGE = false;
     static constexpr uint32_t QUAD_STAGE = 0;
     static constexpr int MAX_A = 512, NCH = MAX_A / 4 / 16;  // chunks per column group, at most
@@ -365,6 +367,21 @@ struct EpiCtrl {
             // weight of logit v: exp((v - max) / tau) = 2^(v * s - max * s), s = log2(e) / tau;
             // a masked column's weight is forced to +0 (its logit may exceed the maximum)
             const float sc = 1.4426950408889634f / p.ctrl_tau, off = -gbv * sc;
+            // ACC: expf((v - max) / tau), the quotient as a product and one correction by its exact
+            // remainder (60 x 64 steps at A = 256: 3.08 ms with a division per column, 2.26 so, 2.06
+            // with the other form's approximation).  floor: e^-128 is 0 in fp32, and an infinite
+            // logit's remainder would be a NaN; tau is kept where its reciprocal is a normal number.
+            const float tau = fminf(fmaxf(p.ctrl_tau, 0x1p-100f), 0x1p100f), rtau = 1.f / tau, floor = -128.f * tau;
+            auto weight = [&](float v) {
+                if constexpr (ACC) {
+                    float d = v - gbv;
+                    asm("max.NaN.f32 %0, %0, %1;" : "+f"(d) : "f"(floor));
+                    const float q = d * rtau;
+                    return expf(fmaf(fmaf(-q, tau, d), rtau, q));
+                } else {
+                    return ex2_approx(fmaf(v, sc, off));
+                }
+            };
             // pass 2: the group's sum of tempered weights, chunk by chunk
             float cs[NCH], S = 0.f;
 #pragma unroll
@@ -377,7 +394,7 @@ struct EpiCtrl {
                 float sk = 0.f;
 #pragma unroll
                 for (int j = 0; j < 16; ++j)
-                    sk += __uint_as_float(__float_as_uint(ex2_approx(fmaf(v[j], sc, off))) & lane_mask(bits, j));
+                    sk += __uint_as_float(__float_as_uint(weight(v[j])) & lane_mask(bits, j));
                 cs[k] = sk;
                 S += sk;
             }
@@ -437,7 +454,7 @@ struct EpiCtrl {
                     uint32_t hit = 0u;  // valid columns at which the running sum has passed the target
 #pragma unroll
                     for (int j = 0; j < 16; ++j) {
-                        cum += __uint_as_float(__float_as_uint(ex2_approx(fmaf(v[j], sc, off))) & lane_mask(bits, j));
+                        cum += __uint_as_float(__float_as_uint(weight(v[j])) & lane_mask(bits, j));
                         hit |= (target < cum ? 1u : 0u) << j;
                     }
                     hit &= bits;
@@ -459,7 +476,7 @@ struct EpiCtrl {
                 }
                 if (draw) {
                     ga = pick >= 0 ? pick : glast;  // rounding past the last valid action
-                    logp = pick >= 0 ? (lvp - gbv) * itau - log_total : 0.f;
+                    logp = pick >= 0 ? (ACC ? (lvp - gbv) / p.ctrl_tau : (lvp - gbv) * itau) - log_total : 0.f;
                 }
             }
         }
@@ -472,6 +489,8 @@ struct EpiCtrl {
         if (p.logp_seq) p.logp_seq[tb] = ga >= 0 ? logp : 0.f;
     }
 };
+using EpiCtrl = EpiCtrlT<false>;
+using EpiCtrlA = EpiCtrlT<true>;
 
 
 // ---- controller logits epilogue (hierarchical actions): every live row's A logits plus
@@ -569,8 +588,8 @@ __global__ void __launch_bounds__(256) k_tc_select(StepIO p) {
 // UNITS: hidden units per tile (64: a 256-column tile; 32: a 128-column tile, for calls with
 // few row tiles, where twice the tiles keep twice the CTA pairs busy and each tile's
 // epilogue is half as long).  Each thread of a quadrant's 4 column groups takes UT units.
-// ACC: the accurate nonlinearities on the bf16 path, for the calls that the stepwise family's
-// accurate ones served before (padded sizes, small batches).
+// ACC: the stepwise family's nonlinearities (sigma as 1 / (1 + e^-x): accurate also where it is
+// small) on the bf16 path, for the calls that family served before (padded sizes, small batches).
 template <int MODE, int UNITS = 64, bool ACC = false>
 struct EpiGatesT {
     static constexpr bool TWO = MODE != 0, F32 = MODE == 2, PRECISE = F32 || ACC;
@@ -653,7 +672,9 @@ struct EpiGatesT {
     }
     // the cell's nonlinearities: the hardware tanh on the bf16 path; accurate ones on the
     // fp32 path (tanh.approx's relative error, about 2^-11, is above its tolerance)
-    static __device__ __forceinline__ float sig_(float x) { return PRECISE ? fmaf(0.5f, tanhf(0.5f * x), 0.5f) : sigmoid_hw(x); }
+    static __device__ __forceinline__ float sig_(float x) {
+        return ACC ? sigmoid_newton(x) : F32 ? fmaf(0.5f, tanhf(0.5f * x), 0.5f) : sigmoid_hw(x);
+    }
     static __device__ __forceinline__ float tanh_(float x) { return PRECISE ? tanhf(x) : tanh_hw(x); }
     // pre-activations of one gate for the thread's 16 units: accumulator + bias + W_a[a]
     // (+ W_a[a2] when TWO)
@@ -2451,6 +2472,10 @@ static cudaError_t tc_run(const wm_handle *h, int teacher, const wm_rollout_dev 
                 if (Ap > 256) e = launch_gemm<256, 2, 2, EpiCtrl, 2, 3>(opc, mc, mc, mc, g1, io, T.sms, s);
                 else if (Ap > 128) e = launch_gemm<256, 1, 3, EpiCtrl, 2, 3>(opc, mc, mc, mc, g1, io, T.sms, s);
                 else e = launch_gemm<128, 1, 3, EpiCtrl, 2, 3>(opc, mc, mc, mc, g1, io, T.sms, s);
+            } else if (acc) {
+                if (Ap > 256) e = launch_gemm<256, 2, 2, EpiCtrlA, 2>(opc, mc, mc, mc, g1, io, T.sms, s);
+                else if (Ap > 128) e = launch_gemm<256, 1, 3, EpiCtrlA, 2>(opc, mc, mc, mc, g1, io, T.sms, s);
+                else e = launch_gemm<128, 1, 3, EpiCtrlA, 2>(opc, mc, mc, mc, g1, io, T.sms, s);
             } else {
                 if (Ap > 256) e = launch_gemm<256, 2, 2, EpiCtrl, 2>(opc, mc, mc, mc, g1, io, T.sms, s);
                 else if (Ap > 128) e = launch_gemm<256, 1, 3, EpiCtrl, 2>(opc, mc, mc, mc, g1, io, T.sms, s);

@@ -115,3 +115,54 @@ def test_forced_path_still_refuses_unaligned_sizes(wm):
     with pytest.raises(wm.WMError) as e:
         m.rollout(torch.zeros(300, 50, device="cuda"), 1)
     assert e.value.status == wm.WM_ERR_UNSUPPORTED
+
+
+# sizes padded, and a small batch of an aligned model; a second action row
+ACCURATE = [(50, 101, 300, 6, 300, 0), (64, 256, 512, 8, 60, 0), (31, 90, 100, 4, 260, 23), (24, 512, 128, 8, 100, 0)]
+
+
+@pytest.mark.parametrize("Z,A,H,K,B,NX", ACCURATE)
+def test_small_sigmoids_keep_their_relative_accuracy(wm, Z, A, H, K, B, NX):
+    """Zero weights, gate biases i = o = -18, f = -30, g = 1: c' = sigma(-18) tanh(1), h' = sigma(-18) tanh(c')."""
+    cfg = _cfg(Z, A, H, K, n_xfers=NX)
+    w = {k: np.zeros_like(v) if isinstance(v, np.ndarray) else v for k, v in synth.weights(cfg, seed=1).items()}
+    w["b_lstm"] = np.repeat(np.float32([-18, -30, 1, -18]), H)
+    s18 = 1 / (1 + np.exp(18.0))
+    c = s18 * np.tanh(1.0)
+    m = wm.WorldModel(cfg, w)
+    outs = [m.rollout(torch.zeros(B, Z, device="cuda"), 1, want_seq=True, want_logp=True)]
+    assert m.last_path == "tensor"
+    if not NX:
+        for T in (1, 12):  # one launch per step (a fused member at H = 128), and one launch
+            outs.append(m.mdn_nll(torch.zeros(T + 1, B, Z, device="cuda"),
+                                  torch.full((T, B), -1, dtype=torch.int32, device="cuda"), want_seq=True))
+            assert m.last_path == ("fused" if T == 1 and H == 128 else "tensor")
+            if m.last_path == "fused":
+                outs.pop()  # (its exponential is the hardware's)
+    for g in outs:
+        # expf, tanhf (2 ulp each), an addition, a reciprocal, a product: under 16 fp32 roundoffs
+        np.testing.assert_allclose(np_(g["c_seq"][0]), c, rtol=16 * 2.0**-24)
+        np.testing.assert_allclose(np_(g["h_seq"][0]), s18 * np.tanh(c), rtol=24 * 2.0**-24)
+
+
+@pytest.mark.parametrize("Z,A,H,K,B,NX", [v for v in ACCURATE if not v[-1]])
+def test_draws_weigh_logits_accurately(wm, Z, A, H, K, B, NX):
+    """Logits that are the bias alone, large beside their differences: the log-probability of the drawn
+    action against 64 bits."""
+    cfg = _cfg(Z, A, H, K, ctrl_sample=1, ctrl_tau=0.05)
+    w = synth.weights(cfg, seed=2)
+    w["W_ctrl"] = np.zeros_like(w["W_ctrl"])
+    w["b_ctrl"] = (100 + np.random.default_rng(2).random(A) * 0.5).astype(np.float32)
+    mask = synth.mask(1, B, A, 0.5, seed=2)
+    m = wm.WorldModel(cfg, w)
+    g = m.rollout(_cuda(synth.z0(B, Z, seed=2)), 1, mask=_cuda(mask), want_logp=True)
+    assert m.last_path == "tensor"
+    acts = np_(g["actions"])[0]
+    valid = np.unpackbits(mask[0].view(np.uint8), axis=-1, bitorder="little")[:, :A].astype(bool)
+    l = np.where(valid, w["b_ctrl"].astype(np.float64) / np.float64(np.float32(0.05)), -np.inf)
+    top = l.max(-1, keepdims=True)
+    lp = l - top - np.log(np.exp(l - top).sum(-1, keepdims=True))
+    ok = acts >= 0
+    assert ok.sum() > B // 2
+    # a quotient up to 10 (2^-24 of it), exponentials (2 ulp each), their sum and its logarithm
+    np.testing.assert_allclose(np_(g["logp_seq"])[0][ok], lp[np.arange(B), acts][ok], rtol=0, atol=64 * 2.0**-24)
