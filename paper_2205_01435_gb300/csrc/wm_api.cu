@@ -703,22 +703,19 @@ wm_status wm_mdn_nll_backward(wm_handle *h, int N, int T, const float *z_seq, co
     size_t need = path == WM_PATH_FUSED ? wm_fused_nll_ws(h, N) : path == WM_PATH_TENSOR ? wm_tc_ws(h, N, T)
                                                                                       : wm_step_nll_ws(h, N);
     if ((e = grow(&h->ws, &h->ws_bytes, need)) != cudaSuccess) return cuda_fail(h, e, "workspace");
-    if ((e = grow(&h->bws, &h->bws_bytes, wm_bw_ws(h, N, T))) != cudaSuccess)
+    wm_bw_fwd f = wm_bw_plan(h, N, T, path == WM_PATH_TENSOR);
+    if ((e = grow(&h->bws, &h->bws_bytes, wm_bw_ws(h, N, T, f))) != cudaSuccess)
         return cuda_fail(h, e, "training-step workspace");
     if ((e = st.begin(h, T, false, s)) != cudaSuccess) return cuda_fail(h, e, "staging inputs");
     wm_nll_dev a{};
     a.N = N; a.T = T; a.z_seq = zs; a.actions = ac; a.lengths = ln;
     void *tail;
-    wm_bw_fwd f{};
     wm_bw_carve(h, N, T, h->bws, &f, &tail);
     a.h_seq = f.hs; a.c_seq = f.cs; a.mdn_seq = f.md;
     a.nll = nl ? nl : f.nll;
     if (path == WM_PATH_TENSOR && N > 0 && T > 0) {
-        f.have_g = wm_tc_scores_in_one(h, N, T) && wm_bw_takes_gates(h, N, T);
         if (f.have_g) a.g_seq = f.G;
-        f.have_dmd = true;  // the head GEMM's epilogue forms it: no head outputs are stored
-        a.dmd = f.dMD; a.dmd_op = f.dMDo;
-        a.mdn_seq = nullptr;
+        a.dmd = f.dMD; a.dmd_op = f.dMDo;  // the head GEMM's epilogue forms it: no head outputs are stored
         if (c.precision == WM_BF16) f.frames = wm_tc_frames(h, N, T, h->ws, &f.ld, &f.h_col);
     }
     int fwd_launches = 0;

@@ -372,13 +372,27 @@ cudaError_t cublas_err(cublasStatus_t st) {
 
 }  // namespace
 
+// X and Y are built unless the forward left them: its operand rows (bf16; h_t is then read from them
+// alone), or z_seq and h_t as they are (fp32, when no product with W_zh is left to do: h_{t-1} is
+// then h_t's row N rows up).  Head outputs are kept unless the forward formed their gradient.
+wm_bw_fwd wm_bw_plan(const wm_handle *h, int N, int T, bool tensor) {
+    const bool bf = h->cfg.precision == WM_BF16;
+    wm_bw_fwd f{};
+    wm_brecur_args a{};
+    f.have_dmd = tensor;
+    f.have_g = tensor && T > 1 && (size_t)N * T < (1u << 30) && wm_tc_scores_in_one(h, N, T) &&
+               wm_brecur_plan(!bf, N, h->cfg.h_dim, &a);  // (the backward recurrence reads pre-activations)
+    f.built = bf ? !tensor : !f.have_g;
+    return f;
+}
+
 // The forward's outputs at the front of the backward's workspace, then its own buffers.
 void wm_bw_carve(const wm_handle *h, int N, int T, void *base, wm_bw_fwd *f, void **tail) {
     const size_t NT = (size_t)N * T, H = h->cfg.h_dim, M = h->M;
     char *p = (char *)base;
-    f->hs = (float *)p; p += al(NT * H * 4);
+    if (f->built || h->cfg.precision == WM_FP32) { f->hs = (float *)p; p += al(NT * H * 4); }
     f->cs = (float *)p; p += al(NT * H * 4);
-    f->md = (float *)p; p += al(NT * M * 4);
+    if (!f->have_dmd) { f->md = (float *)p; p += al(NT * M * 4); }
     f->nll = (float *)p; p += al((size_t)N * 4);
     f->G = (float *)p; p += al(NT * 4 * H * 4);
     f->dMD = (float *)p; p += al(NT * M * 4);
@@ -387,18 +401,14 @@ void wm_bw_carve(const wm_handle *h, int N, int T, void *base, wm_bw_fwd *f, voi
     *tail = p;
 }
 
-bool wm_bw_takes_gates(const wm_handle *h, int N, int T) {
-    wm_brecur_args a{};
-    return T > 1 && (size_t)N * T < (1u << 30) && wm_brecur_plan(h->cfg.precision != WM_BF16, N, h->cfg.h_dim, &a);
-}
-
-size_t wm_bw_ws(const wm_handle *h, int N, int T) {
+size_t wm_bw_ws(const wm_handle *h, int N, int T, const wm_bw_fwd &f) {
     const wm_config &c = h->cfg;
     const size_t Z = c.z_dim, A = c.a_dim, H = c.h_dim, M = h->M, KX = Z + H, H4 = 4 * H;
     const size_t NT = (size_t)N * T, es = c.precision == WM_BF16 ? 2 : 4;
     const size_t part_cols = H4 > M ? H4 : M;
-    return al(NT * H * 4) * 2 + al(NT * M * 4) + al((size_t)N * 4)             // h, c, head outputs, nll
-           + al(NT * KX * es) + al(NT * H * es)                                // X, Y
+    return (f.built || es == 4 ? al(NT * H * 4) : 0) + al(NT * H * 4)          // h, c
+           + (f.have_dmd ? 0 : al(NT * M * 4)) + al((size_t)N * 4)             // head outputs, nll
+           + (f.built ? al(NT * KX * es) + al(NT * H * es) : 0)                // X, Y
            + al(NT * H4 * 4)                                                   // gate activations
            + al(NT * M * 4) + (es == 2 ? al(NT * M * 2) : 0)                   // dMD
            + al(NT * H * 4)                                                    // dY
@@ -476,11 +486,11 @@ static cudaError_t bw_run(const wm_handle *h, int N, int TT, const float *z_seq,
     if (st != CUBLAS_STATUS_SUCCESS) return cublas_err(st);
     const float *hs = f.hs, *cs = f.cs;
     float *G = f.G;
-    // X and Y are built unless the forward left them: its operand rows (bf16), or z_seq and h_t as they
-    // are (fp32, when no product with W_zh is left to do: h_{t-1} is then h_t's row N rows up)
-    const bool built = bf ? !f.frames : !f.have_g;
-    T *X = (T *)p; p += al(NT * KX * sizeof(T));
-    T *Y = (T *)p; p += al(NT * H * sizeof(T));
+    const bool built = f.built;
+    T *X = (T *)p;
+    if (built) p += al(NT * KX * sizeof(T));
+    T *Y = (T *)p;
+    if (built) p += al(NT * H * sizeof(T));
     float *dMD = f.dMD;
     const void *dMDo = bf ? (const void *)f.dMDo : (const void *)dMD;  // the GEMMs' operand
     float *dY = (float *)p; p += al(NT * H * 4);

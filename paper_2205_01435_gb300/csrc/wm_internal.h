@@ -285,12 +285,15 @@ struct wm_bw_fwd {
     float *hs, *cs, *md, *nll, *G, *dMD;
     __nv_bfloat16 *dMDo;  // bf16: dMD's copy
     bool have_g, have_dmd;
+    bool built;  // the weight gradients' operands X, Y are built (else: the frames, or z_seq and hs)
     const __nv_bfloat16 *frames;
     int ld, h_col;
 };
-size_t wm_bw_ws(const wm_handle *h, int N, int T);
+// What a forward of this kernel family leaves; its workspace holds nothing that is then not read
+// (of hs, md, X and Y).
+wm_bw_fwd wm_bw_plan(const wm_handle *h, int N, int T, bool tensor);
+size_t wm_bw_ws(const wm_handle *h, int N, int T, const wm_bw_fwd &f);
 void wm_bw_carve(const wm_handle *h, int N, int T, void *base, wm_bw_fwd *f, void **tail);
-bool wm_bw_takes_gates(const wm_handle *h, int N, int T);  // the backward recurrence reads pre-activations
 cudaError_t wm_bw_prepare(wm_handle *h);
 void wm_bw_free(wm_handle *h);
 cudaError_t wm_bw_launch(const wm_handle *h, int N, int T, const float *z_seq, const int32_t *actions,

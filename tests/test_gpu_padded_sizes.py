@@ -166,3 +166,29 @@ def test_draws_weigh_logits_accurately(wm, Z, A, H, K, B, NX):
     assert ok.sum() > B // 2
     # a quotient up to 10 (2^-24 of it), exponentials (2 ulp each), their sum and its logarithm
     np.testing.assert_allclose(np_(g["logp_seq"])[0][ok], lp[np.arange(B), acts][ok], rtol=0, atol=64 * 2.0**-24)
+
+
+def _scoring(N, T, Z, A):
+    g = torch.Generator(device="cuda").manual_seed(3)
+    return (torch.randn((T + 1, N, Z), generator=g, device="cuda"),
+            torch.randint(0, A, (T, N), generator=g, device="cuda", dtype=torch.int32))
+
+
+@pytest.mark.parametrize("prec", ["bf16", "fp32"])
+def test_training_step_holds_what_it_reads(wm, prec):
+    """Device memory of a first training step: the buffers of the batched backward, with an eighth to spare."""
+    Z, A, H, K, N, T = 64, 256, 512, 5, 512, 64
+    cfg = dict(_cfg(Z, A, H, K), precision=prec)
+    m = wm.WorldModel(cfg, synth.weights(cfg, seed=38))
+    z, a = _scoring(N, T, Z, A)
+    m.mdn_nll_backward(z[:3], a[:2])  # the libraries' own memory
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    r0 = torch.cuda.memory_reserved()
+    m.mdn_nll_backward(z, a)
+    torch.cuda.synchronize()
+    used = before - torch.cuda.mem_get_info()[0] - (torch.cuda.memory_reserved() - r0)
+    M, b = 3 * K * Z, prec == "bf16"
+    rows = 4 * (H + 4 * H + M + H + 4 * H) + (2 * (M + 4 * H) if b else 4 * H)  # c, G, dMD, dY, dG (and copies, or h)
+    rows += (2 if b else 4) * (Z + H) + 4 * 4 * 8                                 # frames, the likelihood's partials
+    assert used < 1.125 * N * T * rows + (96 << 20), (used, N * T * rows)
