@@ -54,7 +54,13 @@
  * instead: the mask slab of step t goes up ahead of step t, and step t's output
  * slabs come down as soon as step t is done, overlapping the other steps.  A call
  * with a host output, or with per-step staging, returns only when every copy
- * touching the caller's arrays is complete (also when it returns an error).  All
+ * touching the caller's arrays is complete (also when it returns an error).
+ * Scratch is a workspace of the handle, grown when a call needs more (not while
+ * the stream is capturing: make a call of the same size first).  Teacher-forced
+ * scoring on the tensor-core family holds the operand rows of all T + 1 frames;
+ * where AUTO took that family only because it is faster and these would pass
+ * 8 GB, have no room, or would have to be allocated under capture, the call runs
+ * on the family that needs N rows' scratch.  All
  * arrays are dense, row-major, in the layouts given, and owned by the caller.
  *
  * Errors: argument errors are returned synchronously and leave outputs

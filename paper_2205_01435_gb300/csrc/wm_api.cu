@@ -5,6 +5,7 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <algorithm>
 #include <new>
 #include <string>
 #include <vector>
@@ -43,6 +44,8 @@ bool is_host_ptr(const void *p) {
 
 float bf16_round_host(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
 
+size_t grown(size_t need) { return need + need / 8; }
+
 cudaError_t grow(void **buf, size_t *have, size_t need) {
     if (need <= *have) return cudaSuccess;
     if (*buf) {
@@ -52,7 +55,7 @@ cudaError_t grow(void **buf, size_t *have, size_t need) {
         *buf = nullptr;
         *have = 0;
     }
-    size_t n = need + need / 8;
+    const size_t n = grown(need);
     cudaError_t e = cudaMalloc(buf, n);
     if (e != cudaSuccess) return e;
     *have = n;
@@ -298,6 +301,51 @@ int pick_score_path(const wm_handle *h, int N, int T, bool train) {
         if (!(kept && wm_fused_supported(h, N))) return WM_PATH_TENSOR;
     }
     return pick_path(h, N, true, true, fits);
+}
+
+bool capturing(cudaStream_t s) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) == cudaSuccess) return st != cudaStreamCaptureStatusNone;
+    cudaGetLastError();
+    return true;  // (the legacy stream beside a capture: nothing may be allocated either)
+}
+
+// The workspaces of a scoring call or a training step.  Where pick_score_path gave an AUTO call to the
+// tensor family for speed alone and its operand rows of all steps have no room, or the call is being
+// captured and would have to allocate it, *path becomes the family that runs the call on N rows' scratch
+// (which the workspace always has room for, so that a call of N rows and any steps can be captured).
+cudaError_t score_room(wm_handle *h, int N, int T, bool train, cudaStream_t s, int *path) {
+    const int other = pick_path(h, N, true, true, false);
+    auto family_ws = [&](int p) {
+        return p == WM_PATH_FUSED ? wm_fused_nll_ws(h, N) : p == WM_PATH_TENSOR ? wm_tc_ws(h, N, T) : wm_step_nll_ws(h, N);
+    };
+    auto ws_of = [&](int p) { return p == other ? family_ws(p) : std::max(family_ws(p), family_ws(other)); };
+    auto bws_of = [&](int p) {
+        return train ? wm_bw_ws(h, N, T, wm_bw_plan(h, N, T, p == WM_PATH_TENSOR)) : (size_t)0;
+    };
+    const size_t ws = ws_of(*path), bws = bws_of(*path);
+    const bool more = ws > h->ws_bytes, bmore = bws > h->bws_bytes;
+    if (*path != other && (more || bmore)) {
+        size_t room = 0, total = 0;  // (what growing frees first counts as room)
+        if (capturing(s)) {
+            *path = other;
+        } else if (cudaMemGetInfo(&room, &total) == cudaSuccess &&
+                   (more ? grown(ws) : 0) + (bmore ? grown(bws) : 0) >
+                       room + (more ? h->ws_bytes : 0) + (bmore ? h->bws_bytes : 0)) {
+            *path = other;
+        }
+    }
+    cudaError_t e = grow(&h->ws, &h->ws_bytes, ws_of(*path));
+    if (e == cudaSuccess) e = grow(&h->bws, &h->bws_bytes, bws_of(*path));
+    if (e != cudaErrorMemoryAllocation || *path == other) return e;
+    cudaGetLastError();
+    if ((e = cudaDeviceSynchronize()) != cudaSuccess) return e;
+    cudaFree(h->ws);  // (its size may be what leaves no room for the other's)
+    h->ws = nullptr;
+    h->ws_bytes = 0;
+    *path = other;
+    e = grow(&h->ws, &h->ws_bytes, ws_of(other));
+    return e == cudaSuccess ? grow(&h->bws, &h->bws_bytes, bws_of(other)) : e;
 }
 
 template <class T>
@@ -695,21 +743,17 @@ wm_status wm_mdn_nll_backward(wm_handle *h, int N, int T, const float *z_seq, co
     st.add((void **)&g.b_mdn, grads->b_mdn, M * 4, true);
 
     // the forward: the teacher-forced pass, keeping h, c and the head outputs of every row
-    const int path = pick_score_path(h, N, T, true);
+    int path = pick_score_path(h, N, T, true);
     if (path == WM_PATH_FUSED && !wm_fused_supported(h, N))
         return fail(h, WM_ERR_UNSUPPORTED, "the fused family does not take this model / batch");
     if (c.path == WM_PATH_TENSOR && !wm_tc_supported(h))
         return fail(h, WM_ERR_UNSUPPORTED, "the tensor family does not take this model");
-    size_t need = path == WM_PATH_FUSED ? wm_fused_nll_ws(h, N) : path == WM_PATH_TENSOR ? wm_tc_ws(h, N, T)
-                                                                                      : wm_step_nll_ws(h, N);
-    if ((e = grow(&h->ws, &h->ws_bytes, need)) != cudaSuccess) return cuda_fail(h, e, "workspace");
-    wm_bw_fwd f = wm_bw_plan(h, N, T, path == WM_PATH_TENSOR);
-    if ((e = grow(&h->bws, &h->bws_bytes, wm_bw_ws(h, N, T, f))) != cudaSuccess)
-        return cuda_fail(h, e, "training-step workspace");
+    if ((e = score_room(h, N, T, true, s, &path)) != cudaSuccess) return cuda_fail(h, e, "training-step workspace");
     if ((e = st.begin(h, T, false, s)) != cudaSuccess) return cuda_fail(h, e, "staging inputs");
     wm_nll_dev a{};
     a.N = N; a.T = T; a.z_seq = zs; a.actions = ac; a.lengths = ln;
     void *tail;
+    wm_bw_fwd f = wm_bw_plan(h, N, T, path == WM_PATH_TENSOR);
     wm_bw_carve(h, N, T, h->bws, &f, &tail);
     a.h_seq = f.hs; a.c_seq = f.cs; a.mdn_seq = f.md;
     a.nll = nl ? nl : f.nll;
@@ -774,10 +818,7 @@ wm_status wm_mdn_nll(wm_handle *h, int N, int T, const float *z_seq, const int32
         return fail(h, WM_ERR_UNSUPPORTED, "the fused family does not take this model / batch");
     if (c.path == WM_PATH_TENSOR && !wm_tc_supported(h))
         return fail(h, WM_ERR_UNSUPPORTED, "the tensor family does not take this model");
-    size_t need = path == WM_PATH_FUSED ? wm_fused_nll_ws(h, N) : path == WM_PATH_TENSOR ? wm_tc_ws(h, N, T)
-                                                                                      : wm_step_nll_ws(h, N);
-    e = grow(&h->ws, &h->ws_bytes, need);
-    if (e != cudaSuccess) return cuda_fail(h, e, "workspace");
+    if ((e = score_room(h, N, T, false, s, &path)) != cudaSuccess) return cuda_fail(h, e, "workspace");
     if ((e = st.begin(h, T, false, s)) != cudaSuccess) return cuda_fail(h, e, "staging inputs");
     if (path == WM_PATH_FUSED)
         e = wm_fused_nll(h, a, h->ws, s);

@@ -174,6 +174,55 @@ def _scoring(N, T, Z, A):
             torch.randint(0, A, (T, N), generator=g, device="cuda", dtype=torch.int32))
 
 
+@pytest.mark.parametrize("train", [False, True])
+def test_a_longer_call_is_captured_after_a_short_one(wm, train):
+    """The operand rows of more steps would have to be allocated under capture: the call goes to the family
+    whose scratch does not grow with the steps.  (A training step's own workspace grows with the rows: a
+    call of more rows comes first.)"""
+    cfg = _cfg(50, 101, 300, 6)
+    w = synth.weights(cfg, seed=36)
+    m = wm.WorldModel(cfg, w)
+    z, a = _scoring(70, 24, 50, 101)
+    run = m.mdn_nll_backward if train else m.mdn_nll
+    run(z[:5], a[:4])  # (the operand rows of 4 steps)
+    if train:
+        run(*_scoring(100, 24, 50, 101))
+    m.sync()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        got = run(z, a)
+    path = m.last_path
+    for v in got.values():
+        v.zero_()
+    g.replay()
+    torch.cuda.synchronize()
+    if not train:
+        assert path == "stepwise"
+    want = (lambda s: s.mdn_nll_backward(z, a) if train else s.mdn_nll(z, a))(wm.WorldModel(cfg, w))
+    for k in want:  # bf16 operands on both families, sums in another order
+        assert float((got[k] - want[k]).norm() / want[k].norm()) < (5e-3 if train else 1e-5), k
+
+
+def test_a_call_whose_operand_rows_have_no_room(wm):
+    """Scoring that the tensor family would need 4 GB for runs on N rows' scratch when 2 GB are free."""
+    N, T, cfg = 12000, 400, _cfg(50, 101, 300, 6)
+    m = wm.WorldModel(cfg, synth.weights(cfg, seed=37))
+    z, a = _scoring(N, T, 50, 101)
+    m.mdn_nll(z[:2, :, :], a[:1])
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    hold = torch.empty(torch.cuda.mem_get_info()[0] - (2 << 30), dtype=torch.uint8, device="cuda")
+    got = m.mdn_nll(z, a)["nll"]
+    m.sync()
+    assert m.last_path == "stepwise"
+    del hold
+    torch.cuda.empty_cache()
+    want = m.mdn_nll(z, a)["nll"]
+    m.sync()
+    assert m.last_path == "tensor"
+    assert float((got - want).norm() / want.norm()) < 1e-5
+
+
 @pytest.mark.parametrize("prec", ["bf16", "fp32"])
 def test_training_step_holds_what_it_reads(wm, prec):
     """Device memory of a first training step: the buffers of the batched backward, with an eighth to spare."""
