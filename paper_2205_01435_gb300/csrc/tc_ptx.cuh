@@ -139,6 +139,14 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t saddr, uint32_t parit
     return false;
 }
 
+// Named barrier of `threads` threads (whole warps): true in all of them if `any` was in one.
+__device__ __forceinline__ bool barrier_or(int id, int threads, bool any) {
+    uint32_t r;
+    asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 q, %3, 0;\n\tbar.red.or.pred p, %1, %2, q;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(r) : "r"(id), "r"(threads), "r"((uint32_t)any) : "memory");
+    return r != 0;
+}
+
 // ---- TMA tensor tiles (K-major bf16 operands, 128-byte swizzle) ---------------------
 __device__ __forceinline__ uint64_t desc_sw128(uint32_t saddr) {
     uint64_t d = 0;

@@ -21,10 +21,12 @@
 // to RECUR_MAX_GROUPS row tiles per CTA this stays ahead of one launch per step (24 steps at H = 512:
 // 1024 / 2048 sequences 221 / 341 us against 288 / 432).
 // Every CTA waits for others: the launch is cooperative (all CTAs resident), every wait is
-// bounded, and a CTA that gives up records WM_ERR_TIMEOUT, skips its remaining work and exits.
+// bounded, and a CTA that gives up records WM_ERR_TIMEOUT and exits: its epilogue leaves the step loop
+// at the barrier before the counter's release, all warps together, so that the CTAs that wait for the
+// counter give up in their turn.
 //
 // Warps: 0 the TMA producer, 1 the MMA issuer (and TMEM), 2..9 the epilogue (two warps per TMEM
-// lane quadrant, U / 2 units each).  TMEM holds two accumulators of 4U columns.
+// lane quadrant, U / 2 units each).  TMEM holds two accumulators of 4U columns (fp32 path: 8U).
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <math.h>
@@ -290,12 +292,13 @@ __global__ void __launch_bounds__(THREADS, 1)
         gather(t1, m1, a1);
         advance();
         a1 = act_of(t1, m1);
-        for (int t = 0; t < T; ++t)
+        bool go = true;
+        for (int t = 0; t < T && go; ++t)
             for (int gi = 0, m = mg; m < p.m_tiles; ++gi, m += p.m_groups) {
                 const int b = m * BM + r;
                 const bool valid = b < p.N;
                 const size_t row = (size_t)t * p.N + (valid ? b : 0);
-                wait(&bar_accf[acc], acc_phase);
+                const bool ok = wait(&bar_accf[acc], acc_phase);
                 __syncwarp();
                 tc::fence_after_sync();
                 const uint32_t ta = tm + ((uint32_t)(32 * quad) << 16) + acc * NA + u0;
@@ -374,7 +377,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                     }
                 }
                 fence_proxy_async_global();
-                asm volatile("bar.sync 1, %0;" :: "n"(EPI_THREADS) : "memory");
+                if (!(go = !tc::barrier_or(1, EPI_THREADS, !ok))) break;
                 if (tid == 64)  // (the release covers the other threads' stores through the barrier)
                     asm volatile("red.release.gpu.global.add.s32 [%0], 1;" :: "l"(p.count + m) : "memory");
                 gather(t1, m1, a1);
