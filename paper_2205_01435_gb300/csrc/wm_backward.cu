@@ -560,6 +560,8 @@ static cudaError_t bw_run(const wm_handle *h, int N, int TT, const float *z_seq,
         ra.act = G; ra.cs = cs; ra.dY = dY; ra.pre = f.have_g;
         ra.dG = dG; ra.dGo = dGo; ra.parts = dG3;
         ra.count = count; ra.status = h->status; ra.w_row0 = bf ? Z : 0;
+        ra.test_wait = h->test_wait;  // an injected wait that the forward did not take
+        h->test_wait = 0;
         cudaError_t e = cudaMemsetAsync(count, 0, (size_t)ra.m_tiles * 4, s);
         if (e != cudaSuccess) return e;
         wm_ktime kt(h, WM_KERNEL_BW, s);

@@ -18,7 +18,11 @@
 //     wait for (as in wm_recur.cu).
 // The activations (or pre-activations), c and dY of the step are loaded before the wait for the
 // product, and prefetched into L2 a step earlier (without: 3338 instead of 3221 us per training step).  Every CTA
-// waits for others: cooperative launch, bounded waits, WM_ERR_TIMEOUT on giving up.
+// waits for others: cooperative launch, bounded waits, WM_ERR_TIMEOUT on giving up.  A CTA that gives up
+// sends no partials that it has not computed, arms no barrier again and releases no counter: its epilogue
+// leaves the step loop at one of the two barriers of a step, all warps together, and the CTAs that wait
+// for it give up in their turn.  Before its cluster's last barrier it gives the partials under way, its
+// own and its peers', time to land.
 //
 // F32: the operands are bf16 hi and lo parts (dG_t's in a two-step ring of their own, W_h's packed
 // once) and the products hi.hi + hi.lo + lo.hi, as everywhere on the fp32 path.
@@ -90,6 +94,16 @@ __global__ void __launch_bounds__(THREADS, 1)
     tc::cluster_sync();  // the cluster's barriers exist before any store reaches them
     tc::fence_after_sync();
     const uint32_t tm = tmem_base;
+    int T = p.T;
+    // injected wait (tests of the timeout path): every CTA gives up before it issues anything
+    if (p.test_wait) {
+        if (tid == 0 && !tc::mbar_wait_bounded(bar(&bar_never), 0, p.test_wait)) {
+            s_abort = 1;
+            atomicExch(p.status, (int)WM_ERR_TIMEOUT);
+        }
+        __syncthreads();
+        if (s_abort) T = 0;
+    }
     auto wait_slow = [&](uint64_t *b, uint32_t parity) {
         for (uint32_t i = 0; i < POLLS; ++i) {
             if (tc::mbar_try_wait(bar(b), parity)) return true;
@@ -105,7 +119,9 @@ __global__ void __launch_bounds__(THREADS, 1)
         return __all_sync(0xffffffffu, ok);
     };
 
-    if (warp == 0) {  // ---- TMA producer
+    if (T == 0) {
+        // (gave up, or nothing to do)
+    } else if (warp == 0) {  // ---- TMA producer
         if (tc::elect_one()) tc::mbar_arrive_expect_tx(bar(&bar_w), (uint32_t)np * W_BYTES);
         for (int i = 0; i < np; ++i)  // W_h: rows of units, gate g's columns (lo parts 4H further)
             if (tc::elect_one())
@@ -113,8 +129,8 @@ __global__ void __launch_bounds__(THREADS, 1)
         int stage = 0, used = 0;
         uint32_t phase = 0;
         bool go = true;
-        for (int t = p.T - 2; t >= 0 && go; --t) {
-            const int want = p.u_tiles * CL * (p.T - 1 - t);  // every unit of dG_{t+1}
+        for (int t = T - 2; t >= 0 && go; --t) {
+            const int want = p.u_tiles * CL * (T - 1 - t);  // every unit of dG_{t+1}
             bool ok = false;
             for (uint32_t i = 0; i < FLAG_POLLS && !ok && !s_abort; ++i) ok = ld_acquire(p.count + m) >= want;
             if (!ok && !s_abort) {
@@ -139,20 +155,18 @@ __global__ void __launch_bounds__(THREADS, 1)
                 if (++stage == S) { stage = 0; phase ^= 1u; }
             }
         }
-        // nothing may be in flight into the cluster's shared memory when a CTA exits
+        // no copy of this CTA's may be in flight into its shared memory when it exits
         __syncwarp();
-        const bool gave_up = s_abort != 0;
         tc::mbar_wait_bounded(bar(&bar_w), 0, POLLS);
         for (int i = used > S ? used - S : 0; i < used; ++i)
-            tc::mbar_wait_bounded(bar(&bar_full[i % S]), (uint32_t)(i / S) & 1u, gave_up ? 1u << 16 : POLLS);
-        if (gave_up) tc::mbar_wait_bounded(bar(&bar_never), 0, 1u << 14);
+            tc::mbar_wait_bounded(bar(&bar_full[i % S]), (uint32_t)(i / S) & 1u, POLLS);
     } else if (warp == 1) {  // ---- MMA issuer
         bool go = wait(&bar_w, 0);
         int stage = 0;
         uint32_t phase = 0;
         // (fp32 path: hi meets hi and lo in one MMA, see wm_recur.cu)
         const uint32_t idesc = tc::idesc_bf16_f32(BM, UC), idesc2 = tc::idesc_bf16_f32(BM, UC * PARTS);
-        for (int t = p.T - 2; t >= 0 && go; --t) {
+        for (int t = T - 2; t >= 0 && go; --t) {
             // (the accumulator is free: dG_{t+1}'s counter covers this CTA's reads of it)
             for (int i0 = 0; i0 < np; i0 += KPS) {
                 const int nk = np - i0 < KPS ? np - i0 : KPS;
@@ -222,11 +236,11 @@ __global__ void __launch_bounds__(THREADS, 1)
             asm volatile("prefetch.global.L2 [%0];" :: "l"(p.dY + row * H + u));
             if (t > 0) asm volatile("prefetch.global.L2 [%0];" :: "l"(p.cs + (row - N) * H + u));
         };
-        ld32(p.cs + ((size_t)(p.T - 1) * N + n) * H + u, c);
-        load(p.T - 1, in);
+        ld32(p.cs + ((size_t)(T - 1) * N + n) * H + u, c);
+        load(T - 1, in);
         uint32_t ph = 0;
-        // (after a wait gave up the steps go on without waiting: every warp meets the same barriers)
-        for (int t = p.T - 1; t >= 0; --t) {
+        bool ok = true;
+        for (int t = T - 1; t >= 0; --t) {
             const size_t row = (size_t)t * N + n;
             if (p.pre) {  // the activations, under the wait for the product
 #pragma unroll
@@ -237,9 +251,9 @@ __global__ void __launch_bounds__(THREADS, 1)
                     in.og[j] = 1.f / (1.f + expf(-in.og[j]));
                 }
             }
-            if (t < p.T - 1) {
+            if (t < T - 1) {
                 if (tid == 64) tc::mbar_arrive_expect_tx(bar(&bar_x), (CL - 1) * SLOT);
-                wait(&bar_acc, ph);
+                ok = wait(&bar_acc, ph);
                 tc::fence_after_sync();
                 float v[32];
                 {
@@ -266,13 +280,14 @@ __global__ void __launch_bounds__(THREADS, 1)
                     for (int k = 0; k < 4; ++k) {
                         const float4 q = make_float4(v[16 * s + 4 * k], v[16 * s + 4 * k + 1], v[16 * s + 4 * k + 2], v[16 * s + 4 * k + 3]);
                         const uint32_t dst = sx + g * SLOT + slot_at(r, k);
+                        if (!ok) continue;
                         if (to != g) st_async16(tc::map_rank(dst, to), q, tc::map_rank(bar(&bar_x), to));
                         else *reinterpret_cast<float4 *>(const_cast<unsigned char *>(xbuf) + g * SLOT + slot_at(r, k)) = q;
                     }
                 }
-                asm volatile("bar.sync 1, %0;" :: "n"(EPI_THREADS) : "memory");  // this CTA's own slot
-                wait(&bar_x, ph);
-                ph ^= 1u;
+                if (tc::barrier_or(1, EPI_THREADS, !ok)) break;  // this CTA's own slot
+                ok = wait(&bar_x, ph);
+                if (ok) ph ^= 1u;  // (else the phase that is open: the drain below waits for it)
 #pragma unroll
                 for (int k = 0; k < 2; ++k) {
                     float4 s = *reinterpret_cast<const float4 *>(xbuf + slot_at(er, 2 * eh + k));
@@ -316,7 +331,7 @@ __global__ void __launch_bounds__(THREADS, 1)
             }
             if (t > 0) {
                 fence_proxy_async_global();
-                asm volatile("bar.sync 1, %0;" :: "n"(EPI_THREADS) : "memory");
+                if (tc::barrier_or(1, EPI_THREADS, !ok)) break;
                 if (tid == 64)  // (the release covers the other threads' stores through the barrier)
                     asm volatile("red.release.gpu.global.add.s32 [%0], 1;" :: "l"(p.count + m) : "memory");
                 load(t - 1, in);
@@ -328,6 +343,9 @@ __global__ void __launch_bounds__(THREADS, 1)
                 for (int q = 0; q < 4; ++q) st32(o + q * H, d[q]);
             }
         }
+        // gave up: the phase of the partials may stay open (a peer that gave up too sends none), and then
+        // the polls are the time that those under way have to land (more than a millisecond)
+        if (__any_sync(0xffffffffu, !ok || s_abort)) tc::mbar_wait_bounded(bar(&bar_x), ph, 1u << 16);
     }
     __syncwarp();
     tc::fence_before_sync();

@@ -257,6 +257,7 @@ struct wm_brecur_args {
     __nv_bfloat16 *parts;        // fp32 path: [2 N, 8H] rows [hi | lo] of two steps
     int *count;                  // [m_tiles] zero on entry
     int *status;
+    uint32_t test_wait;          // injected wait: every CTA gives up before it issues anything
     int w_row0;                  // first row of W_h in its map
     // the plan
     int u_tiles, m_tiles, m_per_launch, m0, stages;

@@ -1,4 +1,4 @@
-"""The timeout path of the fused and tensor-core kernels.
+"""The timeout path of the fused and tensor-core kernels and of the backward recurrence.
 
 Every wait inside those kernels is bounded; when one gives up, the kernel records
 WM_ERR_TIMEOUT in the device status word, stops issuing work, lets nothing of its own
@@ -79,6 +79,26 @@ def test_scoring_wait_runs_out_then_recovers(wm, orc, name, path):
     m.sync()
     o = orc.mdn_nll(cfg, w, zs, acts, want_seq=True)
     check_teacher({k: v.cpu().numpy() for k, v in g.items()}, o, cfg["precision"])
+    m.close()
+
+
+@pytest.mark.parametrize("prec,H,N", [("bf16", 128, 300), ("fp32", 64, 70), ("bf16", 512, 130)])
+def test_backward_recurrence_wait_runs_out_then_recovers(wm, orc, prec, H, N):
+    """A stepwise forward has no waits: the injection reaches the one-launch backward recurrence."""
+    cfg, T = dict(synth.model_config("nll"), z_dim=16, a_dim=64, h_dim=H, k_mix=3, precision=prec), 4
+    w = synth.weights(cfg, seed=6)
+    zs, acts, lens = synth.teacher_inputs(N, T, 16, 64, seed=6, ragged=True)
+    m = wm.WorldModel(dict(cfg, path="stepwise"), w)
+    args = (_cuda(zs), _cuda(acts), _cuda(lens))
+    m.inject_wait_timeout(POLLS)
+    m.mdn_nll_backward(*args)
+    _expect_timeout(wm, m)
+    g = m.mdn_nll_backward(*args)
+    m.sync()
+    o = orc.mdn_nll_grad(cfg, w, zs, acts, lens, nthreads=16)
+    for k in ("W_lstm", "b_lstm", "W_mdn", "b_mdn"):
+        ref = np.asarray(o[k], np.float64)
+        assert np.linalg.norm(g[k].cpu().numpy() - ref) <= {"fp32": 1e-5, "bf16": 1e-2}[prec] * np.linalg.norm(ref), k
     m.close()
 
 
