@@ -531,6 +531,7 @@ static cudaError_t bw_run(const wm_handle *h, int N, int TT, const float *z_seq,
             if (st == CUBLAS_STATUS_SUCCESS)
                 st = gemm(hb, true, false, false, (int)NT, H4, H, f.frames + f.h_col, f.ld,
                           (const __nv_bfloat16 *)h->bw_wzh + (size_t)Z * H4, ldw, G, H4, 1.f);
+            ++launches;
         }
         ++launches;
     }
@@ -540,7 +541,7 @@ static cudaError_t bw_run(const wm_handle *h, int N, int TT, const float *z_seq,
         if (!f.have_g)
             k_bw_gates<<<(unsigned)(NT < 8192 ? NT : 8192), 256, 0, s>>>(NT, N, H, A, G, actions, h->step.Wa, h->step.bg);
         if (!f.have_dmd) k_bw_mdn<<<grid_of(NT * Z), 256, 0, s>>>(N, TT, Z, c.k_mix, f.md, z_seq, lengths, dMD, f.dMDo);
-        launches += 2;
+        launches += !f.have_g + !f.have_dmd;
     }
     {
         wm_ktime kt(h, WM_KERNEL_BW_GEMM, s);

@@ -108,3 +108,15 @@ def test_gradient_against_oracle(wm, orc, Z, A, H, K, N, T, prec):
     again = m.mdn_nll_backward(*args)
     for k in g:
         assert torch.equal(g[k], again[k]), k
+
+
+def test_launches_are_counted(wm):
+    """fp32, H = 1024: one gate GEMM per step, the head GEMM forms the gradient, and the backward goes step by
+    step: operands, gates (GEMM and kernel), dY; a cell kernel a step and a GEMM between; 3 GEMMs; 7 sums."""
+    cfg, T = dict(synth.model_config("nll"), z_dim=16, a_dim=64, h_dim=1024, k_mix=2, precision="fp32"), 3
+    zs, acts, _ = synth.teacher_inputs(20, T, 16, 64, seed=45)
+    m = wm.WorldModel(cfg, synth.weights(cfg, seed=45))
+    m.mdn_nll(_cuda(zs), _cuda(acts))
+    assert m.last_path == "tensor" and m.last_launches == 4 + T
+    m.mdn_nll_backward(_cuda(zs), _cuda(acts))
+    assert m.last_launches == 4 + T + 4 + (2 * T - 1) + 3 + 7
