@@ -727,6 +727,7 @@ wm_status wm_mdn_nll_backward(wm_handle *h, int N, int T, const float *z_seq, co
     cudaError_t e = cudaSetDevice(h->device);
     if (e != cudaSuccess) return cuda_fail(h, e, "cudaSetDevice");
     if ((e = wm_bw_prepare(h)) != cudaSuccess) return cuda_fail(h, e, "training-step set-up (cuBLAS)");
+    if ((e = wm_recur_prepare(h)) != cudaSuccess) return cuda_fail(h, e, "scoring set-up");
 
     const float *zs = z_seq;
     const int32_t *ac = actions, *ln = lengths;
@@ -801,6 +802,7 @@ wm_status wm_mdn_nll(wm_handle *h, int N, int T, const float *z_seq, const int32
     cudaStream_t s = (cudaStream_t)cuda_stream;
     cudaError_t e = cudaSetDevice(h->device);
     if (e != cudaSuccess) return cuda_fail(h, e, "cudaSetDevice");
+    if ((e = wm_recur_prepare(h)) != cudaSuccess) return cuda_fail(h, e, "scoring set-up");
 
     wm_nll_dev a{};
     a.N = N; a.T = T;

@@ -381,7 +381,7 @@ wm_bw_fwd wm_bw_plan(const wm_handle *h, int N, int T, bool tensor) {
     wm_brecur_args a{};
     f.have_dmd = tensor;
     f.have_g = tensor && T > 1 && (size_t)N * T < (1u << 30) && wm_tc_scores_in_one(h, N, T) &&
-               wm_brecur_plan(!bf, N, h->cfg.h_dim, &a);  // (the backward recurrence reads pre-activations)
+               wm_brecur_plan(h, N, h->cfg.h_dim, &a);  // (the backward recurrence reads pre-activations)
     f.built = bf ? !tensor : !f.have_g;
     return f;
 }
@@ -421,6 +421,8 @@ size_t wm_bw_ws(const wm_handle *h, int N, int T, const wm_bw_fwd &f) {
 }
 
 cudaError_t wm_bw_prepare(wm_handle *h) {
+    const cudaError_t re = wm_brecur_prepare(h);
+    if (re != cudaSuccess) return re;
     if (!h->cublas) {
         cublasHandle_t hb;
         cublasStatus_t st = cublasCreate(&hb);
@@ -550,7 +552,7 @@ static cudaError_t bw_run(const wm_handle *h, int N, int TT, const float *z_seq,
     }
     if (st != CUBLAS_STATUS_SUCCESS) return cublas_err(st);
     wm_brecur_args ra{};
-    const bool one = TT > 1 && NT < (1u << 30) && wm_brecur_plan(!bf, N, H, &ra);
+    const bool one = TT > 1 && NT < (1u << 30) && wm_brecur_plan(h, N, H, &ra);
     if (one) {
         CUtensorMap gm, wmap;
         // (bw_wzh: rows z | h of 4H columns; bw_w3: rows [hi | lo | hi])

@@ -367,33 +367,29 @@ void set_attrs(cudaLaunchConfig_t &lc, cudaLaunchAttribute (&at)[2], size_t smem
     lc.numAttrs = 2;
 }
 
-template <bool F32>
-int resident_clusters() {
-    static int per_device[WM_MAX_DEVICES] = {};  // (the shared-memory limit is a device's, too)
-    int &known = per_device[wm_device_slot()];
-    if (!known) {
-        const size_t smem = SMEM_MAX - SMEM_STATIC;
-        cudaLaunchConfig_t lc = {};
-        cudaLaunchAttribute at[2];
-        set_attrs(lc, at, smem);
-        lc.gridDim = dim3(CL);
-        lc.numAttrs = 1;
-        int c = 0;
-        if (cudaFuncSetAttribute(k_brecur<F32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
-            cudaOccupancyMaxActiveClusters(&c, k_brecur<F32>, &lc) != cudaSuccess) {
-            cudaGetLastError();
-            c = 0;
-        }
-        known = c > 0 ? c : -1;
-    }
-    return known;
-}
-
 }  // namespace
 
-bool wm_brecur_plan(bool f32, int N, int H, wm_brecur_args *a) {
+// The clusters that can be resident at once, and the kernel's shared-memory limit on this device.
+cudaError_t wm_brecur_prepare(wm_handle *h) {
+    if (h->brecur_ready) return cudaSuccess;
+    const bool f32 = h->cfg.precision == WM_FP32;
+    const void *kern = f32 ? (const void *)k_brecur<true> : (const void *)k_brecur<false>;
+    const size_t smem = SMEM_MAX - SMEM_STATIC;
+    cudaLaunchConfig_t lc = {};
+    cudaLaunchAttribute at[2];
+    set_attrs(lc, at, smem);
+    lc.gridDim = dim3(CL);
+    lc.numAttrs = 1;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&h->brecur_clusters, kern, &lc);
+    h->brecur_ready = e == cudaSuccess;
+    return e;
+}
+
+bool wm_brecur_plan(const wm_handle *h, int N, int H, wm_brecur_args *a) {
     if (H % UC) return false;
-    const int np = H / BK * (f32 ? 2 : 1), clusters = f32 ? resident_clusters<true>() : resident_clusters<false>();
+    const bool f32 = h->cfg.precision == WM_FP32;
+    const int np = H / BK * (f32 ? 2 : 1), clusters = h->brecur_clusters;
     a->u_tiles = H / UC;
     a->m_tiles = (N + BM - 1) / BM;
     const size_t fixed = 1024 + (size_t)np * W_BYTES + CL * (size_t)SLOT + SMEM_STATIC;

@@ -177,6 +177,10 @@ struct wm_handle {
     void *bw_w3 = nullptr;  // fp32 path: W_h as bf16 rows [hi | lo | hi] for the recurrence GEMM
     void *bws = nullptr;
     size_t bws_bytes = 0;
+    // the one-launch recurrences: CTAs resident at once [mode][16 | 32 units][2 | 3 parts per stage]; clusters
+    bool recur_ready = false, brecur_ready = false;
+    int recur_ctas[3][2][2] = {};
+    int brecur_clusters = 0;
 };
 
 // The current device's place in tables of per-device launch attributes.
@@ -240,7 +244,10 @@ struct wm_recur_args {
     size_t smem;
 };
 // Whether (and how) N sequences run as one launch.
-bool wm_recur_plan(int mode, int N, int Hp, int KX, wm_recur_args *a);
+bool wm_recur_plan(const wm_handle *h, int mode, int N, int Hp, int KX, wm_recur_args *a);
+// What the plans ask the device for, kept on the handle; before the first plan.
+cudaError_t wm_recur_prepare(wm_handle *h);
+cudaError_t wm_brecur_prepare(wm_handle *h);
 // mode: 0 bf16, 1 bf16 with accurate nonlinearities, 2 fp32 as bf16 parts.  Tensor maps: x rows in
 // boxes of 128 rows x 64, weights (128-column packing) in boxes of `units` rows x 64.
 cudaError_t wm_recur_launch(int mode, const void *x_map, const void *xl_map, const void *w_map, const void *wl_map,
@@ -263,7 +270,7 @@ struct wm_brecur_args {
     int u_tiles, m_tiles, m_per_launch, m0, stages;
     size_t smem;
 };
-bool wm_brecur_plan(bool f32, int N, int H, wm_brecur_args *a);
+bool wm_brecur_plan(const wm_handle *h, int N, int H, wm_brecur_args *a);
 // Maps: the product's operand rows (dGo, or parts) in boxes of 128 x 64; W_h's rows of units (4H gate
 // columns, fp32 path: then their lo parts) in boxes of 64 x 64.
 cudaError_t wm_brecur_launch(bool f32, const void *g_map, const void *w_map, wm_brecur_args a, cudaStream_t s);

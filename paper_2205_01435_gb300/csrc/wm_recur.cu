@@ -412,29 +412,29 @@ kern_t kernel_of(int mode, int units, int kps) {
     return units == 16 ? (kps == 3 ? k_recur<0, 16, 3> : k_recur<0, 16, 2>) : (kps == 3 ? k_recur<0, 32, 3> : k_recur<0, 32, 2>);
 }
 
-// CTAs that can be resident at once (one per SM)
-int resident(int mode, int units, int kps) {
-    static int known[WM_MAX_DEVICES][3][2][2] = {};  // (the shared-memory limit is a device's, too)
-    int &n = known[wm_device_slot()][mode][units >> 5][kps - 2];
-    if (!n) {
-        const kern_t kern = kernel_of(mode, units, kps);
-        const size_t smem = SMEM_MAX - SMEM_STATIC;
-        int dev = 0, sms = 0, c = 0;
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
-            cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c, kern, THREADS, smem) != cudaSuccess) {
-            cudaGetLastError();
-            c = 0;
-        }
-        n = c > 0 ? c * sms : -1;
-    }
-    return n;
-}
-
 }  // namespace
 
-bool wm_recur_plan(int mode, int N, int Hp, int KX, wm_recur_args *a) {
+// The CTAs that can be resident at once (one per SM), and the kernels' shared-memory limit on this device.
+cudaError_t wm_recur_prepare(wm_handle *h) {
+    if (h->recur_ready) return cudaSuccess;
+    const bool f32 = h->cfg.precision == WM_FP32;
+    const size_t smem = SMEM_MAX - SMEM_STATIC;
+    int sms = 0;
+    cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
+    for (int mode = f32 ? 2 : 0; mode < (f32 ? 3 : 2); ++mode)
+        for (int units : {16, 32})
+            for (int kps = 2; kps <= (f32 ? 2 : 3); ++kps) {
+                const kern_t kern = kernel_of(mode, units, kps);
+                int n = 0;
+                if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, THREADS, smem);
+                h->recur_ctas[mode][units >> 5][kps - 2] = n * sms;
+            }
+    h->recur_ready = e == cudaSuccess;
+    return e;
+}
+
+bool wm_recur_plan(const wm_handle *h, int mode, int N, int Hp, int KX, wm_recur_args *a) {
     const bool f32 = mode == 2;
     const int ks = (KX + BK - 1) / BK, mt = (N + BM - 1) / BM;
     bool found = false;
@@ -444,7 +444,7 @@ bool wm_recur_plan(int mode, int N, int Hp, int KX, wm_recur_args *a) {
         int mg = 0, groups = 0, kps = 0, stages = 0;
         size_t fixed = 0;
         for (int pass = 0; pass < 2; ++pass) {  // (the states' share depends on the resident CTAs, found with kps = 2)
-            const int ctas = resident(mode, U, pass ? kps : 2);
+            const int ctas = h->recur_ctas[mode][U >> 5][pass ? kps - 2 : 0];
             if (nt > ctas) { stages = 0; break; }
             mg = mt < ctas / nt ? mt : ctas / nt;
             groups = (mt + mg - 1) / mg;

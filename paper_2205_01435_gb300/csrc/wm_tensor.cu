@@ -2124,7 +2124,7 @@ static bool narrow_gates(bool f32, bool acc, int Hp, int tiles, int pairs) {
 static bool one_launch(const wm_handle *h, int N, int T, wm_recur_args *a, int *mode) {
     const wm_tc_weights &w = h->tc;
     *mode = h->cfg.precision == WM_FP32 ? 2 : accurate(h, N, 1) ? 1 : 0;
-    return T > 1 && (uint64_t)(T + 1) * N < (1u << 30) && wm_recur_plan(*mode, N, w.Hp, w.Zp + w.Hp, a);
+    return T > 1 && (uint64_t)(T + 1) * N < (1u << 30) && wm_recur_plan(h, *mode, N, w.Hp, w.Zp + w.Hp, a);
 }
 
 const __nv_bfloat16 *wm_tc_frames(const wm_handle *h, int N, int T, void *ws, int *ld, int *h_col) {

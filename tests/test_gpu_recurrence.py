@@ -21,15 +21,16 @@ def _cuda(a):
     return torch.from_numpy(np.ascontiguousarray(a)).cuda()
 
 
-# Z, A, H, K, N, T, precision (aligned sizes: the tensor family takes both precisions)
-CASES = [(8, 64, 64, 2, 300, 5, "bf16"), (64, 64, 64, 5, 1, 4, "fp32"), (24, 128, 320, 5, 129, 6, "bf16"),
-         (64, 256, 512, 5, 127, 3, "fp32"), (64, 256, 512, 5, 257, 4, "bf16"), (64, 256, 512, 5, 1000, 4, "bf16"),
-         (64, 256, 512, 5, 640, 3, "fp32"), (128, 512, 1024, 8, 256, 3, "bf16"), (128, 512, 1024, 8, 300, 2, "bf16"),
-         (32, 64, 256, 5, 2500, 3, "bf16"), (128, 512, 1024, 8, 40, 2, "fp32")]
+# Z, A, H, K, N, T, precision (aligned sizes: the tensor family takes both precisions), one launch or one per step
+# (more row tiles than four per CTA; weights that do not fit)
+CASES = [(8, 64, 64, 2, 300, 5, "bf16", True), (64, 64, 64, 5, 1, 4, "fp32", True), (24, 128, 320, 5, 129, 6, "bf16", True),
+         (64, 256, 512, 5, 127, 3, "fp32", True), (64, 256, 512, 5, 257, 4, "bf16", True), (64, 256, 512, 5, 1000, 4, "bf16", True),
+         (64, 256, 512, 5, 640, 3, "fp32", True), (128, 512, 1024, 8, 256, 3, "bf16", True), (128, 512, 1024, 8, 300, 2, "bf16", True),
+         (32, 64, 256, 5, 2500, 3, "bf16", True), (32, 64, 256, 5, 9800, 2, "bf16", False), (128, 512, 1024, 8, 40, 2, "fp32", False)]
 
 
-@pytest.mark.parametrize("Z,A,H,K,N,T,prec", CASES)
-def test_scoring_against_oracle(wm, orc, Z, A, H, K, N, T, prec):
+@pytest.mark.parametrize("Z,A,H,K,N,T,prec,one", CASES)
+def test_scoring_against_oracle(wm, orc, Z, A, H, K, N, T, prec, one):
     cfg = dict(synth.model_config("nll"), z_dim=Z, a_dim=A, h_dim=H, k_mix=K, precision=prec)
     w = synth.weights(cfg, seed=41)
     zs, acts, lens = synth.teacher_inputs(N, T, Z, A, seed=41, ragged=True)
@@ -38,6 +39,7 @@ def test_scoring_against_oracle(wm, orc, Z, A, H, K, N, T, prec):
     args = (_cuda(zs), _cuda(acts))
     g = m.mdn_nll(*args, lengths=_cuda(lens), want_seq=True)
     m.sync()
+    assert m.last_launches == 4 + (1 if one else T)  # the state, the frames, the recurrence, the heads, the sums
     idx = np.unique(np.linspace(0, N - 1, 24).round().astype(int))
     o = orc.mdn_nll(cfg, w, zs[:, idx], acts[:, idx], lengths=lens[idx], want_seq=True)
     check_teacher({k: np_(v)[idx] if k == "nll" else np_(v)[:, idx] for k, v in g.items()}, o, prec)
@@ -82,15 +84,20 @@ def test_under_stream_capture(wm):
 
 
 # the backward recurrence: cluster edges of every hidden size (64 units), row-tile edges, two launches
-# (more row tiles than the SMs hold), one step (no recurrence), the fp32 parts, sizes it leaves
-BACKWARD = [(8, 64, 64, 3, 129, 3, "bf16"), (16, 64, 64, 2, 1, 2, "fp32"), (64, 256, 512, 5, 130, 4, "bf16"),
-            (64, 256, 512, 5, 200, 3, "fp32"), (16, 64, 512, 2, 700, 3, "bf16"), (16, 64, 512, 2, 600, 2, "fp32"),
-            (32, 128, 1024, 3, 140, 2, "bf16"), (16, 64, 1024, 2, 20, 2, "fp32"), (24, 128, 320, 5, 60, 4, "bf16"),
-            (16, 64, 128, 2, 50, 1, "bf16"), (11, 45, 100, 3, 40, 5, "bf16")]
+# (more row tiles than the SMs hold), one step (no recurrence), the fp32 parts, sizes it leaves.
+# Launches: the forward's (1 on a fused member, 5 on the tensor family with one recurrence launch), before the
+# recurrence (dY; with a forward that leaves nothing also the operands, the gates' GEMM and kernel and the mixture's
+# gradient), the recurrence (2 T - 1 step by step), and 3 GEMMs and 7 sums
+BACKWARD = [(8, 64, 64, 3, 129, 3, "bf16", 1 + 5 + 1 + 10), (16, 64, 64, 2, 1, 2, "fp32", 1 + 5 + 1 + 10),
+            (64, 256, 512, 5, 130, 4, "bf16", 5 + 1 + 1 + 10), (64, 256, 512, 5, 200, 3, "fp32", 5 + 1 + 1 + 10),
+            (16, 64, 512, 2, 700, 3, "bf16", 5 + 1 + 2 + 10), (16, 64, 512, 2, 600, 2, "fp32", 5 + 1 + 2 + 10),
+            (32, 128, 1024, 3, 140, 2, "bf16", 5 + 1 + 1 + 10), (16, 64, 1024, 2, 20, 2, "fp32", 6 + 4 + 3 + 10),
+            (24, 128, 320, 5, 60, 4, "bf16", 5 + 1 + 1 + 10), (16, 64, 128, 2, 50, 1, "bf16", 1 + 5 + 1 + 10),
+            (11, 45, 100, 3, 40, 5, "bf16", 1 + 5 + 9 + 10)]
 
 
-@pytest.mark.parametrize("Z,A,H,K,N,T,prec", BACKWARD)
-def test_gradient_against_oracle(wm, orc, Z, A, H, K, N, T, prec):
+@pytest.mark.parametrize("Z,A,H,K,N,T,prec,launches", BACKWARD)
+def test_gradient_against_oracle(wm, orc, Z, A, H, K, N, T, prec, launches):
     cfg = dict(synth.model_config("nll"), z_dim=Z, a_dim=A, h_dim=H, k_mix=K, precision=prec)
     w = synth.weights(cfg, seed=44)
     zs, acts, lens = synth.teacher_inputs(N, T, Z, A, seed=44, ragged=True)
@@ -99,6 +106,7 @@ def test_gradient_against_oracle(wm, orc, Z, A, H, K, N, T, prec):
     args = (_cuda(zs), _cuda(acts), _cuda(lens))
     g = m.mdn_nll_backward(*args)
     m.sync()
+    assert m.last_launches == launches
     o = orc.mdn_nll_grad(cfg, w, zs, acts, lens, nthreads=16)
     # relative Frobenius norms: about 100 fp32 roundoffs, 4 bf16 roundoffs (the operands are rounded once)
     tol = {"fp32": 1e-5, "bf16": 1e-2}[prec]
