@@ -287,19 +287,19 @@ int pick_path(const wm_handle *h, int B, bool fused_ok, bool tc_ok, bool pad_ok)
 }
 
 // Scoring (and the training step's forward): AUTO takes the tensor family for a bf16 model whenever its
-// recurrence runs as one launch, also where a member of the fused family would take the call, unless
-// that is short.  Measured (us, fused against tensor) at Z, A, H, K = 32, 64, 256, 5: 16 x 4 steps 40 / 44,
-// x 24 183 / 110, x 100 723 / 407, 1500 x 24 264 / 166; at 7, 45, 40, 3: 16 x 4 27 / 36, x 24 121 / 96;
-// at 85, 168, 94, 7: 271 x 24 1087 / 139.  The crossing lies between 6 and 10 steps.  In a training
-// step of the smallest models and batches the fused member's outputs cost less: 100 x 24 at 7, 45, 40, 3
-// 384 / 392, 600 x 24 732 / 475.  The tensor family holds the operand rows of all steps: a call that
-// another family can run on N rows' scratch goes to it when those pass 8 GB.
-int pick_score_path(const wm_handle *h, int N, int T, bool train) {
+// recurrence runs as one launch, also where a member of the fused family would take the call, from 10
+// steps on.  Measured (us, fused against tensor) at 8 / 10 / 12 steps, the fewest sequences first, where the
+// crossing is latest: 16 sequences at Z, A, H, K = 7, 45, 40, 3: 46 / 49, 56 / 56, 65 / 59; at 16, 64, 64, 3
+// 48 / 51, 58 / 54, 68 / 63; at 20, 50, 128, 5 52 / 56, 62 / 63, 74 / 66; at 32, 64, 256, 5 64 / 57, 77 / 65,
+// 90 / 73; 200 at 20, 50, 128, 5 140 / 59, 171 / 66, 202 / 74.  Training steps alike: 16 at 7, 45, 40, 3
+// 189 / 190, 213 / 208, 243 / 228, 100 there 193 / 197, 214 / 221, 237 / 245 (24 steps 386 / 335), 800
+// 372 / 203, 444 / 233, 500 / 254; 100 at 32, 64, 256, 5 222 / 179, 257 / 199, 292 / 217.  The tensor family
+// holds the operand rows of all steps: a call that another family can run on N rows' scratch goes to it
+// when those pass 8 GB.
+int pick_score_path(const wm_handle *h, int N, int T) {
     const bool fits = wm_tc_auto_ok(h) && wm_tc_ws(h, N, T) <= (size_t)8 << 30;
-    if (h->cfg.path == WM_PATH_AUTO && fits && wm_tc_scores_in_one(h, N, T)) {
-        const bool kept = T < 12 || (train && h->cfg.h_dim < 64 && N <= 400);
-        if (!(kept && wm_fused_supported(h, N))) return WM_PATH_TENSOR;
-    }
+    if (h->cfg.path == WM_PATH_AUTO && fits && wm_tc_scores_in_one(h, N, T) && (T >= 10 || !wm_fused_supported(h, N)))
+        return WM_PATH_TENSOR;
     return pick_path(h, N, true, true, fits);
 }
 
@@ -744,7 +744,7 @@ wm_status wm_mdn_nll_backward(wm_handle *h, int N, int T, const float *z_seq, co
     st.add((void **)&g.b_mdn, grads->b_mdn, M * 4, true);
 
     // the forward: the teacher-forced pass, keeping h, c and the head outputs of every row
-    int path = pick_score_path(h, N, T, true);
+    int path = pick_score_path(h, N, T);
     if (path == WM_PATH_FUSED && !wm_fused_supported(h, N))
         return fail(h, WM_ERR_UNSUPPORTED, "the fused family does not take this model / batch");
     if (c.path == WM_PATH_TENSOR && !wm_tc_supported(h))
@@ -815,7 +815,7 @@ wm_status wm_mdn_nll(wm_handle *h, int N, int T, const float *z_seq, const int32
     st.add((void **)&a.c_seq, c_seq, t * n * H * 4, true);
     st.add((void **)&a.mdn_seq, mdn_seq, t * n * M * 4, true);
 
-    int path = pick_score_path(h, N, T, false);
+    int path = pick_score_path(h, N, T);
     if (path == WM_PATH_FUSED && !wm_fused_supported(h, N))
         return fail(h, WM_ERR_UNSUPPORTED, "the fused family does not take this model / batch");
     if (c.path == WM_PATH_TENSOR && !wm_tc_supported(h))
