@@ -395,6 +395,7 @@ wm_status wm_create(const wm_config *cfg, const wm_weights *w, wm_handle **out) 
     memset(&h->small, 0, sizeof(h->small));
     memset(&h->tc, 0, sizeof(h->tc));
     cudaError_t e = cudaGetDevice(&h->device);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, h->device);
     if (e == cudaSuccess) e = pack_step(h, w);
     h->fused.force_cluster = cfg->fused_cluster;
     if (e == cudaSuccess) e = wm_fused_pack(h, w);

@@ -140,6 +140,7 @@ struct wm_host_weights {
 struct wm_handle {
     wm_config cfg;
     int device;
+    int sms;                     // of the device
     int M;                       // 3 K Z
     int NR;                      // head columns after the mixture: reward, done (+ runtime,
                                  // memory when shaped) (+ value when value_head), in that order

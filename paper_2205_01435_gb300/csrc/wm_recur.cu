@@ -419,8 +419,7 @@ cudaError_t wm_recur_prepare(wm_handle *h) {
     if (h->recur_ready) return cudaSuccess;
     const bool f32 = h->cfg.precision == WM_FP32;
     const size_t smem = SMEM_MAX - SMEM_STATIC;
-    int sms = 0;
-    cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
+    cudaError_t e = cudaSuccess;
     for (int mode = f32 ? 2 : 0; mode < (f32 ? 3 : 2); ++mode)
         for (int units : {16, 32})
             for (int kps = 2; kps <= (f32 ? 2 : 3); ++kps) {
@@ -428,7 +427,7 @@ cudaError_t wm_recur_prepare(wm_handle *h) {
                 int n = 0;
                 if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
                 if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, THREADS, smem);
-                h->recur_ctas[mode][units >> 5][kps - 2] = n * sms;
+                h->recur_ctas[mode][units >> 5][kps - 2] = n * h->sms;
             }
     h->recur_ready = e == cudaSuccess;
     return e;

@@ -509,15 +509,16 @@ void launch_gemm(const wm_handle *hd, bool round, int M, int N, int K1, int K2, 
                  const float *A2, long lda2, const float *W, long ldw, const float *bias, float *C, long ldc,
                  cudaStream_t s) {
     wm_ktime kt(hd, WM_KERNEL_STEP_GEMM, s);
-    // the largest tile that gives the 152 SMs a block each or more; a small batch takes low tiles (20
-    // steps at H = 300: 1 episode 1705 us on the 64 x 64 tile, 844 on 16 x 32 with k-blocks of 16, 659
-    // with 64; 100 episodes 2351 on 64 x 64, 767 on 32 x 64)
+    // the largest tile that gives the SMs a block each or more (32 x 64: two thirds of them); a small
+    // batch takes low tiles (152 SMs, 20 steps at H = 300: 1 episode 1705 us on the 64 x 64 tile, 844 on
+    // 16 x 32 with k-blocks of 16, 659 with 64; 100 episodes 2351 on 64 x 64, 767 on 32 x 64)
+    const long sms = hd->sms;
     auto blocks = [&](int bm, int bn) { return (long)((M + bm - 1) / bm) * ((N + bn - 1) / bn); };
-    if (M > 64 && blocks(128, 128) >= 2 * 152)
+    if (M > 64 && blocks(128, 128) >= 2 * sms)
         launch_tile<128, 128, 8, 8, 16>(round, M, N, K1, K2, A1, lda1, A2, lda2, W, ldw, bias, C, ldc, s);
-    else if (M > 32 && blocks(64, 64) >= 152)
+    else if (M > 32 && blocks(64, 64) >= sms)
         launch_tile<64, 64, 8, 4, 16>(round, M, N, K1, K2, A1, lda1, A2, lda2, W, ldw, bias, C, ldc, s);
-    else if (M > 16 && blocks(32, 64) >= 100)
+    else if (M > 16 && 3 * blocks(32, 64) >= 2 * sms)
         launch_tile<32, 64, 4, 4, 32>(round, M, N, K1, K2, A1, lda1, A2, lda2, W, ldw, bias, C, ldc, s);
     else
         launch_tile<16, 32, 4, 2, 64>(round, M, N, K1, K2, A1, lda1, A2, lda2, W, ldw, bias, C, ldc, s);

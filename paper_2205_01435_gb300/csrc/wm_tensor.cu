@@ -2068,9 +2068,7 @@ cudaError_t wm_tc_pack(wm_handle *h) {
     k_tc_pack<PACK_ACTIONS><<<512, 256>>>(g, 32, 4 * Hp, A, h->step.Wa, 4L * H, (bf *)T.wa_n, (bf *)T.wa_n_lo, nullptr, nullptr);
     k_tc_pack<PACK_HEADS><<<1024, 256>>>(g, 0, (int)nhr, Hp, h->step.Wh, lh, (bf *)T.wh, (bf *)T.wh_lo, h->step.bh, T.bh);
     if ((e = wm_tc_set_controllers(h, 1)) != cudaSuccess) return e;
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&T.sms, cudaDevAttrMultiProcessorCount, dev);
+    T.sms = h->sms;
     T.ok = 1;
     return cudaSuccess;
 }
