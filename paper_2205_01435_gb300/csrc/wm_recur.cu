@@ -353,6 +353,10 @@ __global__ void __launch_bounds__(THREADS, 1)
                     }
                     if (UT > 8) store_pre(j0);  // (held past the counter they would spill)
                 }
+                if (MODE == 1 && nu < UT) {  // a padded unit's h' is 0 also where its gates met 0 x infinity
+#pragma unroll
+                    for (int j = 0; j < UT; ++j) h[j] = j < nu ? h[j] : 0.f;
+                }
                 tc::fence_before_sync();
                 __syncwarp();
                 if (lane == 0)  // the accumulator may be overwritten

@@ -757,6 +757,11 @@ struct EpiGatesT {
 #pragma unroll
             for (int j = 0; j < UT; ++j) hv[j] = sig_(g[j]) * tanh_(cv[j]);
         }
+        if constexpr (ACC) {  // a padded unit's h' is 0 also where its gates met 0 x infinity
+            if (p.H - u0 < UT)  // (uniform over the warp)
+#pragma unroll
+                for (int j = 0; j < UT; ++j) hv[j] = j < p.H - u0 ? hv[j] : 0.f;
+        }
         if (fz) {  // frozen: h is the carried one
             const float4 *h4 = reinterpret_cast<const float4 *>(p.h32 + (size_t)bb * Hp + u0);
 #pragma unroll

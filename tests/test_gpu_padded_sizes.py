@@ -117,6 +117,44 @@ def test_forced_path_still_refuses_unaligned_sizes(wm):
     assert e.value.status == wm.WM_ERR_UNSUPPORTED
 
 
+@pytest.mark.parametrize("Z,A,H,K,B,flags", [(50, 101, 300, 6, 40, {}), (31, 90, 100, 4, 260, dict(n_xfers=23)),
+                                             (33, 129, 130, 5, 300, dict(done_terminates=1))])
+def test_infinite_latents_stay_in_their_row_and_step(wm, Z, A, H, K, B, flags):
+    """An infinite latent saturates the gates it meets; the padded units, whose weights are 0, make no NaN of it."""
+    cfg, T = _cfg(Z, A, H, K, **flags), 3
+    w = synth.weights(cfg, seed=39)
+    z0, x = synth.z0(B, Z, seed=39), {}
+    z0[0, 3], z0[1, 2], z0[B - 1, Z - 1] = np.inf, -np.inf, 3.4e38  # (the last rounds to infinity in bf16)
+    NX = cfg["n_xfers"]
+    if NX:
+        mask, x["loc_mask"] = (_cuda(v) for v in synth.hier_masks(T, B, NX, A - NX, 0.5, seed=39))
+    else:
+        mask = _cuda(synth.mask(T, B, A, 0.4, seed=39))
+    g, s = (wm.WorldModel(dict(cfg, path=p), w).rollout(_cuda(z0), T, mask=mask, want_logp=True, want_seq=True, **x)
+            for p in ("auto", "stepwise"))
+    same = (g["actions"] == s["actions"]).all(0) & (g["comp_seq"] == s["comp_seq"]).all(2).all(0)
+    assert same[[0, 1, B - 1]].any()
+    for k in ("h_seq", "c_seq", "rewards", "mdn_seq"):
+        assert torch.isfinite(g[k]).all(), k
+        assert float((g[k][:, same] - s[k][:, same]).abs().max()) < 2e-2, k  # (the parity bound of bf16 paths)
+
+
+@pytest.mark.parametrize("Z,A,H,K,N,T", [(50, 101, 300, 6, 40, 12), (11, 45, 100, 3, 200, 11)])
+def test_infinite_targets_past_a_sequence_do_not_spread(wm, Z, A, H, K, N, T):
+    cfg = _cfg(Z, A, H, K)
+    w = synth.weights(cfg, seed=40)
+    zs, acts, _ = synth.teacher_inputs(N, T, Z, A, seed=40)
+    zs[5, ::3, 1] = np.inf
+    lens = np.full(N, 4, np.int32)
+    m = wm.WorldModel(cfg, w)
+    g = m.mdn_nll(_cuda(zs), _cuda(acts), lengths=_cuda(lens), want_seq=True)
+    assert m.last_path == "tensor"
+    s = wm.WorldModel(dict(cfg, path="stepwise"), w).mdn_nll(_cuda(zs), _cuda(acts), lengths=_cuda(lens), want_seq=True)
+    for k in g:
+        assert torch.isfinite(g[k]).all(), k
+        assert float((g[k] - s[k]).norm() / s[k].norm()) < 1e-2, k
+
+
 # sizes padded, and a small batch of an aligned model; a second action row
 ACCURATE = [(50, 101, 300, 6, 300, 0), (64, 256, 512, 8, 60, 0), (31, 90, 100, 4, 260, 23), (24, 512, 128, 8, 100, 0)]
 
