@@ -371,7 +371,7 @@ void set_attrs(cudaLaunchConfig_t &lc, cudaLaunchAttribute (&at)[2], size_t smem
 
 // The clusters that can be resident at once, and the kernel's shared-memory limit on this device.
 cudaError_t wm_brecur_prepare(wm_handle *h) {
-    if (h->brecur_ready) return cudaSuccess;
+    if (h->brecur_ready || h->cfg.h_dim % UC) return cudaSuccess;
     const bool f32 = h->cfg.precision == WM_FP32;
     const void *kern = f32 ? (const void *)k_brecur<true> : (const void *)k_brecur<false>;
     const size_t smem = SMEM_MAX - SMEM_STATIC;

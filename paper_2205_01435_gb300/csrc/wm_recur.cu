@@ -420,7 +420,7 @@ kern_t kernel_of(int mode, int units, int kps) {
 
 // The CTAs that can be resident at once (one per SM), and the kernels' shared-memory limit on this device.
 cudaError_t wm_recur_prepare(wm_handle *h) {
-    if (h->recur_ready) return cudaSuccess;
+    if (h->recur_ready || !h->tc.ok) return cudaSuccess;
     const bool f32 = h->cfg.precision == WM_FP32;
     const size_t smem = SMEM_MAX - SMEM_STATIC;
     cudaError_t e = cudaSuccess;
