@@ -33,8 +33,10 @@
  * counter = (episode lo32, t0 + t, purpose << 24 | block, episode hi32), where
  * episode = episode_offset + b.  Purpose 0: component uniforms (4 dims per
  * block); 1: Box-Muller normals (4 dims per block); 2: controller uniform.
- * A uniform is (x >> 8) * 2^-24.  Results therefore do not depend on how the
- * episodes are split across calls or devices.
+ * A uniform is (x >> 8) * 2^-24.  The draws therefore do not depend on how the
+ * episodes are split across calls or devices, and neither do results as long as
+ * the parts run on the same kernel family (AUTO chooses by the model, the
+ * outputs and B, never by a rollout's T).
  *
  * Precision: WM_FP32 gives fp32-accurate results: the stepwise family computes
  * in fp32; the tensor-core family computes each contraction as three bf16
@@ -42,7 +44,10 @@
  * accumulation (about 3e-6 relative error), and everything else in fp32.
  * WM_BF16 rounds every weight matrix to bf16 (RNE) at wm_create and rounds the
  * GEMM operands [z_t; h_t] and h' to bf16; biases, accumulation,
- * nonlinearities, state and sampling stay fp32.
+ * nonlinearities, state and sampling stay fp32 (the fused tcgen05 kernel and
+ * the tensor-core family at its own sizes and B >= 256 take the hardware's
+ * approximations of tanh, relative error about 2^-11, and of the exponentials
+ * in the draws; padded sizes and smaller batches the accurate functions).
  *
  * Memory: every array argument below may be device memory (cudaMalloc'd,
  * managed) or host memory (pinned or pageable); the library tells them apart
@@ -105,7 +110,8 @@ enum { WM_FP32 = 0, WM_BF16 = 1 };
  *             or a hierarchical action.
  *   TENSOR    three tcgen05 GEMM launches per step (H % 64 == 0, A % 64 == 0).  AUTO also
  *             gives it bf16 models of other sizes (A <= 512, K <= 8), padded with zero
- *             weights. */
+ *             weights, but not their rollouts with H > 512.  Teacher-forced scoring runs
+ *             the recurrence as one launch where its weights fit. */
 enum { WM_PATH_AUTO = 0, WM_PATH_STEPWISE = 1, WM_PATH_FUSED = 2, WM_PATH_TENSOR = 3 };
 
 typedef struct {
@@ -225,7 +231,8 @@ wm_status wm_create(const wm_config *cfg, const wm_weights *weights, wm_handle *
  * on cuda_stream (a cudaStream_t; NULL = legacy default stream).  Episode b is
  * keyed to Philox as episode_offset + b and its steps as t0 + t, so a rollout
  * split over calls (resume: pass z_out[T], h_final, c_final, done[T-1]) or over
- * devices (shard: episode_offset) reproduces the unsplit one bit for bit.
+ * devices (shard: episode_offset; on the same kernel family, see wm_last_path)
+ * reproduces the unsplit one bit for bit.
  * B = 0 or T = 0 are valid (T = 0 only copies z0 to z_out[0]).
  *
  * Models whose episodes end (done_terminates or noop_terminates) with one
@@ -279,7 +286,9 @@ typedef struct {
  * split into three bf16 parts; plain fp32 where the library lacks it), the
  * recurrence's dH = dG_t W_h^T takes each operand as two bf16 parts and
  * accumulates the three products hi.hi + hi.lo + lo.hi in fp32 (each product
- * within 3 * 2^-16 of the fp32 one at worst), all for finite inputs and weights
+ * within 3 * 2^-16 of the fp32 one at worst), and the gate pre-activations
+ * that the forward left are the forward's (three products as well, the action
+ * row and the bias added in fp32), all for finite inputs and weights
  * (non-finite values are not propagated as IEEE arithmetic would), and the
  * forward is fp32-accurate (see Precision above).  The forward runs on the
  * kernel family wm_mdn_nll would pick; the batched GEMMs of the backward (the

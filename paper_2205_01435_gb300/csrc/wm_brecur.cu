@@ -1,7 +1,7 @@
 // wm_brecur.cu -- the training step's backward recurrence as one persistent kernel: for t = T-1 .. 0
 //   dH_t = dG_{t+1} W_h^T,  dh = dY_t + dH_t,  the cell's backward step -> dG_t      (Sec. 3.3.2)
 // in one launch (as two launches per step, a cell kernel and a library GEMM, a step took 11.8 us at
-// 512 sequences and H = 512, almost all of it latency; 6.3 us here: clock64 stamps, counter to product
+// 512 sequences and H = 512, almost all of it latency; about 7 us here; clock64 stamps of one CTA: counter to product
 // 3.9K cycles, exchange 2.9K, cell 0.9K, stores and the counter's release 3.3K, release to acquire 1.7K).
 //
 // The product contracts over 4H gate columns, four times what the forward's does, so a CTA could not

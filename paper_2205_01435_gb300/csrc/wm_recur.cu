@@ -15,7 +15,7 @@
 //     nothing is overwritten and one counter is the only dependency.  Every CTA loads its whole
 //     operand blocks itself.
 // A step (512 sequences, H = 512) takes about 4 us: operands through L2, MMAs, cell, stores and the
-// hand-off are one chain.  A call of 512 x 128 takes 0.64 ms, 1.28 as one launch per step; on the
+// hand-off are one chain.  A call of 512 x 128 takes 0.65 ms, 1.28 as one launch per step; on the
 // fp32 path (two parts per block through a ring that holds 4; paced by the issuer's MMAs) 1.22 ms,
 // 2.38 before.  (With the loads of a row tile shared by a cluster of four CTAs: 0.67 and 1.21.)  Up
 // to RECUR_MAX_GROUPS row tiles per CTA this stays ahead of one launch per step (24 steps at H = 512:

@@ -835,7 +835,7 @@ using EpiGatesA = EpiGatesT<0, 64, true>;    // accurate nonlinearities, bf16 pa
 using EpiGatesNA = EpiGatesT<0, 32, true>;
 // Two action rows (hierarchical actions) take 128-column tiles at every size: with 256-column
 // ones the second row's words make the epilogue spill.  16384 x 8 steps, H = 1024: gates
-// 161 -> 130 us a step, call 2550 -> 2328 us; 64 to 16384 rows, H = 512 and 1024: 1-13% less.
+// 161 -> 130 us a step, call 2540 -> 2311 us; 64 to 16384 rows, H = 512 and 1024: 1-13% less.
 using EpiGates2N = EpiGatesT<1, 32>;
 using EpiGates2NA = EpiGatesT<1, 32, true>;
 
