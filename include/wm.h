@@ -54,8 +54,8 @@
  * with cudaPointerGetAttributes.  Host arrays are staged through device
  * buffers owned by the handle.  In general they are copied whole on the call's
  * stream, inputs before the kernels and outputs after them.  When the call runs
- * step by step (wm_rollout on the tensor-core family, T > 1, a stream that is not
- * capturing), per-step slabs move on two copy streams owned by the handle
+ * step by step (wm_rollout on the tensor-core family, T > 1, all host arrays
+ * pinned, a stream that is not capturing), per-step slabs move on two copy streams owned by the handle
  * instead: the mask slab of step t goes up ahead of step t, and step t's output
  * slabs come down as soon as step t is done, overlapping the other steps.  A call
  * with a host output, or with per-step staging, returns only when every copy

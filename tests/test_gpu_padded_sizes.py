@@ -1,6 +1,8 @@
 """The tensor-core family on sizes it pads (AUTO's choice for bf16 models the fused family does
 not take): tile edges, single columns and the largest of each range, against the oracle and
 against the stepwise family that served these calls before."""
+import time
+
 import numpy as np
 import pytest
 import torch
@@ -279,3 +281,24 @@ def test_training_step_holds_what_it_reads(wm, prec):
     rows = 4 * (H + 4 * H + M + H + 4 * H) + (2 * (M + 4 * H) if b else 4 * H)  # c, G, dMD, dY, dG (and copies, or h)
     rows += (2 if b else 4) * (Z + H) + 4 * 4 * 8                                 # frames, the likelihood's partials
     assert used < 1.125 * N * T * rows + (96 << 20), (used, N * T * rows)
+
+
+def test_pageable_outputs_do_not_hold_up_the_steps(wm):
+    """A call with every output in pageable host memory takes no longer than on the family whose host arrays
+    are copied whole (copied step by step it took seven times as long)."""
+    Z, A, H, K, B, T = 50, 101, 300, 6, 2000, 30
+    cfg = _cfg(Z, A, H, K)
+    w, z0 = synth.weights(cfg, seed=46), torch.from_numpy(synth.z0(B, Z, seed=46))
+    mask = torch.from_numpy(synth.mask(T, B, A, 0.4, seed=46))
+
+    def best(path):
+        m, ms = wm.WorldModel(dict(cfg, path=path), w), []
+        m.rollout(z0, T, mask=mask, want_seq=True)
+        for _ in range(4):
+            t = time.perf_counter()
+            m.rollout(z0, T, mask=mask, want_seq=True)  # (allocates its outputs)
+            ms.append(time.perf_counter() - t)
+        return min(ms), m.last_path
+
+    (auto, path), (step, _) = best("auto"), best("stepwise")
+    assert path == "tensor" and auto < 1.5 * step, (auto, step)
